@@ -50,7 +50,7 @@ struct vtx_ctx {
       hostin_e, hostout, covlist, covmask, stage, defer;
   bool cov_ok = false;  // the covered-pixel list of the last prepared launch fits (two-pass resolve)
   bool occl_ok = false;  // the occlusion pass's buffers of the last prepared launch fit
-  Buf ses_sas, ses_a, ses_b, ses_edt, ses_blk, ses_base, ses_total, ses_bbox, ses_case;
+  Buf ses_bits, ses_a, ses_b, ses_edt, ses_blk, ses_base, ses_total, ses_bbox, ses_case;
   uint32_t cap_rec = 0;
   unsigned long long cap_entries = 0;
   Status *h_status = nullptr;
@@ -446,7 +446,7 @@ vtx_status vtx_destroy(vtx_ctx *c) {
   drop_graphs(c);
   Buf *bufs[] = {&c->keys,   &c->surv,   &c->state,  &c->tcount,   &c->tstart,   &c->tcursor,  &c->tlist,
                  &c->bsums,  &c->recs,   &c->recimg, &c->recbox,   &c->recof,    &c->entries,  &c->status,
-                 &c->counts, &c->hostin_x, &c->hostin_e, &c->hostout, &c->covlist, &c->covmask, &c->stage, &c->defer, &c->ses_sas, &c->ses_a, &c->ses_b,
+                 &c->counts, &c->hostin_x, &c->hostin_e, &c->hostout, &c->covlist, &c->covmask, &c->stage, &c->defer, &c->ses_bits, &c->ses_a, &c->ses_b,
                  &c->ses_edt, &c->ses_blk, &c->ses_base, &c->ses_total, &c->ses_bbox, &c->ses_case};
   for (Buf *b : bufs)
     if (b->p) cudaFree(b->p);
@@ -1246,9 +1246,11 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
     return fail(c, VTX_ERR_INVALID_ARG, "ses: misaligned output");
   const long long nb = ses_blocks(g->dims);
   vtx_status st;
-  if (!ds && (st = ensure(c, c->ses_sas, (size_t)n_pts, "ses sas"))) return st;
-  if ((st = ensure(c, c->ses_a, 2 * (size_t)n_pts, "ses pass a"))) return st;
-  if ((st = ensure(c, c->ses_b, 2 * (size_t)n_pts, "ses pass b"))) return st;
+  if ((st = ensure(c, c->ses_bits, 4 * (size_t)ses_words(g->dims), "ses interior"))) return st;
+  if (ses_three_pass(g->probe, g->spacing)) {
+    if ((st = ensure(c, c->ses_a, 2 * (size_t)n_pts, "ses pass a"))) return st;
+    if ((st = ensure(c, c->ses_b, 2 * (size_t)n_pts, "ses pass b"))) return st;
+  }
   if (!de && (st = ensure(c, c->ses_edt, 2 * (size_t)n_pts, "ses edt"))) return st;
   if ((st = ensure(c, c->ses_blk, sizeof(unsigned) * (size_t)(nb + 1), "ses blocks"))) return st;
   if ((st = ensure(c, c->ses_case, (size_t)n_pts, "ses cases"))) return st;  // >= one byte per cell
@@ -1263,7 +1265,8 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
   }
   L.h = g->spacing;
   L.probe = g->probe;
-  L.sas = ds ? (uint8_t *)ds : (uint8_t *)c->ses_sas.p;
+  L.bits = (uint32_t *)c->ses_bits.p;
+  L.sas = (uint8_t *)ds;
   L.g_a = (uint16_t *)c->ses_a.p;
   L.g_b = (uint16_t *)c->ses_b.p;
   L.edt2 = de ? (uint16_t *)de : (uint16_t *)c->ses_edt.p;

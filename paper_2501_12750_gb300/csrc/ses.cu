@@ -6,11 +6,13 @@
 //      has ((X-c)_x^2 + (X-c)_y^2) + (X-c)_z^2 < (r + p)^2, evaluated in FP64
 //      with every operation explicitly rounded (no contraction), so the
 //      decision is a pure function of the inputs.  One warp per atom, one
-//      lane per grid row of the atom's box.
+//      lane per grid row of the atom's box; the interior is one bit per point.
 //   2. Squared distance (grid units) to the nearest point outside the SAS
 //      interior, exact inside a (2K+1)^3 window (K = ceil(p/h) + 1) and
-//      K^2 + 1 beyond: three separable min-plus passes (x, y, z), integers
-//      only.  Marching cubes only ever needs values <= K^2.
+//      K^2 + 1 beyond, integers only.  Marching cubes only ever needs values
+//      <= K^2.  Windows of K <= 6 (p/h <= 5): 32 points at a time, as bit
+//      sets of the points within each possible distance; larger windows: three
+//      separable min-plus passes (x, y, z).
 //   3. SES interior: edt2 >= 1 and edt2 h^2 >= p^2 (FP64; an integer threshold
 //      here, as the product is monotone in edt2).  Marching cubes in two passes:
 //      each CTA classifies a run of cells (one case byte per cell) and counts
@@ -23,6 +25,7 @@
 //      become a star of triangles around their mean vertex.
 #include <cmath>
 #include <mutex>
+#include <utility>
 
 #include "vtx_internal.h"
 
@@ -149,6 +152,7 @@ static bool ses_table_ready(int device) {
 struct SesGrid {
   float ox, oy, oz, h, p;
   int nx, ny, nz;
+  int wx;        // 32-bit words per row of the interior bits: ceil(nx / 32)
   int K;
   int t_in;      // smallest edt2 with edt2 * h^2 >= p^2 in FP64 (the SES test, monotone in edt2)
   float xmax;    // largest |coordinate| of any grid point (bounds the FP32 rounding of the SAS filter)
@@ -158,131 +162,274 @@ __device__ __forceinline__ double grid_coord(float o, float h, long long i) {
   return __dadd_rn((double)o, __dmul_rn((double)h, (double)i));
 }
 
-// Set n bytes to 1: bytes up to a 4-byte boundary, then words, then bytes.
-__device__ __forceinline__ void fill_ones(uint8_t *p, long long n) {
-  while (n > 0 && ((uintptr_t)p & 3u)) {
-    *p++ = 1;
-    --n;
-  }
-  uint32_t *w = reinterpret_cast<uint32_t *>(p);
-  for (; n >= 4; n -= 4) *w++ = 0x01010101u;
-  p = reinterpret_cast<uint8_t *>(w);
-  while (n-- > 0) *p++ = 1;
-}
-
 __device__ __forceinline__ bool sas_exact(const SesGrid &G, long long i, double dy2, double dz2, double cx, double R2) {
   const double dx = __dsub_rn(grid_coord(G.ox, G.h, i), cx);
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), dy2), dz2) < R2;
 }
 
-// SAS interior: one warp per atom, lanes over the (j, k) rows of its box.
-// Each point is first classified in FP32 with a bound M on the FP32 error of
-// d^2 (coordinates, differences and squares, all at most a few ulps of
-// numbers <= xmax + R + 2h, and of R^2 itself); only points within M of the
-// sphere are decided by the exact FP64 test, so every decision equals the
-// FP64 one.  Per row, only the points of the chord |dx|^2 <= R^2 - dy^2 -
-// dz^2 + M are visited.
-__global__ __launch_bounds__(256) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n,
-                                                 uint8_t *__restrict__ sas) {
+// SAS interior, one bit per grid point (bit i & 31 of word i >> 5 of a row; wx words a row): one warp per atom
+// (`parts` warps when there are few atoms), lanes over the (j, k) rows of its box.  A row meets the sphere in a
+// chord: with t = R^2 - dy^2 - dz^2 in FP32 and M the bound on the FP32 error of d^2 (coordinates, differences
+// and squares, all at most a few ulps of numbers <= xmax + R + 2h, and of R^2 itself), every point with
+// |dx| <= sqrt(t - M) is inside and none with |dx| > sqrt(t + M) is; the index bounds of both are widened by the
+// rounding of the index itself.  The points between the two (a few in a thousand rows have one) are decided by
+// the exact FP64 test, so every decision equals the FP64 one.  The chord's bits are set with one atomic a word.
+//
+// Bound by the row loop's issue and its atomics, not by memory: the bits of 3.4e7 points are 4.6 MB and stay in
+// L2.  1e5 atoms at 0.5 A (3.4e7 points): 179 us; 1302 us with a byte per point, each point classified on its own.
+__global__ __launch_bounds__(256) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n, int parts,
+                                                 uint32_t *__restrict__ bits) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long a = warp; a < n; a += n_warps) {
-    const float4 c = X[a];
+  for (long long item = warp; item < n * parts; item += n_warps) {
+    const float4 c = X[item / parts];
     // FP32 throughout except on the rare points the filter cannot decide (the
     // FP64 pipes are a small fraction of the FP32 ones on this part)
     const float Rf = c.w + G.p, R2f = Rf * Rf;
     const float span = G.xmax + Rf + 2.0f * G.h;
     const float delta = 4e-7f * span;                      // |FP32 difference - exact| per axis
-    const float ext = Rf + 2.0f * G.h;
+    const float ext = fabsf(Rf) + 2.0f * G.h;
     const float M = 8.0f * ext * delta + 4.0f * delta * delta + 1e-6f * ext * ext + 1e-6f;
     // candidate index ranges, two points wider than the sphere's extent on each side
     const float inv_h = 1.0f / G.h;
-    long long lo[3], hi[3];
     const float cf[3] = {c.x, c.y, c.z};
     const float of[3] = {G.ox, G.oy, G.oz};
-    const long long nn[3] = {G.nx, G.ny, G.nz};
+    const int nn[3] = {G.nx, G.ny, G.nz};
+    int lo[3], hi[3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      lo[d] = (long long)floorf((cf[d] - Rf - of[d]) * inv_h) - 2;
-      hi[d] = (long long)ceilf((cf[d] + Rf - of[d]) * inv_h) + 2;
-      lo[d] = lo[d] < 0 ? 0 : lo[d];
-      hi[d] = hi[d] > nn[d] - 1 ? nn[d] - 1 : hi[d];
+      // clamped as floats first, so that the conversions cannot overflow
+      const float top = (float)nn[d];
+      lo[d] = max((int)fminf(fmaxf(floorf((cf[d] - Rf - of[d]) * inv_h) - 2.0f, 0.0f), top), 0);
+      hi[d] = min((int)fminf(fmaxf(ceilf((cf[d] + Rf - of[d]) * inv_h) + 2.0f, -1.0f), top), nn[d] - 1);
     }
     if (lo[0] > hi[0] || lo[1] > hi[1] || lo[2] > hi[2]) continue;
-    const long long ny_box = hi[1] - lo[1] + 1;
-    const long long rows = ny_box * (hi[2] - lo[2] + 1);
-    for (long long r = lane; r < rows; r += 32) {
-      const long long j = lo[1] + r % ny_box, k = lo[2] + r / ny_box;
+    // rounding of a chord end's grid index: FP32 sums and products of numbers <= |c| + |o| + R
+    const float eps = 1e-5f + 2e-6f * (fabsf(c.x) + fabsf(G.ox) + fabsf(Rf)) * inv_h;
+    // row r of the box is (lo[1] + r % ny_box, lo[2] + r / ny_box); this lane takes every (32 parts)-th
+    const unsigned ny_box = (unsigned)(hi[1] - lo[1] + 1), step = 32u * (unsigned)parts;
+    const unsigned r0 = 32u * (unsigned)(item % parts) + (unsigned)lane;
+    const int step_j = (int)(step % ny_box), step_k = (int)(step / ny_box);
+    int j = lo[1] + (int)(r0 % ny_box), k = lo[2] + (int)(r0 / ny_box);
+    for (; k <= hi[2]; k += step_k) {
       const float dyf = __fsub_rn(__fmaf_rn(G.h, (float)j, G.oy), c.y);
       const float dzf = __fsub_rn(__fmaf_rn(G.h, (float)k, G.oz), c.z);
       const float yz = __fmaf_rn(dyf, dyf, __fmul_rn(dzf, dzf));
       const float t = R2f - yz;
-      if (t < -M) continue;  // the whole row is outside
-      const float w = sqrtf(fmaxf(t + M, 0.0f)) + 2.0f * delta;
-      long long i0 = (long long)floorf((c.x - w - G.ox) * inv_h) - 2, i1 = (long long)ceilf((c.x + w - G.ox) * inv_h) + 2;
-      i0 = i0 < lo[0] ? lo[0] : i0;
-      i1 = i1 > hi[0] ? hi[0] : i1;
-      bool have64 = false;
-      double dy2 = 0.0, dz2 = 0.0, R2 = 0.0;
-      uint8_t *row = sas + (k * G.ny + j) * (long long)G.nx;
-      // 1 = certainly inside, 0 = certainly outside, else the exact FP64 decision
-      auto classify = [&](long long i, bool &certain) -> bool {
-        const float dxf = __fsub_rn(__fmaf_rn(G.h, (float)i, G.ox), c.x);
-        const float d2f = __fmaf_rn(dxf, dxf, yz);
-        certain = d2f < R2f - M;
-        if (certain) return true;
-        if (d2f > R2f + M) return false;
-        if (!have64) {
-          const double dy = __dsub_rn(grid_coord(G.oy, G.h, j), (double)c.y);
-          const double dz = __dsub_rn(grid_coord(G.oz, G.h, k), (double)c.z);
-          dy2 = __dmul_rn(dy, dy);
-          dz2 = __dmul_rn(dz, dz);
-          const double R = __dadd_rn((double)c.w, (double)G.p);
-          R2 = __dmul_rn(R, R);
-          have64 = true;
-        }
-        return sas_exact(G, i, dy2, dz2, (double)c.x, R2);
-      };
-      // from each end of the chord, decide points one by one up to the first one
-      // certainly inside; d^2 is convex along the row, so every point between the
-      // two certain ones is inside with the same margin and is filled directly
-      long long a_in = -1, b_in = -1;
-      for (long long i = i0; i <= i1; ++i) {
-        bool certain;
-        if (classify(i, certain)) row[i] = 1;
-        if (certain) {
-          a_in = i;
-          break;
-        }
-      }
-      if (a_in >= 0) {
-        for (long long i = i1; i > a_in; --i) {
-          bool certain;
-          if (classify(i, certain)) row[i] = 1;
-          if (certain) {
-            b_in = i;
-            break;
+      if (!(t < -M)) {  // else the whole row is outside
+        const float w_out = sqrtf(fmaxf(t + M, 0.0f)) * 1.000001f + 2.0f * delta;
+        const float w_in = t > M ? sqrt_approx(t - M) * 0.999999f - 2.0f * delta : -1.0f;
+        const float top = (float)(hi[0] + 1);
+        const int i0 = max((int)fminf(fmaxf(ceilf((c.x - w_out - G.ox) * inv_h - eps), 0.0f), top), lo[0]);
+        const int i1 = min((int)fminf(fmaxf(floorf((c.x + w_out - G.ox) * inv_h + eps), -1.0f), top), hi[0]);
+        int a = i1 + 1, b = i1;  // the certain points [a, b] (none yet)
+        if (w_in >= 0.0f) {
+          const int ca = (int)fminf(fmaxf(ceilf((c.x - w_in - G.ox) * inv_h + eps), 0.0f), top);
+          const int cb = (int)fminf(fmaxf(floorf((c.x + w_in - G.ox) * inv_h - eps), -1.0f), top);
+          if (max(ca, i0) <= min(cb, i1)) {
+            a = max(ca, i0);
+            b = min(cb, i1);
           }
         }
-        if (b_in > a_in + 1) fill_ones(row + a_in + 1, b_in - a_in - 1);
+        uint32_t *row = bits + ((size_t)k * (size_t)G.ny + (size_t)j) * (size_t)G.wx;
+        if (a <= b) {
+          const int wa = a >> 5, wb = b >> 5;
+          for (int w = wa; w <= wb; ++w) {
+            uint32_t m = 0xffffffffu;
+            if (w == wa) m <<= a & 31;
+            if (w == wb) m &= 0xffffffffu >> (31 - (b & 31));
+            atomicOr(row + w, m);
+          }
+        }
+        if (a > i0 || b < i1) {
+          const double dy = __dsub_rn(grid_coord(G.oy, G.h, j), (double)c.y);
+          const double dz = __dsub_rn(grid_coord(G.oz, G.h, k), (double)c.z);
+          const double dy2 = __dmul_rn(dy, dy), dz2 = __dmul_rn(dz, dz);
+          const double R = __dadd_rn((double)c.w, (double)G.p);
+          const double R2 = __dmul_rn(R, R);
+          for (int i = i0; i <= i1; ++i) {
+            if (i == a) {  // past the certain points
+              i = b;
+              continue;
+            }
+            if (sas_exact(G, i, dy2, dz2, (double)c.x, R2)) atomicOr(row + (i >> 5), 1u << (i & 31));
+          }
+        }
+      }
+      j += step_j;
+      if (j > hi[1]) {
+        j -= (int)ny_box;
+        ++k;
       }
     }
   }
 }
 
+// The interior as one byte per point (only when the caller asks for the plane).
+__global__ __launch_bounds__(256) void k_ses_sas_bytes(SesGrid G, const uint32_t *__restrict__ bits, long long n_pts,
+                                                       uint8_t *__restrict__ sas) {
+  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n_pts;
+       q += (long long)gridDim.x * blockDim.x) {
+    const long long row = q / G.nx, i = q - row * G.nx;
+    sas[q] = (uint8_t)((bits[row * G.wx + (i >> 5)] >> (i & 31)) & 1u);
+  }
+}
+
+// ------------------------------------------------- distances as bit sets --
+
+// Largest window of the bit-set distance pass.
+constexpr int kSesBitK = 6;
+
+// The lattice offsets (dx >= 0, dy, dz) of squared length <= K^2 in ascending order of length ("steps"), and the
+// distinct squared lengths ("levels": sums of three squares).  Offsets are those of the pass's shared-memory tile.
+template <int K>
+struct SesSteps {
+  static constexpr int TY = 32, TZ = 8;                           // rows of a tile
+  static constexpr int PY = TY + 2 * K, PZ = TZ + 2 * K, PL = PY * PZ;  // with their halo; one plane per dx
+  static constexpr int max_steps = (K + 1) * (2 * K + 1) * (2 * K + 1);
+  int n = 0, n_levels = 0;
+  int off[max_steps] = {};
+  int level[max_steps + 1] = {};   // level of each step
+  int value[K * K + 2] = {};       // squared length of each level, then the sentinel K^2 + 1
+  constexpr SesSteps() {
+    for (int m = 0; m <= K * K; ++m) {
+      bool any = false;
+      for (int dx = 0; dx <= K; ++dx)
+        for (int dz = -K; dz <= K; ++dz)
+          for (int dy = -K; dy <= K; ++dy)
+            if (dx * dx + dy * dy + dz * dz == m) {
+              off[n] = dx * PL + dz * PY + dy;
+              level[n++] = n_levels;
+              any = true;
+            }
+      if (any) value[n_levels++] = m;
+    }
+    level[n] = n_levels;
+    value[n_levels] = K * K + 1;
+  }
+};
+template <int K>
+constexpr SesSteps<K> kSesSteps{};
+
+template <int K>
+struct SesLevelState {
+  uint32_t acc = 0u, prev = 0u;  // points within the levels so far; within the levels before the current one
+  uint32_t plane[6] = {};        // binary digits of each point's level
+};
+
+template <int K, int I>
+__device__ __forceinline__ void ses_step(const uint32_t *e, SesLevelState<K> &s) {
+  constexpr int off = kSesSteps<K>.off[I], lv = kSesSteps<K>.level[I];
+  constexpr bool last = kSesSteps<K>.level[I + 1] != lv;
+  s.acc |= e[off];
+  if constexpr (last) {
+    const uint32_t newly = s.acc & ~s.prev;
+    if constexpr ((lv & 1) != 0) s.plane[0] |= newly;
+    if constexpr ((lv & 2) != 0) s.plane[1] |= newly;
+    if constexpr ((lv & 4) != 0) s.plane[2] |= newly;
+    if constexpr ((lv & 8) != 0) s.plane[3] |= newly;
+    if constexpr ((lv & 16) != 0) s.plane[4] |= newly;
+    if constexpr ((lv & 32) != 0) s.plane[5] |= newly;
+    s.prev = s.acc;
+  }
+}
+
+template <int K, int... I>
+__device__ __forceinline__ void ses_steps(const uint32_t *e, SesLevelState<K> &s, std::integer_sequence<int, I...>) {
+  (ses_step<K, I>(e, s), ...);
+}
+
+// s_val[level] = its squared length (the last one: the sentinel).
+template <int K, int I>
+__device__ __forceinline__ void ses_value(uint16_t *s_val) {
+  constexpr int v = kSesSteps<K>.value[I];
+  if (threadIdx.x == I) s_val[I] = (uint16_t)v;
+}
+template <int K, int... I>
+__device__ __forceinline__ void ses_values(uint16_t *s_val, std::integer_sequence<int, I...>) {
+  (ses_value<K, I>(s_val), ...);
+}
+
+// Windowed squared distance for windows K <= 6, 32 points at a time.  A CTA takes one word of 32 x 8 rows (y, z).
+// E_d, d = 0..K, is the set of points with a point outside the SAS interior exactly d along x; the points within
+// squared distance m are the union of E_dx over the rows (dy, dz) with dx^2 + dy^2 + dz^2 <= m, so going through
+// the lattice offsets by length, one shared-memory read and one OR give 32 points' worth of each.  A point's
+// level (the ordinal of its distance) is kept as binary digit planes and spread to one 16-bit value per point at
+// the end.  Points beyond the grid are not outside points.
+//
+// Bound by shared-memory reads and issue (K = 4: 153 reads a word).  3.4e7 points at K = 4: 60 us; the three
+// separable passes over 16-bit planes (one point per thread) take 105 + 2 x 172 us.  K <= 6 because the offsets
+// grow with K^3 (519 at K = 6) and every one is an unrolled instruction.
+template <int K>
+__global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *__restrict__ bits,
+                                                    uint16_t *__restrict__ edt2) {
+  using S = SesSteps<K>;
+  constexpr int n_levels = kSesSteps<K>.n_levels;
+  __shared__ uint32_t s_e[(K + 1) * S::PL];
+  __shared__ uint16_t s_val[64];
+  const int lane = threadIdx.x & 31, zw = threadIdx.x >> 5;
+  const unsigned ty = (unsigned)(G.ny + S::TY - 1) / S::TY;
+  const unsigned b = blockIdx.x;
+  const int w = (int)(b % (unsigned)G.wx);
+  const unsigned q = b / (unsigned)G.wx;
+  const long long y0 = (long long)(q % ty) * S::TY, z0 = (long long)(q / ty) * S::TZ;
+  const int tail = G.nx - 32 * (G.wx - 1);  // points of a row's last word
+  const uint32_t last_mask = 0xffffffffu >> (32 - tail);
+  ses_values<K>(s_val, std::make_integer_sequence<int, n_levels + 1>{});
+  for (int r = threadIdx.x; r < S::PL; r += 256) {
+    const int yy = r % S::PY, zz = r / S::PY;
+    const long long y = y0 + yy - K, z = z0 + zz - K;
+    uint32_t zp = 0u, zc = 0u, zn = 0u;  // points outside the interior: the words before, at and after w
+    if (y >= 0 && y < G.ny && z >= 0 && z < G.nz) {
+      const uint32_t *p = bits + (z * G.ny + y) * G.wx + w;
+      zc = ~p[0] & (w == G.wx - 1 ? last_mask : 0xffffffffu);
+      if (w > 0) zp = ~p[-1];
+      if (w + 1 < G.wx) zn = ~p[1] & (w + 1 == G.wx - 1 ? last_mask : 0xffffffffu);
+    }
+    s_e[r] = zc;
+#pragma unroll
+    for (int d = 1; d <= K; ++d) s_e[d * S::PL + r] = __funnelshift_r(zc, zn, d) | __funnelshift_l(zp, zc, d);
+  }
+  __syncthreads();
+  SesLevelState<K> st;
+  ses_steps<K>(s_e + (zw + K) * S::PY + lane + K, st, std::make_integer_sequence<int, kSesSteps<K>.n>{});
+  const uint32_t rest = ~st.acc;  // farther than K: the last level
+#pragma unroll
+  for (int p = 0; p < 6; ++p)
+    if ((n_levels >> p) & 1) st.plane[p] |= rest;
+  // spread: row r of the warp's 32 (y0 + r), one point per lane
+  constexpr int planes = n_levels < 2 ? 1 : n_levels < 4 ? 2 : n_levels < 8 ? 3 : n_levels < 16 ? 4 : n_levels < 32 ? 5 : 6;
+  const long long z = z0 + zw, x = 32LL * w + lane;
+  if (z >= G.nz) return;  // uniform in the warp; no barrier follows
+  const int rows = (int)min((long long)S::TY, G.ny - y0);
+  uint16_t *dst = edt2 + (z * G.ny + y0) * G.nx + x;
+  for (int r = 0; r < rows; ++r, dst += G.nx) {
+    unsigned lv = 0u;
+#pragma unroll
+    for (int p = 0; p < planes; ++p) lv |= ((__shfl_sync(0xffffffffu, st.plane[p], r) >> lane) & 1u) << p;
+    if (x < G.nx) *dst = s_val[lv];
+  }
+}
+
+// --------------------------------------------- distances in three passes --
+
 // Pass x: distance^2 along x to the nearest point outside the SAS interior, within K.
-__global__ __launch_bounds__(256) void k_ses_edt_x(SesGrid G, const uint8_t *__restrict__ sas,
+__global__ __launch_bounds__(256) void k_ses_edt_x(SesGrid G, const uint32_t *__restrict__ bits,
                                                    uint16_t *__restrict__ g1, long long n_pts) {
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n_pts;
        q += (long long)gridDim.x * blockDim.x) {
-    const long long i = q % G.nx;
+    const long long r = q / G.nx;
+    const int i = (int)(q - r * G.nx);
+    const uint32_t *row = bits + r * G.wx;
+    auto out = [&](int at) { return ((row[at >> 5] >> (at & 31)) & 1u) == 0u; };
     uint16_t best = kSesInf;
-    if (!sas[q]) {
+    if (out(i)) {
       best = 0;
     } else {
       for (int d = 1; d <= G.K; ++d) {
-        const bool l = i - d >= 0 && !sas[q - d], r = i + d < G.nx && !sas[q + d];
-        if (l || r) {
+        const bool l = i - d >= 0 && out(i - d), rt = i + d < G.nx && out(i + d);
+        if (l || rt) {
           best = (uint16_t)(d * d);
           break;
         }
@@ -548,6 +695,17 @@ __global__ __launch_bounds__(256) void k_ses_bbox(const float4 *__restrict__ X, 
 
 int ses_window(float probe, float h) { return (int)std::ceil((double)probe / (double)h) + 1; }
 
+bool ses_three_pass(float probe, float h) { return ses_window(probe, h) > kSesBitK; }
+
+long long ses_words(const int32_t dims[3]) { return ((long long)dims[0] + 31) / 32 * dims[1] * dims[2]; }
+
+template <int K>
+static void launch_levels(const SesGrid &G, const SesLaunch &L, cudaStream_t st) {
+  using S = SesSteps<K>;
+  const long long tiles = (long long)G.wx * (((long long)G.ny + S::TY - 1) / S::TY) * (((long long)G.nz + S::TZ - 1) / S::TZ);
+  k_ses_levels<K><<<(unsigned)tiles, 256, 0, st>>>(G, L.bits, L.edt2);
+}
+
 cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *partial, int n_blocks, cudaStream_t st) {
   k_ses_bbox<<<n_blocks, 256, 0, st>>>(X, n, probe, partial);
   return cudaGetLastError();
@@ -558,7 +716,7 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
   cudaGetDevice(&dev);
   if (!ses_table_ready(dev)) return cudaErrorInvalidValue;
   SesGrid G{L.origin[0], L.origin[1], L.origin[2], L.h, L.probe, L.dims[0], L.dims[1], L.dims[2],
-            ses_window(L.probe, L.h), 1, 0.0f};
+            (int)(((long long)L.dims[0] + 31) / 32), ses_window(L.probe, L.h), 1, 0.0f};
   {
     // SES interior <=> edt2 >= 1 (inside the SAS) and edt2 * h^2 >= p^2 in FP64: the product is monotone in
     // edt2, so the test is edt2 >= t_in for the smallest such integer
@@ -577,17 +735,33 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
   }
   const long long n_pts = (long long)G.nx * G.ny * G.nz;
   const int sms = sm_count();
-  cudaError_t e = cudaMemsetAsync(L.sas, 0, (size_t)n_pts, st);
+  cudaError_t e = cudaMemsetAsync(L.bits, 0, 4 * (size_t)ses_words(L.dims), st);
   if (e != cudaSuccess) return e;
   if (L.n_atoms > 0) {
-    const long long warps = L.n_atoms < 64LL * sms * 8 ? L.n_atoms : 64LL * sms * 8;
-    k_ses_sas<<<(int)((warps * 32 + 255) / 256), 256, 0, st>>>(G, L.X, L.n_atoms, L.sas);
+    // one warp per atom, or up to 8 when the atoms alone would not fill the GPU (8 CTAs of 8 warps per SM)
+    const long long fill = 64LL * sms;
+    const long long share = fill / L.n_atoms;
+    const int parts = (int)(share < 1 ? 1 : (share > 8 ? 8 : share));
+    const long long warps = L.n_atoms * parts < 8 * fill ? L.n_atoms * parts : 8 * fill;
+    k_ses_sas<<<(int)((warps * 32 + 255) / 256), 256, 0, st>>>(G, L.X, L.n_atoms, parts, L.bits);
   }
   const long long pb = (n_pts + 255) / 256;
   const int grid = (int)(pb < 16LL * sms ? pb : 16LL * sms);
-  k_ses_edt_x<<<grid, 256, 0, st>>>(G, L.sas, L.g_a, n_pts);
-  k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_a, L.g_b, n_pts, (long long)G.nx, (long long)G.ny, 0);
-  k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_b, L.edt2, n_pts, (long long)G.nx * G.ny, (long long)G.nz, 1);
+  if (L.sas) k_ses_sas_bytes<<<grid, 256, 0, st>>>(G, L.bits, n_pts, L.sas);
+  if (G.K <= kSesBitK) {
+    switch (G.K) {
+      case 1: launch_levels<1>(G, L, st); break;
+      case 2: launch_levels<2>(G, L, st); break;
+      case 3: launch_levels<3>(G, L, st); break;
+      case 4: launch_levels<4>(G, L, st); break;
+      case 5: launch_levels<5>(G, L, st); break;
+      default: launch_levels<6>(G, L, st); break;
+    }
+  } else {
+    k_ses_edt_x<<<grid, 256, 0, st>>>(G, L.bits, L.g_a, n_pts);
+    k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_a, L.g_b, n_pts, (long long)G.nx, (long long)G.ny, 0);
+    k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_b, L.edt2, n_pts, (long long)G.nx * G.ny, (long long)G.nz, 1);
+  }
   const long long n_cells = (long long)(G.nx - 1) * (G.ny - 1) * (G.nz - 1);
   const long long n_blocks = (n_cells + kSesCellsPerBlock - 1) / kSesCellsPerBlock;
   if (n_blocks > 0) {

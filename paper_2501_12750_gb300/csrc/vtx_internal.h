@@ -90,8 +90,9 @@ struct SesLaunch {
   float origin[3];
   float h, probe;
   int32_t dims[3];
-  uint8_t *sas;                   // [nz][ny][nx] SAS interior (0/1)
-  uint16_t *g_a, *g_b;            // distance-pass scratch, one value per grid point each
+  uint32_t *bits;                 // [nz][ny][ceil(nx / 32)] SAS interior, one bit per grid point
+  uint8_t *sas;                   // [nz][ny][nx] SAS interior as bytes (0/1), or null
+  uint16_t *g_a, *g_b;            // scratch of the three distance passes (ses_three_pass), one value per grid point
   uint16_t *edt2;                 // [nz][ny][nx] windowed squared distance (grid units)
   uint8_t *cases;                 // [(nz-1)(ny-1)(nx-1)] marching-cubes case of every cell
   unsigned *block_tris;           // [ses_blocks(dims)]
@@ -105,6 +106,8 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st);
 cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *partial, int n_blocks, cudaStream_t st);
 long long ses_blocks(const int32_t dims[3]);
 int ses_window(float probe, float h);
+bool ses_three_pass(float probe, float h);  // the window is too large for the bit-set distance pass
+long long ses_words(const int32_t dims[3]);  // 32-bit words of the interior bits
 
 int sm_count();
 
