@@ -50,7 +50,7 @@ struct vtx_ctx {
       hostin_e, hostout, covlist, covmask, stage, defer;
   bool cov_ok = false;  // the covered-pixel list of the last prepared launch fits (two-pass resolve)
   bool occl_ok = false;  // the occlusion pass's buffers of the last prepared launch fit
-  Buf ses_bits, ses_a, ses_b, ses_edt, ses_blk, ses_base, ses_total, ses_bbox, ses_case;
+  Buf ses_bits, ses_a, ses_b, ses_edt, ses_blk, ses_base, ses_total, ses_bbox, ses_in;
   uint32_t cap_rec = 0;
   unsigned long long cap_entries = 0;
   Status *h_status = nullptr;
@@ -447,7 +447,7 @@ vtx_status vtx_destroy(vtx_ctx *c) {
   Buf *bufs[] = {&c->keys,   &c->surv,   &c->state,  &c->tcount,   &c->tstart,   &c->tcursor,  &c->tlist,
                  &c->bsums,  &c->recs,   &c->recimg, &c->recbox,   &c->recof,    &c->entries,  &c->status,
                  &c->counts, &c->hostin_x, &c->hostin_e, &c->hostout, &c->covlist, &c->covmask, &c->stage, &c->defer, &c->ses_bits, &c->ses_a, &c->ses_b,
-                 &c->ses_edt, &c->ses_blk, &c->ses_base, &c->ses_total, &c->ses_bbox, &c->ses_case};
+                 &c->ses_edt, &c->ses_blk, &c->ses_base, &c->ses_total, &c->ses_bbox, &c->ses_in};
   for (Buf *b : bufs)
     if (b->p) cudaFree(b->p);
   if (c->h_status) cudaFreeHost(c->h_status);
@@ -1246,14 +1246,14 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
     return fail(c, VTX_ERR_INVALID_ARG, "ses: misaligned output");
   const long long nb = ses_blocks(g->dims);
   vtx_status st;
-  if ((st = ensure(c, c->ses_bits, 4 * (size_t)ses_words(g->dims), "ses interior"))) return st;
+  if ((st = ensure(c, c->ses_bits, 4 * (size_t)(ses_words(g->dims) + 1), "ses interior"))) return st;
+  if ((st = ensure(c, c->ses_in, 4 * (size_t)ses_words(g->dims), "ses surface interior"))) return st;
   if (ses_three_pass(g->probe, g->spacing)) {
     if ((st = ensure(c, c->ses_a, 2 * (size_t)n_pts, "ses pass a"))) return st;
     if ((st = ensure(c, c->ses_b, 2 * (size_t)n_pts, "ses pass b"))) return st;
   }
   if (!de && (st = ensure(c, c->ses_edt, 2 * (size_t)n_pts, "ses edt"))) return st;
   if ((st = ensure(c, c->ses_blk, sizeof(unsigned) * (size_t)(nb + 1), "ses blocks"))) return st;
-  if ((st = ensure(c, c->ses_case, (size_t)n_pts, "ses cases"))) return st;  // >= one byte per cell
   if ((st = ensure(c, c->ses_base, sizeof(unsigned long long) * (size_t)(nb + 1), "ses bases"))) return st;
   if ((st = ensure(c, c->ses_total, sizeof(unsigned long long), "ses total"))) return st;
   SesLaunch L;
@@ -1266,11 +1266,11 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
   L.h = g->spacing;
   L.probe = g->probe;
   L.bits = (uint32_t *)c->ses_bits.p;
+  L.inside = (uint32_t *)c->ses_in.p;
   L.sas = (uint8_t *)ds;
   L.g_a = (uint16_t *)c->ses_a.p;
   L.g_b = (uint16_t *)c->ses_b.p;
   L.edt2 = de ? (uint16_t *)de : (uint16_t *)c->ses_edt.p;
-  L.cases = (uint8_t *)c->ses_case.p;
   L.block_tris = (unsigned *)c->ses_blk.p;
   L.block_base = (unsigned long long *)c->ses_base.p;
   L.total = (unsigned long long *)c->ses_total.p;

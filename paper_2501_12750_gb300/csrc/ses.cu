@@ -14,15 +14,16 @@
 //      sets of the points within each possible distance; larger windows: three
 //      separable min-plus passes (x, y, z).
 //   3. SES interior: edt2 >= 1 and edt2 h^2 >= p^2 (FP64; an integer threshold
-//      here, as the product is monotone in edt2).  Marching cubes in two passes:
-//      each CTA classifies a run of cells (one case byte per cell) and counts
-//      their triangles, one CTA scans the counts, then each CTA writes its
-//      cells' triangles in cell order, so the output order is deterministic.  The per-case
-//      loops come from a table built once on the host: faces with four
-//      crossings cut their inside corners apart, segments are directed by the
-//      face's outward normal so loops turn counter-clockwise about the
-//      outward (inside to outside) normal, and loops longer than three edges
-//      become a star of triangles around their mean vertex.
+//      here, as the product is monotone in edt2), again one bit per point.
+//      Marching cubes in two passes over "groups" of 32 cells of a row: one
+//      counts the triangles of every 256 groups (the last CTA scans the
+//      counts), the other writes them in cell order, so the output order is
+//      deterministic.  The per-case loops come from a table built once on the
+//      host: faces with four crossings cut their inside corners apart, segments
+//      are directed by the face's outward normal so loops turn
+//      counter-clockwise about the outward (inside to outside) normal, and
+//      loops longer than three edges become a star of triangles around their
+//      mean vertex.
 #include <cmath>
 #include <mutex>
 #include <utility>
@@ -32,23 +33,19 @@
 namespace vtx {
 
 constexpr int kSesThreads = 256;
-constexpr int kSesCellsPerThread = 4;
-constexpr int kSesCellsPerBlock = kSesThreads * kSesCellsPerThread;
+constexpr int kSesGroups = 256;  // groups of 32 cells per CTA of the marching-cubes passes
 constexpr uint16_t kSesInf = 0xffffu;
 
-// Per case: number of loops, their lengths, and their edges back to back.
-struct SesCase {
+// Per case: number of loops, their lengths, their edges back to back, and the triangles as three 4-bit vertex
+// codes each (0..11: the vertex on that edge; 12 + l: the mean of loop l).
+struct __align__(16) SesCase {
   unsigned char n_loops;
   unsigned char n_tris;
   unsigned char len[4];
   unsigned char edge[12];
+  unsigned short tri[12];
 };
-__constant__ SesCase c_ses_case[256];
-
-// Corners (x, y, z offsets) and edges (corner pairs) of a cell.
-__constant__ int c_corner[8][3] = {{0, 0, 0}, {1, 0, 0}, {1, 1, 0}, {0, 1, 0}, {0, 0, 1}, {1, 0, 1}, {1, 1, 1}, {0, 1, 1}};
-__constant__ int c_edge[12][2] = {{0, 1}, {1, 2}, {2, 3}, {3, 0}, {4, 5}, {5, 6},
-                                  {6, 7}, {7, 4}, {0, 4}, {1, 5}, {2, 6}, {3, 7}};
+__device__ SesCase g_ses_case[256];
 
 // ------------------------------------------------------------ case table --
 
@@ -124,8 +121,14 @@ SesCase build_case(int cs) {
       seen[e] = true;
       out.edge[at + L++] = (unsigned char)e;
     }
+    const unsigned char *e = out.edge + at;
+    if (L == 3) {
+      out.tri[out.n_tris++] = (unsigned short)(e[0] | e[1] << 4 | e[2] << 8);
+    } else {
+      for (int v = 0; v < L; ++v)
+        out.tri[out.n_tris++] = (unsigned short)((12 + out.n_loops) | e[v] << 4 | e[v + 1 == L ? 0 : v + 1] << 8);
+    }
     out.len[out.n_loops++] = (unsigned char)L;
-    out.n_tris += (unsigned char)(L == 3 ? 1 : L);
     at += L;
   }
   return out;
@@ -136,13 +139,13 @@ bool g_table_ok[64];
 
 }  // namespace
 
-// Upload the case table to this device's constant memory (once per device).
+// Upload the case table to this device's memory (once per device).
 static bool ses_table_ready(int device) {
   if (device < 0 || device >= 64) return false;
   std::call_once(g_table_once[device], [device] {
     SesCase t[256];
     for (int cs = 0; cs < 256; ++cs) t[cs] = build_case(cs);
-    g_table_ok[device] = cudaMemcpyToSymbol(c_ses_case, t, sizeof(t)) == cudaSuccess;
+    g_table_ok[device] = cudaMemcpyToSymbol(g_ses_case, t, sizeof(t)) == cudaSuccess;
   });
   return g_table_ok[device];
 }
@@ -315,15 +318,18 @@ constexpr SesSteps<K> kSesSteps{};
 template <int K>
 struct SesLevelState {
   uint32_t acc = 0u, prev = 0u;  // points within the levels so far; within the levels before the current one
+  uint32_t outside = 0u;         // points whose distance is below the SES threshold
   uint32_t plane[6] = {};        // binary digits of each point's level
 };
 
 template <int K, int I>
-__device__ __forceinline__ void ses_step(const uint32_t *e, SesLevelState<K> &s) {
+__device__ __forceinline__ void ses_step(const uint32_t *e, int t_in, SesLevelState<K> &s) {
   constexpr int off = kSesSteps<K>.off[I], lv = kSesSteps<K>.level[I];
   constexpr bool last = kSesSteps<K>.level[I + 1] != lv;
   s.acc |= e[off];
   if constexpr (last) {
+    constexpr int value = kSesSteps<K>.value[lv];
+    if (value < t_in) s.outside = s.acc;
     const uint32_t newly = s.acc & ~s.prev;
     if constexpr ((lv & 1) != 0) s.plane[0] |= newly;
     if constexpr ((lv & 2) != 0) s.plane[1] |= newly;
@@ -336,8 +342,9 @@ __device__ __forceinline__ void ses_step(const uint32_t *e, SesLevelState<K> &s)
 }
 
 template <int K, int... I>
-__device__ __forceinline__ void ses_steps(const uint32_t *e, SesLevelState<K> &s, std::integer_sequence<int, I...>) {
-  (ses_step<K, I>(e, s), ...);
+__device__ __forceinline__ void ses_steps(const uint32_t *e, int t_in, SesLevelState<K> &s,
+                                          std::integer_sequence<int, I...>) {
+  (ses_step<K, I>(e, t_in, s), ...);
 }
 
 // s_val[level] = its squared length (the last one: the sentinel).
@@ -363,7 +370,7 @@ __device__ __forceinline__ void ses_values(uint16_t *s_val, std::integer_sequenc
 // grow with K^3 (519 at K = 6) and every one is an unrolled instruction.
 template <int K>
 __global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *__restrict__ bits,
-                                                    uint16_t *__restrict__ edt2) {
+                                                    uint16_t *__restrict__ edt2, uint32_t *__restrict__ inside) {
   using S = SesSteps<K>;
   constexpr int n_levels = kSesSteps<K>.n_levels;
   __shared__ uint32_t s_e[(K + 1) * S::PL];
@@ -393,7 +400,7 @@ __global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *_
   }
   __syncthreads();
   SesLevelState<K> st;
-  ses_steps<K>(s_e + (zw + K) * S::PY + lane + K, st, std::make_integer_sequence<int, kSesSteps<K>.n>{});
+  ses_steps<K>(s_e + (zw + K) * S::PY + lane + K, G.t_in, st, std::make_integer_sequence<int, kSesSteps<K>.n>{});
   const uint32_t rest = ~st.acc;  // farther than K: the last level
 #pragma unroll
   for (int p = 0; p < 6; ++p)
@@ -403,6 +410,7 @@ __global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *_
   const long long z = z0 + zw, x = 32LL * w + lane;
   if (z >= G.nz) return;  // uniform in the warp; no barrier follows
   const int rows = (int)min((long long)S::TY, G.ny - y0);
+  if (lane < rows) inside[(z * G.ny + y0 + lane) * G.wx + w] = ~st.outside;
   uint16_t *dst = edt2 + (z * G.ny + y0) * G.nx + x;
   for (int r = 0; r < rows; ++r, dst += G.nx) {
     unsigned lv = 0u;
@@ -468,34 +476,64 @@ __global__ __launch_bounds__(256) void k_ses_edt_yz(SesGrid G, const uint16_t *_
   }
 }
 
-
-
-__device__ __forceinline__ int cell_case(const SesGrid &G, const uint16_t *__restrict__ edt, long long i, long long j,
-                                         long long k) {
-  int cs = 0;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const long long q = ((k + c_corner[c][2]) * G.ny + (j + c_corner[c][1])) * (long long)G.nx + (i + c_corner[c][0]);
-    if ((int)edt[q] >= G.t_in) cs |= 1 << c;
+// SES interior bits from the distances (three-pass windows): one warp per word.
+__global__ __launch_bounds__(256) void k_ses_inside(SesGrid G, const uint16_t *__restrict__ edt2, long long n_words,
+                                                    uint32_t *__restrict__ inside) {
+  const int lane = threadIdx.x & 31;
+  const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  for (long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n_words; q += n_warps) {
+    const long long row = q / G.wx;
+    const int x = 32 * (int)(q - row * G.wx) + lane;
+    const unsigned m = __ballot_sync(0xffffffffu, x < G.nx && (int)edt2[row * G.nx + x] >= G.t_in);
+    if (lane == 0) inside[q] = m;
   }
-  return cs;
 }
 
-// Triangles of the cells [c0, c0 + kSesCellsPerThread) of a thread; their cases
-// are stored (one byte per cell) for the emit pass.
-__device__ __forceinline__ int thread_cells_count(const SesGrid &G, const uint16_t *__restrict__ edt, long long c0,
-                                                  long long n_cells, uint8_t *__restrict__ cases) {
-  int n = 0;
-  const long long cx = G.nx - 1, cy = G.ny - 1;
-  for (int u = 0; u < kSesCellsPerThread; ++u) {
-    const long long c = c0 + u;
-    if (c >= n_cells) break;
-    const long long i = c % cx, j = (c / cx) % cy, k = c / (cx * cy);
-    const int cs = cell_case(G, edt, i, j, k);
-    cases[c] = (uint8_t)cs;
-    n += c_ses_case[cs].n_tris;
-  }
-  return n;
+// --------------------------------------------------------- marching cubes --
+
+// The corner bits of a group's 32 cells (i0 .. i0 + 31 of row (j, k)) and which of the cells cross the surface.
+struct SesGroup {
+  int i0, j, k;
+  uint32_t c[8];   // c[q] bit t: corner q of cell i0 + t is inside
+  uint32_t active;
+};
+
+__device__ __forceinline__ SesGroup ses_group(const SesGrid &G, const uint32_t *__restrict__ inside, uint32_t g,
+                                              uint32_t n_groups) {
+  SesGroup s;
+  const uint32_t wc = (uint32_t)(G.nx + 30) / 32u;  // groups per row of nx - 1 cells
+  const uint32_t row = g / wc, w = g - row * wc;
+  s.i0 = (int)(w * 32u);
+  s.k = (int)(row / (uint32_t)(G.ny - 1));
+  s.j = (int)(row - (uint32_t)s.k * (uint32_t)(G.ny - 1));
+  s.active = 0u;
+  if (g >= n_groups) return s;
+  const uint32_t *p = inside + ((size_t)s.k * G.ny + s.j) * G.wx + w;
+  const size_t up = (size_t)G.ny * G.wx;
+  const bool next = (int)w + 1 < G.wx;
+  const uint32_t r0 = p[0], r1 = p[G.wx], r2 = p[up], r3 = p[up + G.wx];
+  const uint32_t n0 = next ? p[1] : 0u, n1 = next ? p[G.wx + 1] : 0u;
+  const uint32_t n2 = next ? p[up + 1] : 0u, n3 = next ? p[up + G.wx + 1] : 0u;
+  s.c[0] = r0;
+  s.c[3] = r1;
+  s.c[4] = r2;
+  s.c[7] = r3;
+  s.c[1] = __funnelshift_r(r0, n0, 1);
+  s.c[2] = __funnelshift_r(r1, n1, 1);
+  s.c[5] = __funnelshift_r(r2, n2, 1);
+  s.c[6] = __funnelshift_r(r3, n3, 1);
+  const uint32_t any = s.c[0] | s.c[1] | s.c[2] | s.c[3] | s.c[4] | s.c[5] | s.c[6] | s.c[7];
+  const uint32_t all = s.c[0] & s.c[1] & s.c[2] & s.c[3] & s.c[4] & s.c[5] & s.c[6] & s.c[7];
+  const int cells = G.nx - 1 - s.i0;  // > 0
+  s.active = any & ~all & (cells >= 32 ? 0xffffffffu : (1u << cells) - 1u);
+  return s;
+}
+
+__device__ __forceinline__ unsigned ses_case_of(const SesGroup &s, int t) {
+  unsigned cs = 0u;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) cs |= ((s.c[q] >> t) & 1u) << q;
+  return cs;
 }
 
 __device__ __forceinline__ unsigned block_exclusive_sum(unsigned v, unsigned *total) {
@@ -509,151 +547,210 @@ __device__ __forceinline__ unsigned block_exclusive_sum(unsigned v, unsigned *to
   }
   if (lane == 31) s_warp[w] = x;
   __syncthreads();
-  if (w == 0) {
-    unsigned s = lane < kSesThreads / 32 ? s_warp[lane] : 0u;
+  unsigned before = x - v, sum = 0u;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
-    }
-    if (lane < kSesThreads / 32) s_warp[lane] = s;
+  for (int q = 0; q < kSesThreads / 32; ++q) {
+    const unsigned t = s_warp[q];
+    if (q < w) before += t;
+    sum += t;
   }
   __syncthreads();
-  const unsigned before = (w > 0 ? s_warp[w - 1] : 0u) + x - v;
-  if (total) *total = s_warp[kSesThreads / 32 - 1];
-  __syncthreads();
+  *total = sum;
   return before;
 }
 
-__global__ __launch_bounds__(kSesThreads) void k_ses_count(SesGrid G, const uint16_t *__restrict__ edt,
-                                                           long long n_cells, uint8_t *__restrict__ cases,
-                                                           unsigned *__restrict__ block_tris) {
-  const long long c0 = (long long)blockIdx.x * kSesCellsPerBlock + (long long)threadIdx.x * kSesCellsPerThread;
-  unsigned total;
-  block_exclusive_sum((unsigned)thread_cells_count(G, edt, c0, n_cells, cases), &total);
-  if (threadIdx.x == 0) block_tris[blockIdx.x] = total;
-}
-
-// Exclusive scan of the per-block counts in one CTA (64-bit totals).
-__global__ __launch_bounds__(kSesThreads) void k_ses_scan(const unsigned *__restrict__ block_tris, long long n_blocks,
-                                                          unsigned long long *__restrict__ block_base,
-                                                          unsigned long long *__restrict__ total) {
-  __shared__ unsigned long long s_carry;
-  if (threadIdx.x == 0) s_carry = 0ull;
+// Triangles of every 256 groups (one group per thread, going through its crossing cells), and, in the last CTA to
+// finish, their exclusive scan: block_base[b] is the first triangle of CTA b's groups.  *done counts finished CTAs
+// (zero at launch); no CTA waits for another.  3.4e7 points: 27 us, of which most is the table lookups of the
+// crossing cells; 307 us with one thread per four cells reading the distance plane, and 100 us for the scan of
+// its eight times as many counts in a launch of its own.
+__global__ __launch_bounds__(kSesThreads) void k_ses_count(SesGrid G, const uint32_t *__restrict__ inside,
+                                                           uint32_t n_groups, unsigned *__restrict__ block_tris,
+                                                           unsigned long long *__restrict__ block_base,
+                                                           unsigned long long *__restrict__ total, unsigned *done) {
+  __shared__ unsigned char s_tris[256];
+  __shared__ bool s_last;
+  s_tris[threadIdx.x] = g_ses_case[threadIdx.x].n_tris;
   __syncthreads();
-  for (long long b0 = 0; b0 < n_blocks; b0 += kSesThreads) {
-    const long long b = b0 + threadIdx.x;
-    const unsigned v = b < n_blocks ? block_tris[b] : 0u;
-    unsigned tot;
-    const unsigned ex = block_exclusive_sum(v, &tot);
-    if (b < n_blocks) block_base[b] = s_carry + ex;
+  const SesGroup s = ses_group(G, inside, blockIdx.x * (unsigned)kSesGroups + threadIdx.x, n_groups);
+  unsigned n = 0u;
+  for (uint32_t m = s.active; m != 0u; m &= m - 1u) n += s_tris[ses_case_of(s, __ffs(m) - 1)];
+  unsigned sum;
+  block_exclusive_sum(n, &sum);
+  if (threadIdx.x == 0) {
+    block_tris[blockIdx.x] = sum;
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  // consecutive counts per thread: their sum, a block scan of the sums (64 bits in two halves), then the bases
+  __threadfence();
+  const unsigned nb = gridDim.x, per = (nb + kSesThreads - 1) / kSesThreads;
+  const unsigned b0 = min(threadIdx.x * per, nb), b1 = min(b0 + per, nb);
+  unsigned long long mine = 0ull;
+#pragma unroll 8
+  for (unsigned b = b0; b < b1; ++b) mine += __ldcg(block_tris + b);
+  __shared__ unsigned long long s_sum[kSesThreads];
+  s_sum[threadIdx.x] = mine;
+  __syncthreads();
+  for (int o = 1; o < kSesThreads; o <<= 1) {
+    const unsigned long long y = (int)threadIdx.x >= o ? s_sum[threadIdx.x - o] : 0ull;
     __syncthreads();
-    if (threadIdx.x == 0) s_carry += tot;
+    s_sum[threadIdx.x] += y;
     __syncthreads();
   }
-  if (threadIdx.x == 0) *total = s_carry;
-}
-
-__device__ __forceinline__ void store_tri(float *__restrict__ tris, long long *__restrict__ labels,
-                                          unsigned long long t, unsigned long long max_tris, const float3 &a,
-                                          const float3 &b, const float3 &c, long long la, long long lb, long long lc) {
-  if (t >= max_tris) return;
-  float *o = tris + t * 9;
-  o[0] = a.x, o[1] = a.y, o[2] = a.z;
-  o[3] = b.x, o[4] = b.y, o[5] = b.z;
-  o[6] = c.x, o[7] = c.y, o[8] = c.z;
-  if (labels) {
-    labels[t * 3] = la;
-    labels[t * 3 + 1] = lb;
-    labels[t * 3 + 2] = lc;
+  unsigned long long run = s_sum[threadIdx.x] - mine;
+#pragma unroll 8
+  for (unsigned b = b0; b < b1; ++b) {
+    block_base[b] = run;
+    run += __ldcg(block_tris + b);
   }
+  if (threadIdx.x == kSesThreads - 1) *total = s_sum[threadIdx.x];
 }
 
-// Vertex on edge e of cell (i, j, k): X_a + t (X_b - X_a), t = f_a / (f_a - f_b) clamped.
-__device__ __forceinline__ float3 edge_vertex(const SesGrid &G, const uint16_t *__restrict__ edt, long long i,
-                                              long long j, long long k, int e) {
-  const int a = c_edge[e][0], b = c_edge[e][1];
-  const long long ai = i + c_corner[a][0], aj = j + c_corner[a][1], ak = k + c_corner[a][2];
-  const long long bi = i + c_corner[b][0], bj = j + c_corner[b][1], bk = k + c_corner[b][2];
-  const float fa = sqrtf((float)edt[(ak * G.ny + aj) * (long long)G.nx + ai]) * G.h - G.p;
-  const float fb = sqrtf((float)edt[(bk * G.ny + bj) * (long long)G.nx + bi]) * G.h - G.p;
-  float s = fa == fb ? 0.5f : fa / (fa - fb);
-  s = fminf(fmaxf(s, 0.0f), 1.0f);
-  const float3 A = make_float3(G.ox + G.h * (float)ai, G.oy + G.h * (float)aj, G.oz + G.h * (float)ak);
-  const float3 B = make_float3(G.ox + G.h * (float)bi, G.oy + G.h * (float)bj, G.oz + G.h * (float)bk);
-  return make_float3(A.x + s * (B.x - A.x), A.y + s * (B.y - A.y), A.z + s * (B.z - A.z));
+// Position of the vertex at parameter t on edge e of cell (i, j, k): X_a + t (X_b - X_a).
+__device__ __forceinline__ float3 edge_point(const SesGrid &G, int i, int j, int k, int e, float t) {
+  // edges 0-3 and 4-7 go round the squares z = 0 and z = 1 from corner (0, 0) in +x, +y, -x, -y; 8-11 in +z
+  const int q = e & 3;
+  const int ax = (q == 1 || q == 2) ? 1 : 0, ay = q >> 1, az = (e >= 4 && e < 8) ? 1 : 0;
+  const int dz = e >= 8 ? 1 : 0;
+  const int dx = dz ? 0 : (q == 0) - (q == 2), dy = dz ? 0 : (q == 1) - (q == 3);
+  const float3 A = make_float3(fmaf(G.h, (float)(i + ax), G.ox), fmaf(G.h, (float)(j + ay), G.oy),
+                               fmaf(G.h, (float)(k + az), G.oz));
+  const float3 B = make_float3(fmaf(G.h, (float)(i + ax + dx), G.ox), fmaf(G.h, (float)(j + ay + dy), G.oy),
+                               fmaf(G.h, (float)(k + az + dz), G.oz));
+  return make_float3(fmaf(t, B.x - A.x, A.x), fmaf(t, B.y - A.y, A.y), fmaf(t, B.z - A.z, A.z));
 }
 
-// One thread per output triangle of the CTA's run of cells: the cells'
-// triangle offsets are scanned into shared memory, each thread finds its cell
-// by binary search, its loop and fan position from the case table, and writes
-// its triangle next to its neighbours' (coalesced).
+// Shared memory of the emit pass, for 256 crossing cells at a time.
+struct SesEmitShared {
+  float t[12][kSesThreads];        // vertex parameter of every crossing edge of each cell
+  float mean[12][kSesThreads];     // means of its loops: x, y, z of loop l at 3 l
+  float stage[kSesThreads / 32][32 * 9];  // per warp: 32 triangles on their way out
+  int ci[kSesThreads], cj[kSesThreads], ck[kSesThreads];
+  unsigned off[kSesThreads];       // first triangle of each cell
+  unsigned char cs[kSesThreads];   // case
+  unsigned char cell_of[kSesThreads * 12];  // cell of each triangle
+};
+
+// Triangles of the groups of CTA blockIdx.x, in cell order.  The groups' crossing cells are taken 256 at a time,
+// one per thread: the eight distances are read once and give the parameter of every crossing edge and the means
+// of the longer loops; then one thread per triangle puts its three vertices together and the warp writes its 32
+// triangles as one run of floats.
+//
+// Bound by issue (a crossing cell has about five vertices and two triangles) and the triangles' writes.  5.9e6
+// triangles (212 MB): 146 us; 789 us with one thread per triangle finding its cell by binary search over
+// a case byte per cell, recomputing its loop's vertices from the distance plane and storing 36-byte strides.
 __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint16_t *__restrict__ edt,
-                                                          const uint8_t *__restrict__ cases, long long n_cells,
+                                                          const uint32_t *__restrict__ inside, uint32_t n_groups,
                                                           const unsigned long long *__restrict__ block_base,
                                                           float *__restrict__ tris, long long *__restrict__ labels,
                                                           unsigned long long max_tris) {
-  __shared__ unsigned s_off[kSesCellsPerBlock + 1];
-  __shared__ unsigned char s_case[kSesCellsPerBlock];
-  const long long cb = (long long)blockIdx.x * kSesCellsPerBlock;
-  unsigned n4[kSesCellsPerThread];
-  unsigned mine = 0;
-  for (int u = 0; u < kSesCellsPerThread; ++u) {
-    const int lc = threadIdx.x * kSesCellsPerThread + u;
-    const unsigned char cs = cb + lc < n_cells ? cases[cb + lc] : 0;
-    s_case[lc] = cs;
-    n4[u] = c_ses_case[cs].n_tris;
-    mine += n4[u];
-  }
-  unsigned total;
-  unsigned run = block_exclusive_sum(mine, &total);
-  for (int u = 0; u < kSesCellsPerThread; ++u) {
-    s_off[threadIdx.x * kSesCellsPerThread + u] = run;
-    run += n4[u];
-  }
-  if (threadIdx.x == 0) s_off[kSesCellsPerBlock] = total;
-  __syncthreads();
-  const unsigned long long base_t = block_base[blockIdx.x];
-  const long long cx = G.nx - 1, cy = G.ny - 1;
-  for (unsigned q = threadIdx.x; q < total; q += kSesThreads) {
-    int lo = 0, hi = kSesCellsPerBlock - 1;  // last cell with s_off <= q
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (s_off[mid] <= q) lo = mid; else hi = mid - 1;
+  __shared__ SesEmitShared sh;
+  unsigned long long base = block_base[blockIdx.x];
+  if (base >= max_tris) return;
+  const SesGroup s = ses_group(G, inside, blockIdx.x * (unsigned)kSesGroups + threadIdx.x, n_groups);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  unsigned n_cells;
+  unsigned rank = block_exclusive_sum((unsigned)__popc(s.active), &n_cells);
+  uint32_t rem = s.active;
+  const size_t ny = (size_t)G.ny, nx = (size_t)G.nx;
+  for (unsigned c0 = 0; c0 < n_cells; c0 += kSesThreads) {
+    for (; rem != 0u && rank < c0 + kSesThreads; rem &= rem - 1u, ++rank) {
+      const int t = __ffs(rem) - 1;
+      const unsigned at = rank - c0;
+      sh.ci[at] = s.i0 + t;
+      sh.cj[at] = s.j;
+      sh.ck[at] = s.k;
+      sh.cs[at] = (unsigned char)ses_case_of(s, t);
     }
-    const long long c = cb + lo;
-    const SesCase &tc = c_ses_case[s_case[lo]];
-    unsigned r = q - s_off[lo];
-    int at = 0, l = 0;
-    while (l < tc.n_loops) {
-      const unsigned nt = tc.len[l] == 3 ? 1u : tc.len[l];
-      if (r < nt) break;
-      r -= nt;
-      at += tc.len[l];
-      ++l;
-    }
-    const long long i = c % cx, j = (c / cx) % cy, k = c / (cx * cy);
-    const long long base = c * 16;
-    const int L = tc.len[l];
-    if (L == 3) {
-      const int e0 = tc.edge[at], e1 = tc.edge[at + 1], e2 = tc.edge[at + 2];
-      store_tri(tris, labels, base_t + q, max_tris, edge_vertex(G, edt, i, j, k, e0), edge_vertex(G, edt, i, j, k, e1),
-                edge_vertex(G, edt, i, j, k, e2), base + e0, base + e1, base + e2);
-    } else {
-      float3 M = make_float3(0.0f, 0.0f, 0.0f);
-      for (int v = 0; v < L; ++v) {
-        const float3 p = edge_vertex(G, edt, i, j, k, tc.edge[at + v]);
-        M.x += p.x;
-        M.y += p.y;
-        M.z += p.z;
+    __syncthreads();
+    unsigned n_tri = 0u;
+    const bool have = c0 + tid < n_cells;
+    if (have) {
+      const int i = sh.ci[tid], j = sh.cj[tid], k = sh.ck[tid];
+      const unsigned cs = sh.cs[tid];
+      const SesCase &tc = g_ses_case[cs];
+      n_tri = tc.n_tris;
+      const uint16_t *q = edt + ((size_t)k * ny + (size_t)j) * nx + (size_t)i;
+      const size_t up = ny * nx;
+      float f[8];
+      f[0] = (float)q[0];
+      f[1] = (float)q[1];
+      f[2] = (float)q[nx + 1];
+      f[3] = (float)q[nx];
+      f[4] = (float)q[up];
+      f[5] = (float)q[up + 1];
+      f[6] = (float)q[up + nx + 1];
+      f[7] = (float)q[up + nx];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) f[c] = fmaf(sqrtf(f[c]), G.h, -G.p);
+      constexpr int ea[12] = {0, 1, 2, 3, 4, 5, 6, 7, 0, 1, 2, 3};
+      constexpr int eb[12] = {1, 2, 3, 0, 5, 6, 7, 4, 4, 5, 6, 7};
+#pragma unroll
+      for (int e = 0; e < 12; ++e) {
+        if (((cs >> ea[e]) ^ (cs >> eb[e])) & 1u) {
+          const float fa = f[ea[e]], fb = f[eb[e]];
+          const float t = fa == fb ? 0.5f : fa / (fa - fb);
+          sh.t[e][tid] = fminf(fmaxf(t, 0.0f), 1.0f);
+        }
       }
-      const float inv = 1.0f / (float)L;
-      M = make_float3(M.x * inv, M.y * inv, M.z * inv);
-      const int q0 = (int)r, q1 = q0 + 1 == L ? 0 : q0 + 1;
-      const int ea = tc.edge[at + q0], eb = tc.edge[at + q1];
-      store_tri(tris, labels, base_t + q, max_tris, M, edge_vertex(G, edt, i, j, k, ea),
-                edge_vertex(G, edt, i, j, k, eb), base + 12 + l, base + ea, base + eb);
+      for (int l = 0, at = 0; l < tc.n_loops; at += tc.len[l], ++l) {
+        const int len = tc.len[l];
+        if (len == 3) continue;
+        float3 M = make_float3(0.0f, 0.0f, 0.0f);
+        for (int v = 0; v < len; ++v) {
+          const int e = tc.edge[at + v];
+          const float3 p = edge_point(G, i, j, k, e, sh.t[e][tid]);
+          M.x += p.x;
+          M.y += p.y;
+          M.z += p.z;
+        }
+        const float inv = 1.0f / (float)len;
+        sh.mean[3 * l][tid] = M.x * inv;
+        sh.mean[3 * l + 1][tid] = M.y * inv;
+        sh.mean[3 * l + 2][tid] = M.z * inv;
+      }
     }
+    unsigned total;
+    const unsigned off = block_exclusive_sum(n_tri, &total);
+    sh.off[tid] = off;
+    for (unsigned t = 0; t < n_tri; ++t) sh.cell_of[off + t] = (unsigned char)tid;
+    __syncthreads();
+    for (unsigned q0 = 32u * wid; q0 < total && base + q0 < max_tris; q0 += kSesThreads) {
+      const unsigned q = q0 + lane;
+      const unsigned live = min(min(32u, total - q0), (unsigned)min(max_tris - (base + q0), 32ull));
+      if (lane < live) {
+        const int cell = sh.cell_of[q];
+        const int i = sh.ci[cell], j = sh.cj[cell], k = sh.ck[cell];
+        const unsigned code = g_ses_case[sh.cs[cell]].tri[q - sh.off[cell]];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          const int e = (int)((code >> (4 * v)) & 15u);
+          float3 p;
+          if (e < 12)
+            p = edge_point(G, i, j, k, e, sh.t[e][cell]);
+          else
+            p = make_float3(sh.mean[3 * (e - 12)][cell], sh.mean[3 * (e - 12) + 1][cell], sh.mean[3 * (e - 12) + 2][cell]);
+          sh.stage[wid][9 * lane + 3 * v] = p.x;
+          sh.stage[wid][9 * lane + 3 * v + 1] = p.y;
+          sh.stage[wid][9 * lane + 3 * v + 2] = p.z;
+          if (labels) {
+            const long long cell_id = ((long long)k * (G.ny - 1) + j) * (G.nx - 1) + i;
+            labels[(base + q) * 3 + v] = cell_id * 16 + e;
+          }
+        }
+      }
+      __syncwarp();
+      float *out = tris + (base + q0) * 9;
+#pragma unroll
+      for (unsigned o = 0; o < 9; ++o)
+        if (32u * o + lane < 9u * live) out[32u * o + lane] = sh.stage[wid][32u * o + lane];
+      __syncwarp();
+    }
+    base += total;
+    __syncthreads();  // the cells are read before the next ones replace them
   }
 }
 
@@ -697,13 +794,18 @@ int ses_window(float probe, float h) { return (int)std::ceil((double)probe / (do
 
 bool ses_three_pass(float probe, float h) { return ses_window(probe, h) > kSesBitK; }
 
+// Groups of 32 cells (dims >= 2 and at most 2^32 points: at most 2^31 groups).
+static long long ses_groups(const int32_t dims[3]) {
+  return ((long long)dims[0] + 30) / 32 * (dims[1] - 1) * (dims[2] - 1);
+}
+
 long long ses_words(const int32_t dims[3]) { return ((long long)dims[0] + 31) / 32 * dims[1] * dims[2]; }
 
 template <int K>
 static void launch_levels(const SesGrid &G, const SesLaunch &L, cudaStream_t st) {
   using S = SesSteps<K>;
   const long long tiles = (long long)G.wx * (((long long)G.ny + S::TY - 1) / S::TY) * (((long long)G.nz + S::TZ - 1) / S::TZ);
-  k_ses_levels<K><<<(unsigned)tiles, 256, 0, st>>>(G, L.bits, L.edt2);
+  k_ses_levels<K><<<(unsigned)tiles, 256, 0, st>>>(G, L.bits, L.edt2, L.inside);
 }
 
 cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *partial, int n_blocks, cudaStream_t st) {
@@ -735,7 +837,7 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
   }
   const long long n_pts = (long long)G.nx * G.ny * G.nz;
   const int sms = sm_count();
-  cudaError_t e = cudaMemsetAsync(L.bits, 0, 4 * (size_t)ses_words(L.dims), st);
+  cudaError_t e = cudaMemsetAsync(L.bits, 0, 4 * (size_t)(ses_words(L.dims) + 1), st);  // and the counter after them
   if (e != cudaSuccess) return e;
   if (L.n_atoms > 0) {
     // one warp per atom, or up to 8 when the atoms alone would not fill the GPU (8 CTAs of 8 warps per SM)
@@ -761,23 +863,22 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
     k_ses_edt_x<<<grid, 256, 0, st>>>(G, L.bits, L.g_a, n_pts);
     k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_a, L.g_b, n_pts, (long long)G.nx, (long long)G.ny, 0);
     k_ses_edt_yz<<<grid, 256, 0, st>>>(G, L.g_b, L.edt2, n_pts, (long long)G.nx * G.ny, (long long)G.nz, 1);
+    const long long n_words = ses_words(L.dims);
+    const long long wb = (n_words + 7) / 8;
+    k_ses_inside<<<(int)(wb < 16LL * sms ? wb : 16LL * sms), 256, 0, st>>>(G, L.edt2, n_words, L.inside);
   }
-  const long long n_cells = (long long)(G.nx - 1) * (G.ny - 1) * (G.nz - 1);
-  const long long n_blocks = (n_cells + kSesCellsPerBlock - 1) / kSesCellsPerBlock;
-  if (n_blocks > 0) {
-    k_ses_count<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.edt2, n_cells, L.cases, L.block_tris);
-    k_ses_scan<<<1, kSesThreads, 0, st>>>(L.block_tris, n_blocks, L.block_base, L.total);
-    k_ses_emit<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.edt2, L.cases, n_cells, L.block_base, L.tris,
-                                                           L.labels, (unsigned long long)L.max_tris);
-  } else {
-    cudaMemsetAsync(L.total, 0, sizeof(unsigned long long), st);
+  const long long n_blocks = ses_blocks(L.dims);
+  unsigned *done = reinterpret_cast<unsigned *>(L.bits + ses_words(L.dims));  // cleared with the bits
+  k_ses_count<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.inside, (uint32_t)ses_groups(L.dims), L.block_tris,
+                                                          L.block_base, L.total, done);
+  if (L.max_tris > 0) {
+    k_ses_emit<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(
+        G, L.edt2, L.inside, (uint32_t)ses_groups(L.dims), L.block_base, L.tris, L.labels,
+        (unsigned long long)L.max_tris);
   }
   return cudaGetLastError();
 }
 
-long long ses_blocks(const int32_t dims[3]) {
-  const long long n_cells = (long long)(dims[0] - 1) * (dims[1] - 1) * (dims[2] - 1);
-  return (n_cells + kSesCellsPerBlock - 1) / kSesCellsPerBlock;
-}
+long long ses_blocks(const int32_t dims[3]) { return (ses_groups(dims) + kSesGroups - 1) / kSesGroups; }
 
 }  // namespace vtx

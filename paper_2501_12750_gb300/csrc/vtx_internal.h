@@ -90,11 +90,11 @@ struct SesLaunch {
   float origin[3];
   float h, probe;
   int32_t dims[3];
-  uint32_t *bits;                 // [nz][ny][ceil(nx / 32)] SAS interior, one bit per grid point
+  uint32_t *bits;                 // [nz][ny][ceil(nx / 32)] SAS interior, one bit per grid point, then one word
+  uint32_t *inside;               // [nz][ny][ceil(nx / 32)] SES interior, likewise
   uint8_t *sas;                   // [nz][ny][nx] SAS interior as bytes (0/1), or null
   uint16_t *g_a, *g_b;            // scratch of the three distance passes (ses_three_pass), one value per grid point
   uint16_t *edt2;                 // [nz][ny][nx] windowed squared distance (grid units)
-  uint8_t *cases;                 // [(nz-1)(ny-1)(nx-1)] marching-cubes case of every cell
   unsigned *block_tris;           // [ses_blocks(dims)]
   unsigned long long *block_base; // [ses_blocks(dims)]
   unsigned long long *total;      // [1]
