@@ -402,11 +402,24 @@ vtx_status vtx_ses_fit_grid(vtx_ctx *ctx, const float *xyzr, int64_t n_atoms, fl
  * j) (nx-1) + i; sas (nullable) uint8 and edt2 (nullable) uint16, both
  * [nz][ny][nx].  *n_tris (host) receives the total number of triangles;
  * when it exceeds max_tris only the first max_tris are written and the call
- * returns VTX_ERR_CAPACITY.  Scratch (8 bytes per grid point) is owned by
- * the context.  Synchronises.
+ * returns VTX_ERR_CAPACITY.  Scratch (2.25 bytes per grid point; 6.25 when
+ * p / h > 5) is owned by the context.  Synchronises.
  */
 vtx_status vtx_ses_mesh(vtx_ctx *ctx, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *grid, float *tris,
                         int64_t max_tris, int64_t *labels, uint8_t *sas, uint16_t *edt2, int64_t *n_tris);
+
+/*
+ * The same surface in two calls, for a caller that sizes its triangle buffer
+ * by the count: vtx_ses_count does everything but write triangles (sas and
+ * edt2 as above) and leaves the surface in the context's scratch; vtx_ses_emit
+ * writes the triangles (and labels) of the surface that the latest
+ * vtx_ses_count left, any number of times, until the next vtx_ses_count or
+ * vtx_ses_mesh (VTX_ERR_STATE when there is none).  Capacity and buffers as
+ * for vtx_ses_mesh.  The paper has no counterpart.  Both synchronise.
+ */
+vtx_status vtx_ses_count(vtx_ctx *ctx, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *grid, uint8_t *sas,
+                         uint16_t *edt2, int64_t *n_tris);
+vtx_status vtx_ses_emit(vtx_ctx *ctx, float *tris, int64_t max_tris, int64_t *labels);
 
 /* Synchronise the context's stream and report (once) any device-side error. */
 vtx_status vtx_sync_status(vtx_ctx *ctx);

@@ -204,7 +204,7 @@ class Renderer:
         """Solvent excluded surface on `grid` as a triangle soup (device float32 (T, 3, 3)).
 
         Returns a dict with "tris" and, on request, "labels" (int64 (T, 3)) and the "sas" / "edt2" planes
-        (uint8 / uint16 (nz, ny, nx)).  With max_tris None the call runs twice: once to count.
+        (uint8 / uint16 (nz, ny, nx)).  With max_tris None the triangles are counted first and then written.
         """
         torch = self._torch
         assert self._visible(xyzr) and xyzr.dtype == torch.float32 and xyzr.is_contiguous()
@@ -213,16 +213,18 @@ class Renderer:
         sas = torch.empty((nz, ny, nx), dtype=torch.uint8, device=dev) if planes else None
         edt = torch.empty((nz, ny, nx), dtype=torch.int16, device=dev) if planes else None
         n = ctypes.c_int64(0)
-        if max_tris is None:
-            code = self.lib.vtx_ses_mesh(self.ctx, _ptr(xyzr), xyzr.shape[0], ctypes.byref(grid), None, 0, None,
-                                         None, None, ctypes.byref(n))
-            if code not in (0, 4):
-                self._check(code)
+        counted = max_tris is None
+        if counted:
+            self._check(self.lib.vtx_ses_count(self.ctx, _ptr(xyzr), xyzr.shape[0], ctypes.byref(grid), _ptr(sas),
+                                               _ptr(edt), ctypes.byref(n)))
             max_tris = n.value
         tris = torch.empty((max(max_tris, 1), 3, 3), dtype=torch.float32, device=dev)
         lab = torch.empty((max(max_tris, 1), 3), dtype=torch.int64, device=dev) if labels else None
-        self._check(self.lib.vtx_ses_mesh(self.ctx, _ptr(xyzr), xyzr.shape[0], ctypes.byref(grid), _ptr(tris),
-                                          max_tris, _ptr(lab), _ptr(sas), _ptr(edt), ctypes.byref(n)))
+        if counted:
+            self._check(self.lib.vtx_ses_emit(self.ctx, _ptr(tris), max_tris, _ptr(lab)))
+        else:
+            self._check(self.lib.vtx_ses_mesh(self.ctx, _ptr(xyzr), xyzr.shape[0], ctypes.byref(grid), _ptr(tris),
+                                              max_tris, _ptr(lab), _ptr(sas), _ptr(edt), ctypes.byref(n)))
         out = {"tris": tris[:n.value], "n": n.value}
         if labels:
             out["labels"] = lab[:n.value]

@@ -130,6 +130,8 @@ SIGNATURES = {
     "vtx_ses_fit_grid": ([c_void_p, c_void_p, c_int64, c_float, c_float, c_void_p], c_int32),
     "vtx_ses_mesh": ([c_void_p, c_void_p, c_int64, c_void_p, c_void_p, c_int64, c_void_p, c_void_p, c_void_p,
                       c_void_p], c_int32),
+    "vtx_ses_count": ([c_void_p, c_void_p, c_int64, c_void_p, c_void_p, c_void_p, c_void_p], c_int32),
+    "vtx_ses_emit": ([c_void_p, c_void_p, c_int64, c_void_p], c_int32),
     "vtx_export_rgba8": ([c_void_p, c_void_p, c_void_p, c_int32, c_int32, c_int32, c_float, c_void_p], c_int32),
     "vtx_render_visibility_static": ([c_void_p, c_int64, c_void_p, c_void_p, c_void_p, c_void_p], c_int32),
     "vtx_tuned_settings": ([c_void_p, c_void_p, c_void_p, c_void_p], c_int32),

@@ -54,6 +54,12 @@ struct vtx_ctx {
   uint32_t cap_rec = 0;
   unsigned long long cap_entries = 0;
   Status *h_status = nullptr;
+  struct SesHost {             // page-locked: what the surface calls read back
+    unsigned long long total;  // triangles
+    float box[6];              // fitted bounds
+  } *h_ses = nullptr;
+  vtx_ses_grid ses_grid{};     // grid of the surface that vtx_ses_count left in the scratch
+  bool ses_counted = false;    // it is still there
   long long *h_counts = nullptr;
   int h_counts_cap = 0;
   cudaEvent_t counts_done = nullptr;
@@ -434,6 +440,12 @@ vtx_status vtx_create(vtx_ctx **out, int32_t device, void *cuda_stream) {
     return VTX_ERR_OOM;
   }
   memset(c->h_status, 0, sizeof(Status));
+  if (cudaMallocHost((void **)&c->h_ses, sizeof(vtx_ctx::SesHost)) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFreeHost(c->h_status);
+    delete c;
+    return VTX_ERR_OOM;
+  }
   cudaEventCreateWithFlags(&c->counts_done, cudaEventDisableTiming);
   *out = c;
   return VTX_OK;
@@ -451,6 +463,7 @@ vtx_status vtx_destroy(vtx_ctx *c) {
   for (Buf *b : bufs)
     if (b->p) cudaFree(b->p);
   if (c->h_status) cudaFreeHost(c->h_status);
+  if (c->h_ses) cudaFreeHost(c->h_ses);
   if (c->h_counts) cudaFreeHost(c->h_counts);
   if (c->counts_done) cudaEventDestroy(c->counts_done);
   for (cudaEvent_t *set : c->ev_sets) {
@@ -1194,25 +1207,19 @@ vtx_status vtx_ses_fit_grid(vtx_ctx *c, const float *xyzr, int64_t n_atoms, floa
   const void *dx = nullptr;
   if (!device_visible(c, xyzr, &dx, "ses: xyzr not device or page-locked host memory")) return VTX_ERR_INVALID_ARG;
   if (((uintptr_t)dx & 15u) != 0) return fail(c, VTX_ERR_INVALID_ARG, "ses: xyzr must be 16-byte aligned");
-  const int nb = 4 * sm_count();
-  vtx_status st = ensure(c, c->ses_bbox, sizeof(float) * 6 * (size_t)nb, "ses bbox");
+  vtx_status st = ensure(c, c->ses_bbox, ses_bbox_bytes(), "ses bbox");
   if (st) return st;
-  cudaError_t e = run_ses_bbox((const float4 *)dx, n_atoms, probe, (float *)c->ses_bbox.p, nb, c->stream);
-  std::vector<float> part((size_t)nb * 6);
+  float *box = c->h_ses->box;  // lower corner, upper corner
+  cudaError_t e = run_ses_bbox((const float4 *)dx, n_atoms, probe, (float *)c->ses_bbox.p, c->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(part.data(), c->ses_bbox.p, sizeof(float) * part.size(), cudaMemcpyDeviceToHost, c->stream);
+    e = cudaMemcpyAsync(box, c->ses_bbox.p, sizeof(float) * 6, cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "ses bbox");
-  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (int b = 0; b < nb; ++b)
-    for (int d = 0; d < 3; ++d) {
-      lo[d] = std::fmin(lo[d], part[(size_t)b * 6 + d]);
-      hi[d] = std::fmax(hi[d], part[(size_t)b * 6 + 3 + d]);
-    }
   for (int d = 0; d < 3; ++d) {
-    if (!std::isfinite(lo[d]) || !std::isfinite(hi[d])) return fail(c, VTX_ERR_INVALID_ARG, "ses: non-finite atoms");
-    g->origin[d] = (float)((double)lo[d] - 2.0 * (double)spacing);
-    const double n = std::floor(((double)hi[d] - (double)lo[d]) / (double)spacing) + 6.0;
+    const float lo = box[d], hi = box[3 + d];
+    if (!std::isfinite(lo) || !std::isfinite(hi)) return fail(c, VTX_ERR_INVALID_ARG, "ses: non-finite atoms");
+    g->origin[d] = (float)((double)lo - 2.0 * (double)spacing);
+    const double n = std::floor(((double)hi - (double)lo) / (double)spacing) + 6.0;
     if (n > 2147483647.0) return fail(c, VTX_ERR_INVALID_ARG, "ses: grid too large");
     g->dims[d] = (int32_t)n;
   }
@@ -1221,11 +1228,11 @@ vtx_status vtx_ses_fit_grid(vtx_ctx *c, const float *xyzr, int64_t n_atoms, floa
   return VTX_OK;
 }
 
-vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *g, float *tris,
-                        int64_t max_tris, int64_t *labels, uint8_t *sas, uint16_t *edt2, int64_t *n_tris) {
-  if (!c) return VTX_ERR_INVALID_ARG;
-  if (!g || !n_tris || max_tris < 0 || (max_tris > 0 && !tris) || n_atoms < 0 || (n_atoms > 0 && !xyzr))
-    return fail(c, VTX_ERR_INVALID_ARG, "ses: bad arguments");
+// Checks a surface call's atoms, grid and planes, sizes the scratch and fills in the launch: everything but the
+// triangle buffers.  keep_edt: the distances stay in the context's scratch for a later emit, whatever edt2 is.
+static vtx_status ses_launch(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *g, uint8_t *sas,
+                             uint16_t *edt2, bool keep_edt, SesLaunch &L) {
+  c->ses_counted = false;
   if (!(g->spacing > 0.0f) || !(g->probe >= 0.0f) || !std::isfinite(g->spacing) || !std::isfinite(g->probe) ||
       (double)g->probe / (double)g->spacing > 150.0)
     return fail(c, VTX_ERR_INVALID_ARG, "ses: spacing > 0, probe >= 0 and probe / spacing <= 150 required");
@@ -1234,16 +1241,14 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
   const long long n_pts = (long long)g->dims[0] * g->dims[1] * g->dims[2];
   if (n_pts > 4294967296LL) return fail(c, VTX_ERR_INVALID_ARG, "ses: more than 2^32 grid points");
   cudaSetDevice(c->device);
-  const void *dx = nullptr, *dt = nullptr, *dl = nullptr, *ds = nullptr, *de = nullptr;
+  const void *dx = nullptr, *ds = nullptr, *de = nullptr;
   if (!device_visible(c, xyzr, &dx, "ses: xyzr not device or page-locked host memory") ||
-      !device_visible(c, tris, &dt, "ses: tris not device or page-locked host memory") ||
-      !device_visible(c, labels, &dl, "ses: labels not device or page-locked host memory") ||
       !device_visible(c, sas, &ds, "ses: sas not device or page-locked host memory") ||
       !device_visible(c, edt2, &de, "ses: edt2 not device or page-locked host memory"))
     return VTX_ERR_INVALID_ARG;
   if (((uintptr_t)dx & 15u) != 0) return fail(c, VTX_ERR_INVALID_ARG, "ses: xyzr must be 16-byte aligned");
-  if (((uintptr_t)dt & 3u) != 0 || ((uintptr_t)dl & 7u) != 0 || ((uintptr_t)de & 1u) != 0)
-    return fail(c, VTX_ERR_INVALID_ARG, "ses: misaligned output");
+  if (((uintptr_t)de & 1u) != 0) return fail(c, VTX_ERR_INVALID_ARG, "ses: misaligned output");
+  const bool own_edt = keep_edt || !de;
   const long long nb = ses_blocks(g->dims);
   vtx_status st;
   if ((st = ensure(c, c->ses_bits, 4 * (size_t)(ses_words(g->dims) + 1), "ses interior"))) return st;
@@ -1252,11 +1257,10 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
     if ((st = ensure(c, c->ses_a, 2 * (size_t)n_pts, "ses pass a"))) return st;
     if ((st = ensure(c, c->ses_b, 2 * (size_t)n_pts, "ses pass b"))) return st;
   }
-  if (!de && (st = ensure(c, c->ses_edt, 2 * (size_t)n_pts, "ses edt"))) return st;
+  if (own_edt && (st = ensure(c, c->ses_edt, 2 * (size_t)n_pts, "ses edt"))) return st;
   if ((st = ensure(c, c->ses_blk, sizeof(unsigned) * (size_t)(nb + 1), "ses blocks"))) return st;
   if ((st = ensure(c, c->ses_base, sizeof(unsigned long long) * (size_t)(nb + 1), "ses bases"))) return st;
   if ((st = ensure(c, c->ses_total, sizeof(unsigned long long), "ses total"))) return st;
-  SesLaunch L;
   L.X = (const float4 *)dx;
   L.n_atoms = n_atoms;
   for (int d = 0; d < 3; ++d) {
@@ -1270,21 +1274,92 @@ vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vt
   L.sas = (uint8_t *)ds;
   L.g_a = (uint16_t *)c->ses_a.p;
   L.g_b = (uint16_t *)c->ses_b.p;
-  L.edt2 = de ? (uint16_t *)de : (uint16_t *)c->ses_edt.p;
+  L.edt2 = own_edt ? (uint16_t *)c->ses_edt.p : (uint16_t *)de;
+  L.edt2_copy = own_edt ? (uint16_t *)de : nullptr;
   L.block_tris = (unsigned *)c->ses_blk.p;
   L.block_base = (unsigned long long *)c->ses_base.p;
   L.total = (unsigned long long *)c->ses_total.p;
+  L.tris = nullptr;
+  L.labels = nullptr;
+  L.max_tris = 0;
+  return VTX_OK;
+}
+
+// Device-visible triangle buffers of a surface call.
+static vtx_status ses_buffers(vtx_ctx *c, float *tris, int64_t max_tris, int64_t *labels, SesLaunch &L) {
+  const void *dt = nullptr, *dl = nullptr;
+  if (!device_visible(c, tris, &dt, "ses: tris not device or page-locked host memory") ||
+      !device_visible(c, labels, &dl, "ses: labels not device or page-locked host memory"))
+    return VTX_ERR_INVALID_ARG;
+  if (((uintptr_t)dt & 3u) != 0 || ((uintptr_t)dl & 7u) != 0)
+    return fail(c, VTX_ERR_INVALID_ARG, "ses: misaligned output");
   L.tris = (float *)dt;
   L.labels = (long long *)dl;
   L.max_tris = max_tris;
-  cudaError_t e = run_ses_grid(L, c->stream);
-  unsigned long long total = 0;
+  return VTX_OK;
+}
+
+// Reads the triangle count back (synchronises).
+static vtx_status ses_total(vtx_ctx *c, cudaError_t e, const SesLaunch &L, int64_t *n_tris) {
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&total, L.total, sizeof(total), cudaMemcpyDeviceToHost, c->stream);
+    e = cudaMemcpyAsync(&c->h_ses->total, L.total, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "ses mesh");
-  *n_tris = (int64_t)total;
-  if ((long long)total > max_tris) return fail(c, VTX_ERR_CAPACITY, "ses: more triangles than max_tris");
+  *n_tris = (int64_t)c->h_ses->total;
+  return VTX_OK;
+}
+
+vtx_status vtx_ses_mesh(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *g, float *tris,
+                        int64_t max_tris, int64_t *labels, uint8_t *sas, uint16_t *edt2, int64_t *n_tris) {
+  if (!c) return VTX_ERR_INVALID_ARG;
+  if (!g || !n_tris || max_tris < 0 || (max_tris > 0 && !tris) || n_atoms < 0 || (n_atoms > 0 && !xyzr))
+    return fail(c, VTX_ERR_INVALID_ARG, "ses: bad arguments");
+  SesLaunch L;
+  vtx_status st = ses_launch(c, xyzr, n_atoms, g, sas, edt2, false, L);
+  if (st) return st;
+  if ((st = ses_buffers(c, tris, max_tris, labels, L))) return st;
+  cudaError_t e = run_ses_count(L, c->stream);
+  if (e == cudaSuccess) e = run_ses_emit(L, c->stream);
+  if ((st = ses_total(c, e, L, n_tris))) return st;
+  if (*n_tris > max_tris) return fail(c, VTX_ERR_CAPACITY, "ses: more triangles than max_tris");
+  return VTX_OK;
+}
+
+vtx_status vtx_ses_count(vtx_ctx *c, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *g, uint8_t *sas,
+                         uint16_t *edt2, int64_t *n_tris) {
+  if (!c) return VTX_ERR_INVALID_ARG;
+  if (!g || !n_tris || n_atoms < 0 || (n_atoms > 0 && !xyzr))
+    return fail(c, VTX_ERR_INVALID_ARG, "ses: bad arguments");
+  SesLaunch L;
+  vtx_status st = ses_launch(c, xyzr, n_atoms, g, sas, edt2, true, L);
+  if (st) return st;
+  if ((st = ses_total(c, run_ses_count(L, c->stream), L, n_tris))) return st;
+  c->ses_grid = *g;
+  c->ses_counted = true;
+  return VTX_OK;
+}
+
+vtx_status vtx_ses_emit(vtx_ctx *c, float *tris, int64_t max_tris, int64_t *labels) {
+  if (!c) return VTX_ERR_INVALID_ARG;
+  if (max_tris < 0 || (max_tris > 0 && !tris)) return fail(c, VTX_ERR_INVALID_ARG, "ses: bad arguments");
+  if (!c->ses_counted) return fail(c, VTX_ERR_STATE, "ses: no surface counted since the last surface call");
+  cudaSetDevice(c->device);
+  SesLaunch L{};
+  vtx_status st = ses_buffers(c, tris, max_tris, labels, L);
+  if (st) return st;
+  for (int d = 0; d < 3; ++d) {
+    L.origin[d] = c->ses_grid.origin[d];
+    L.dims[d] = c->ses_grid.dims[d];
+  }
+  L.h = c->ses_grid.spacing;
+  L.probe = c->ses_grid.probe;
+  L.inside = (uint32_t *)c->ses_in.p;
+  L.edt2 = (uint16_t *)c->ses_edt.p;
+  L.block_base = (unsigned long long *)c->ses_base.p;
+  L.total = (unsigned long long *)c->ses_total.p;
+  int64_t n = 0;
+  if ((st = ses_total(c, run_ses_emit(L, c->stream), L, &n))) return st;
+  if (n > max_tris) return fail(c, VTX_ERR_CAPACITY, "ses: more triangles than max_tris");
   return VTX_OK;
 }
 

@@ -754,19 +754,12 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
   }
 }
 
-// Bounding box of the SAS spheres: min and max of c -/+ (r + p), as float bits of
-// non-negative-shifted values would be awkward, so each CTA reduces and writes one
-// partial; the host finishes the (small) reduction.
-__global__ __launch_bounds__(256) void k_ses_bbox(const float4 *__restrict__ X, long long n, float p,
-                                                  float *__restrict__ partial) {
-  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (long long)gridDim.x * blockDim.x) {
-    const float4 c = X[a];
-    const float R = c.w + p;
-    lo[0] = fminf(lo[0], c.x - R), hi[0] = fmaxf(hi[0], c.x + R);
-    lo[1] = fminf(lo[1], c.y - R), hi[1] = fmaxf(hi[1], c.y + R);
-    lo[2] = fminf(lo[2], c.z - R), hi[2] = fmaxf(hi[2], c.z + R);
-  }
+// Bounding box of the SAS spheres: min and max of c -/+ (r + p).  Each CTA leaves its bounds, and the last one to
+// finish reduces them into box[0..5]: one launch and 24 bytes for the host.  *done counts finished CTAs (zero at
+// launch).
+constexpr int kSesBoxCtas = 512;
+
+__device__ __forceinline__ void ses_box_reduce(float (&lo)[3], float (&hi)[3], float *out) {
   __shared__ float s[6][8];
   for (int d = 0; d < 3; ++d) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -784,8 +777,39 @@ __global__ __launch_bounds__(256) void k_ses_bbox(const float4 *__restrict__ X, 
   if (threadIdx.x < 6) {
     float v = s[threadIdx.x][0];
     for (int q = 1; q < 8; ++q) v = threadIdx.x < 3 ? fminf(v, s[threadIdx.x][q]) : fmaxf(v, s[threadIdx.x][q]);
-    partial[blockIdx.x * 6 + threadIdx.x] = v;
+    out[threadIdx.x] = v;
   }
+  __syncthreads();
+}
+
+__global__ __launch_bounds__(256) void k_ses_bbox(const float4 *__restrict__ X, long long n, float p, float *box,
+                                                  float *partial, unsigned *done) {
+  __shared__ bool s_last;
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < n; a += (long long)gridDim.x * blockDim.x) {
+    const float4 c = X[a];
+    const float R = c.w + p;
+    lo[0] = fminf(lo[0], c.x - R), hi[0] = fmaxf(hi[0], c.x + R);
+    lo[1] = fminf(lo[1], c.y - R), hi[1] = fmaxf(hi[1], c.y + R);
+    lo[2] = fminf(lo[2], c.z - R), hi[2] = fmaxf(hi[2], c.z + R);
+  }
+  ses_box_reduce(lo, hi, partial + 6 * blockIdx.x);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int d = 0; d < 3; ++d) {
+    lo[d] = INFINITY;
+    hi[d] = -INFINITY;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+      lo[d] = fminf(lo[d], __ldcg(partial + 6 * b + d));
+      hi[d] = fmaxf(hi[d], __ldcg(partial + 6 * b + 3 + d));
+    }
+  }
+  ses_box_reduce(lo, hi, box);
 }
 
 // ------------------------------------------------------------- launchers --
@@ -808,15 +832,19 @@ static void launch_levels(const SesGrid &G, const SesLaunch &L, cudaStream_t st)
   k_ses_levels<K><<<(unsigned)tiles, 256, 0, st>>>(G, L.bits, L.edt2, L.inside);
 }
 
-cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *partial, int n_blocks, cudaStream_t st) {
-  k_ses_bbox<<<n_blocks, 256, 0, st>>>(X, n, probe, partial);
+size_t ses_bbox_bytes() { return sizeof(float) * (8 + 6 * (size_t)kSesBoxCtas); }
+
+cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *box, cudaStream_t st) {
+  // box: six bounds, the counter, one unused word, then the CTAs' bounds
+  unsigned *done = reinterpret_cast<unsigned *>(box + 6);
+  cudaError_t e = cudaMemsetAsync(done, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  const long long want = (n + 255) / 256;
+  k_ses_bbox<<<(int)(want < kSesBoxCtas ? want : kSesBoxCtas), 256, 0, st>>>(X, n, probe, box, box + 8, done);
   return cudaGetLastError();
 }
 
-cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (!ses_table_ready(dev)) return cudaErrorInvalidValue;
+static SesGrid make_grid(const SesLaunch &L) {
   SesGrid G{L.origin[0], L.origin[1], L.origin[2], L.h, L.probe, L.dims[0], L.dims[1], L.dims[2],
             (int)(((long long)L.dims[0] + 31) / 32), ses_window(L.probe, L.h), 1, 0.0f};
   {
@@ -835,6 +863,14 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
     }
     G.xmax = (float)(xm * 1.001 + 1.0);
   }
+  return G;
+}
+
+cudaError_t run_ses_count(const SesLaunch &L, cudaStream_t st) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!ses_table_ready(dev)) return cudaErrorInvalidValue;
+  const SesGrid G = make_grid(L);
   const long long n_pts = (long long)G.nx * G.ny * G.nz;
   const int sms = sm_count();
   cudaError_t e = cudaMemsetAsync(L.bits, 0, 4 * (size_t)(ses_words(L.dims) + 1), st);  // and the counter after them
@@ -867,15 +903,22 @@ cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st) {
     const long long wb = (n_words + 7) / 8;
     k_ses_inside<<<(int)(wb < 16LL * sms ? wb : 16LL * sms), 256, 0, st>>>(G, L.edt2, n_words, L.inside);
   }
+  if (L.edt2_copy) {
+    e = cudaMemcpyAsync(L.edt2_copy, L.edt2, 2 * (size_t)n_pts, cudaMemcpyDefault, st);
+    if (e != cudaSuccess) return e;
+  }
   const long long n_blocks = ses_blocks(L.dims);
   unsigned *done = reinterpret_cast<unsigned *>(L.bits + ses_words(L.dims));  // cleared with the bits
   k_ses_count<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.inside, (uint32_t)ses_groups(L.dims), L.block_tris,
                                                           L.block_base, L.total, done);
-  if (L.max_tris > 0) {
-    k_ses_emit<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(
-        G, L.edt2, L.inside, (uint32_t)ses_groups(L.dims), L.block_base, L.tris, L.labels,
-        (unsigned long long)L.max_tris);
-  }
+  return cudaGetLastError();
+}
+
+cudaError_t run_ses_emit(const SesLaunch &L, cudaStream_t st) {
+  if (L.max_tris == 0) return cudaSuccess;
+  k_ses_emit<<<(unsigned)ses_blocks(L.dims), kSesThreads, 0, st>>>(
+      make_grid(L), L.edt2, L.inside, (uint32_t)ses_groups(L.dims), L.block_base, L.tris, L.labels,
+      (unsigned long long)L.max_tris);
   return cudaGetLastError();
 }
 

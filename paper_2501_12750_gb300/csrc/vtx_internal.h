@@ -95,6 +95,7 @@ struct SesLaunch {
   uint8_t *sas;                   // [nz][ny][nx] SAS interior as bytes (0/1), or null
   uint16_t *g_a, *g_b;            // scratch of the three distance passes (ses_three_pass), one value per grid point
   uint16_t *edt2;                 // [nz][ny][nx] windowed squared distance (grid units)
+  uint16_t *edt2_copy;            // another place that it goes to, or null
   unsigned *block_tris;           // [ses_blocks(dims)]
   unsigned long long *block_base; // [ses_blocks(dims)]
   unsigned long long *total;      // [1]
@@ -102,8 +103,13 @@ struct SesLaunch {
   long long *labels;              // [max_tris][3] or null
   long long max_tris;
 };
-cudaError_t run_ses_grid(const SesLaunch &L, cudaStream_t st);
-cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *partial, int n_blocks, cudaStream_t st);
+// Interior, distances and triangle counts; then the triangles (nothing when max_tris is 0), which read inside, edt2
+// and block_base only.
+cudaError_t run_ses_count(const SesLaunch &L, cudaStream_t st);
+cudaError_t run_ses_emit(const SesLaunch &L, cudaStream_t st);
+// Bounds of the SAS spheres into box[0..5] (lower corner, upper corner), the first of ses_bbox_bytes() of scratch.
+cudaError_t run_ses_bbox(const float4 *X, long long n, float probe, float *box, cudaStream_t st);
+size_t ses_bbox_bytes();
 long long ses_blocks(const int32_t dims[3]);
 int ses_window(float probe, float h);
 bool ses_three_pass(float probe, float h);  // the window is too large for the bit-set distance pass

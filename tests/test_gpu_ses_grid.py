@@ -27,3 +27,33 @@ def test_ses_window_sizes_at_tile_edges(dims, K):
     origin = np.array([0.0, 0.013, -0.007], np.float32)
     d = np.array(dims, np.int32)
     check_same(gpu_ses(x, origin, h, d, probe), oracle.ses(x, origin, h, d, probe=probe), "K=%d %s" % (K, dims))
+
+
+def test_ses_count_then_emit():
+    """The two-call form: no surface before the first count or after a plain call; partial and repeated writes; the
+    distances also go to the caller's plane."""
+    import ctypes
+
+    import torch
+
+    import paper_2501_12750_gb300 as vtx
+    rng = np.random.default_rng(3)
+    x = torch.from_numpy(np.concatenate([rng.uniform(0, 8, (30, 3)), rng.uniform(1, 2, (30, 1))], 1)
+                         .astype(np.float32)).cuda()
+    r = vtx.Renderer()
+    g = r.ses_fit_grid(x, probe=1.4, spacing=0.5)
+    ref = r.ses_mesh(x, g, max_tris=20000, labels=True, planes=True)
+    n = ctypes.c_int64(0)
+    buf = torch.zeros((ref["n"], 3, 3), device="cuda")
+    assert r.lib.vtx_ses_emit(r.ctx, buf.data_ptr(), ref["n"], None) == 7  # VTX_ERR_STATE
+    edt = torch.empty_like(ref["edt2"])
+    assert r.lib.vtx_ses_count(r.ctx, x.data_ptr(), 30, ctypes.byref(g), None, edt.data_ptr(), ctypes.byref(n)) == 0
+    assert n.value == ref["n"] and torch.equal(edt, ref["edt2"])
+    edt.zero_()  # the caller's plane is its own again
+    part = torch.zeros((100, 3, 3), device="cuda")
+    assert r.lib.vtx_ses_emit(r.ctx, part.data_ptr(), 100, None) == 4  # VTX_ERR_CAPACITY
+    assert torch.equal(part, ref["tris"][:100])
+    assert r.lib.vtx_ses_emit(r.ctx, buf.data_ptr(), n.value, None) == 0
+    assert torch.equal(buf, ref["tris"])
+    full = r.ses_mesh(x, g, labels=True)
+    assert torch.equal(full["tris"], ref["tris"]) and torch.equal(full["labels"], ref["labels"])
