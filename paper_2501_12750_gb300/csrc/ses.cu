@@ -165,37 +165,61 @@ __device__ __forceinline__ double grid_coord(float o, float h, long long i) {
   return __dadd_rn((double)o, __dmul_rn((double)h, (double)i));
 }
 
-__device__ __forceinline__ bool sas_exact(const SesGrid &G, long long i, double dy2, double dz2, double cx, double R2) {
-  const double dx = __dsub_rn(grid_coord(G.ox, G.h, i), cx);
+__device__ __forceinline__ bool sas_exact(float ox, float h, long long i, double dy2, double dz2, double cx, double R2) {
+  const double dx = __dsub_rn(grid_coord(ox, h, i), cx);
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), dy2), dz2) < R2;
+}
+
+// The points of one row that FP32 cannot decide, [i0, i1] but for the certain ones [a, b], by the exact FP64 test.
+static __device__ __noinline__ void sas_row_exact(float ox, float oy, float oz, float h, float p, float4 c, int j, int k,
+                                                  int i0, int i1, int a, int b, uint32_t *row) {
+  const double dy = __dsub_rn(grid_coord(oy, h, j), (double)c.y);
+  const double dz = __dsub_rn(grid_coord(oz, h, k), (double)c.z);
+  const double dy2 = __dmul_rn(dy, dy), dz2 = __dmul_rn(dz, dz);
+  const double R = __dadd_rn((double)c.w, (double)p);
+  const double R2 = __dmul_rn(R, R);
+  for (int i = i0; i <= i1; ++i) {
+    if (i >= a && i <= b) {
+      i = b;
+      continue;
+    }
+    if (sas_exact(ox, h, i, dy2, dz2, (double)c.x, R2)) atomicOr(row + (i >> 5), 1u << (i & 31));
+  }
 }
 
 // SAS interior, one bit per grid point (bit i & 31 of word i >> 5 of a row; wx words a row): one warp per atom
 // (`parts` warps when there are few atoms), lanes over the (j, k) rows of its box.  A row meets the sphere in a
 // chord: with t = R^2 - dy^2 - dz^2 in FP32 and M the bound on the FP32 error of d^2 (coordinates, differences
 // and squares, all at most a few ulps of numbers <= xmax + R + 2h, and of R^2 itself), every point with
-// |dx| <= sqrt(t - M) is inside and none with |dx| > sqrt(t + M) is; the index bounds of both are widened by the
-// rounding of the index itself.  The points between the two (a few in a thousand rows have one) are decided by
-// the exact FP64 test, so every decision equals the FP64 one.  The chord's bits are set with one atomic a word.
+// |dx| <= sqrt(t - M) is inside and none with |dx| > sqrt(t + M) is.  Both lie within M / sqrt(t) of sqrt(t) (t > M),
+// so the chord's ends, as grid indices, are known to within u = (M / sqrt(t) + 2 delta) / h plus the rounding eps of
+// the index arithmetic itself; the points within u of an end (a few in a thousand rows have one), and every point of
+// a row with t <= 4 M, are decided by the exact FP64 test, so every decision equals the FP64 one.  Both
+// bounds are kept near the roundings they stand for: an exact test costs its warp some 300 cycles of the FP64 pipe
+// (four times wider bounds took 262 us instead of 102).  The chord's bits are set with one atomic a word.
 //
 // Bound by the row loop's issue and its atomics, not by memory: the bits of 3.4e7 points are 4.6 MB and stay in
-// L2.  1e5 atoms at 0.5 A (3.4e7 points): 179 us; 1302 us with a byte per point, each point classified on its own.
-__global__ __launch_bounds__(256) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n, int parts,
-                                                 uint32_t *__restrict__ bits) {
+// L2.  1e5 atoms at 0.5 A (3.4e7 points): 102 us; 179 us with both ends of both bounds computed per row over a box
+// two points wider on each side; 1302 us with a byte per point, each point classified on its own.
+__global__ __launch_bounds__(256, 6) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n, int parts,
+                                                    uint32_t *__restrict__ bits) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const float inv_h = 1.0f / G.h;
+  const long long plane = (long long)G.ny * G.wx;
   for (long long item = warp; item < n * parts; item += n_warps) {
     const float4 c = X[item / parts];
     // FP32 throughout except on the rare points the filter cannot decide (the
     // FP64 pipes are a small fraction of the FP32 ones on this part)
     const float Rf = c.w + G.p, R2f = Rf * Rf;
-    const float span = G.xmax + Rf + 2.0f * G.h;
-    const float delta = 4e-7f * span;                      // |FP32 difference - exact| per axis
+    // error of an FP32 difference X - c along y or z: the roundings of the grid index and coordinate and of the
+    // difference, at most three times 2^-24 of the largest number; M: of dy^2 + dz^2 (2 |d| delta an axis, with
+    // |dy| + |dz| <= sqrt(2) ext) and the relative roundings of the squares, of R, R^2 and of t
     const float ext = fabsf(Rf) + 2.0f * G.h;
-    const float M = 8.0f * ext * delta + 4.0f * delta * delta + 1e-6f * ext * ext + 1e-6f;
+    const float delta = 2e-7f * (G.xmax + ext);
+    float M = 2.9f * ext * delta + 4.0f * delta * delta + 6e-7f * ext * ext;
     // candidate index ranges, two points wider than the sphere's extent on each side
-    const float inv_h = 1.0f / G.h;
     const float cf[3] = {c.x, c.y, c.z};
     const float of[3] = {G.ox, G.oy, G.oz};
     const int nn[3] = {G.nx, G.ny, G.nz};
@@ -206,64 +230,62 @@ __global__ __launch_bounds__(256) void k_ses_sas(SesGrid G, const float4 *__rest
       const float top = (float)nn[d];
       lo[d] = max((int)fminf(fmaxf(floorf((cf[d] - Rf - of[d]) * inv_h) - 2.0f, 0.0f), top), 0);
       hi[d] = min((int)fminf(fmaxf(ceilf((cf[d] + Rf - of[d]) * inv_h) + 2.0f, -1.0f), top), nn[d] - 1);
+      if (d > 0) {
+        // rows farther than sqrt(R^2 + M) from the centre are outside as a whole: the box without them
+        const float w = sqrtf(R2f + M) * 1.000001f + 2.0f * delta;
+        const float e = 1e-5f + 2e-6f * (fabsf(cf[d]) + fabsf(of[d]) + w) * inv_h;
+        lo[d] = max(lo[d], (int)fminf(fmaxf(ceilf((cf[d] - w - of[d]) * inv_h - e), 0.0f), top));
+        hi[d] = min(hi[d], (int)fminf(fmaxf(floorf((cf[d] + w - of[d]) * inv_h + e), -1.0f), top));
+      }
     }
     if (lo[0] > hi[0] || lo[1] > hi[1] || lo[2] > hi[2]) continue;
-    // rounding of a chord end's grid index: FP32 sums and products of numbers <= |c| + |o| + R
-    const float eps = 1e-5f + 2e-6f * (fabsf(c.x) + fabsf(G.ox) + fabsf(Rf)) * inv_h;
+    // the centre's grid index, and the rounding of a chord end's index: of the difference, of 1 / h and the product,
+    // and of the end's sum, each 2^-24 of numbers <= (|c - o| + R) / h
+    const float xc = (c.x - G.ox) * inv_h;
+    const float eps = 1e-6f + 4e-7f * (fabsf(xc) + fabsf(Rf) * inv_h);
+    if (!(fabsf(xc) < 1e30f)) M = INFINITY;  // no usable index (1 / h overflows): the exact test decides
+    const float Mh = M * inv_h * 1.001f;
     // row r of the box is (lo[1] + r % ny_box, lo[2] + r / ny_box); this lane takes every (32 parts)-th
     const unsigned ny_box = (unsigned)(hi[1] - lo[1] + 1), step = 32u * (unsigned)parts;
     const unsigned r0 = 32u * (unsigned)(item % parts) + (unsigned)lane;
     const int step_j = (int)(step % ny_box), step_k = (int)(step / ny_box);
     int j = lo[1] + (int)(r0 % ny_box), k = lo[2] + (int)(r0 / ny_box);
+    uint32_t *row = bits + (long long)k * plane + (long long)j * G.wx;
+    const long long step_row = (long long)step_k * plane + (long long)step_j * G.wx;
+    const long long wrap_row = plane - (long long)ny_box * G.wx;
     for (; k <= hi[2]; k += step_k) {
       const float dyf = __fsub_rn(__fmaf_rn(G.h, (float)j, G.oy), c.y);
       const float dzf = __fsub_rn(__fmaf_rn(G.h, (float)k, G.oz), c.z);
       const float yz = __fmaf_rn(dyf, dyf, __fmul_rn(dzf, dzf));
       const float t = R2f - yz;
-      if (!(t < -M)) {  // else the whole row is outside
-        const float w_out = sqrtf(fmaxf(t + M, 0.0f)) * 1.000001f + 2.0f * delta;
-        const float w_in = t > M ? sqrt_approx(t - M) * 0.999999f - 2.0f * delta : -1.0f;
-        const float top = (float)(hi[0] + 1);
-        const int i0 = max((int)fminf(fmaxf(ceilf((c.x - w_out - G.ox) * inv_h - eps), 0.0f), top), lo[0]);
-        const int i1 = min((int)fminf(fmaxf(floorf((c.x + w_out - G.ox) * inv_h + eps), -1.0f), top), hi[0]);
-        int a = i1 + 1, b = i1;  // the certain points [a, b] (none yet)
-        if (w_in >= 0.0f) {
-          const int ca = (int)fminf(fmaxf(ceilf((c.x - w_in - G.ox) * inv_h + eps), 0.0f), top);
-          const int cb = (int)fminf(fmaxf(floorf((c.x + w_in - G.ox) * inv_h - eps), -1.0f), top);
-          if (max(ca, i0) <= min(cb, i1)) {
-            a = max(ca, i0);
-            b = min(cb, i1);
-          }
-        }
-        uint32_t *row = bits + ((size_t)k * (size_t)G.ny + (size_t)j) * (size_t)G.wx;
+      if (t > 4.0f * M) {
+        const float rs = rsqrtf(t);
+        const float w = t * rs * inv_h, u = fmaf(Mh, rs, eps + 1e-6f * w);
+        const int i0 = max(__float2int_ru(xc - w - u), lo[0]), a = max(__float2int_ru(xc - w + u), lo[0]);
+        const int i1 = min(__float2int_rd(xc + w + u), hi[0]), b = min(__float2int_rd(xc + w - u), hi[0]);
         if (a <= b) {
           const int wa = a >> 5, wb = b >> 5;
-          for (int w = wa; w <= wb; ++w) {
-            uint32_t m = 0xffffffffu;
-            if (w == wa) m <<= a & 31;
-            if (w == wb) m &= 0xffffffffu >> (31 - (b & 31));
-            atomicOr(row + w, m);
+          const uint32_t ma = 0xffffffffu << (a & 31), mb = 0xffffffffu >> (31 - (b & 31));
+          if (wa == wb) {
+            atomicOr(row + wa, ma & mb);
+          } else {
+            atomicOr(row + wa, ma);
+            for (int q = wa + 1; q < wb; ++q) atomicOr(row + q, 0xffffffffu);
+            atomicOr(row + wb, mb);
           }
         }
-        if (a > i0 || b < i1) {
-          const double dy = __dsub_rn(grid_coord(G.oy, G.h, j), (double)c.y);
-          const double dz = __dsub_rn(grid_coord(G.oz, G.h, k), (double)c.z);
-          const double dy2 = __dmul_rn(dy, dy), dz2 = __dmul_rn(dz, dz);
-          const double R = __dadd_rn((double)c.w, (double)G.p);
-          const double R2 = __dmul_rn(R, R);
-          for (int i = i0; i <= i1; ++i) {
-            if (i == a) {  // past the certain points
-              i = b;
-              continue;
-            }
-            if (sas_exact(G, i, dy2, dz2, (double)c.x, R2)) atomicOr(row + (i >> 5), 1u << (i & 31));
-          }
-        }
+        if (a != i0 || b != i1) sas_row_exact(G.ox, G.oy, G.oz, G.h, G.p, c, j, k, i0, i1, a, b, row);
+      } else if (!(t < -M)) {  // else the whole row is outside
+        const float w = sqrtf(fmaxf(t + M, 0.0f)) * 1.000001f * inv_h;
+        const int i0 = max(__float2int_ru(xc - w - eps), lo[0]), i1 = min(__float2int_rd(xc + w + eps), hi[0]);
+        sas_row_exact(G.ox, G.oy, G.oz, G.h, G.p, c, j, k, i0, i1, 1, 0, row);
       }
       j += step_j;
+      row += step_row;
       if (j > hi[1]) {
         j -= (int)ny_box;
         ++k;
+        row += wrap_row;
       }
     }
   }
@@ -347,6 +369,18 @@ __device__ __forceinline__ void ses_steps(const uint32_t *e, int t_in, SesLevelS
   (ses_step<K, I>(e, t_in, s), ...);
 }
 
+// Transpose of a 32 x 32 bit matrix, row l in lane l: lane l receives bit l of every row (blocks of 16, 8, 4, 2, 1
+// columns exchanged between lanes that far apart).
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t v, int lane) {
+  uint32_t m = 0x0000ffffu;  // the columns whose index has bit s clear
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1, m ^= m << s) {
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, v, s);
+    v = (lane & s) ? ((v & ~m) | ((o >> s) & m)) : ((v & m) | ((o << s) & ~m));
+  }
+  return v;
+}
+
 // s_val[level] = its squared length (the last one: the sentinel).
 template <int K, int I>
 __device__ __forceinline__ void ses_value(uint16_t *s_val) {
@@ -405,18 +439,23 @@ __global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *_
 #pragma unroll
   for (int p = 0; p < 6; ++p)
     if ((n_levels >> p) & 1) st.plane[p] |= rest;
-  // spread: row r of the warp's 32 (y0 + r), one point per lane
+  // spread: one point per lane and row.  Each digit plane's 32 x 32 bits (row r in lane r) are transposed across
+  // the warp, so that lane x holds point x of every row; a row's level is then a bit of each plane.
   constexpr int planes = n_levels < 2 ? 1 : n_levels < 4 ? 2 : n_levels < 8 ? 3 : n_levels < 16 ? 4 : n_levels < 32 ? 5 : 6;
   const long long z = z0 + zw, x = 32LL * w + lane;
   if (z >= G.nz) return;  // uniform in the warp; no barrier follows
   const int rows = (int)min((long long)S::TY, G.ny - y0);
   if (lane < rows) inside[(z * G.ny + y0 + lane) * G.wx + w] = ~st.outside;
+#pragma unroll
+  for (int p = 0; p < planes; ++p) st.plane[p] = warp_transpose(st.plane[p], lane);
   uint16_t *dst = edt2 + (z * G.ny + y0) * G.nx + x;
+  const bool mine = x < G.nx;
+#pragma unroll 8
   for (int r = 0; r < rows; ++r, dst += G.nx) {
     unsigned lv = 0u;
 #pragma unroll
-    for (int p = 0; p < planes; ++p) lv |= ((__shfl_sync(0xffffffffu, st.plane[p], r) >> lane) & 1u) << p;
-    if (x < G.nx) *dst = s_val[lv];
+    for (int p = planes - 1; p >= 0; --p) lv = 2u * lv + ((st.plane[p] >> r) & 1u);
+    if (mine) *dst = s_val[lv];
   }
 }
 
@@ -609,30 +648,31 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_count(SesGrid G, const uint
   if (threadIdx.x == kSesThreads - 1) *total = s_sum[threadIdx.x];
 }
 
-// Position of the vertex at parameter t on edge e of cell (i, j, k): X_a + t (X_b - X_a).
-__device__ __forceinline__ float3 edge_point(const SesGrid &G, int i, int j, int k, int e, float t) {
-  // edges 0-3 and 4-7 go round the squares z = 0 and z = 1 from corner (0, 0) in +x, +y, -x, -y; 8-11 in +z
-  const int q = e & 3;
-  const int ax = (q == 1 || q == 2) ? 1 : 0, ay = q >> 1, az = (e >= 4 && e < 8) ? 1 : 0;
-  const int dz = e >= 8 ? 1 : 0;
-  const int dx = dz ? 0 : (q == 0) - (q == 2), dy = dz ? 0 : (q == 1) - (q == 3);
-  const float3 A = make_float3(fmaf(G.h, (float)(i + ax), G.ox), fmaf(G.h, (float)(j + ay), G.oy),
-                               fmaf(G.h, (float)(k + az), G.oz));
-  const float3 B = make_float3(fmaf(G.h, (float)(i + ax + dx), G.ox), fmaf(G.h, (float)(j + ay + dy), G.oy),
-                               fmaf(G.h, (float)(k + az + dz), G.oz));
-  return make_float3(fmaf(t, B.x - A.x, A.x), fmaf(t, B.y - A.y, A.y), fmaf(t, B.z - A.z, A.z));
-}
-
 // Shared memory of the emit pass, for 256 crossing cells at a time.
 struct SesEmitShared {
-  float t[12][kSesThreads];        // vertex parameter of every crossing edge of each cell
+  float at[12][kSesThreads];       // the vertex of every crossing edge of each cell: its coordinate along the edge
   float mean[12][kSesThreads];     // means of its loops: x, y, z of loop l at 3 l
+  float grid[6][kSesThreads];      // its lower and upper grid coordinates: x, y, z at 2 axis + upper
   float stage[kSesThreads / 32][32 * 9];  // per warp: 32 triangles on their way out
   int ci[kSesThreads], cj[kSesThreads], ck[kSesThreads];
   unsigned off[kSesThreads];       // first triangle of each cell
   unsigned char cs[kSesThreads];   // case
   unsigned char cell_of[kSesThreads * 12];  // cell of each triangle
 };
+static_assert(sizeof(SesEmitShared) <= 48 * 1024, "static shared memory");
+
+// Edges by direction (bit e): along x, y, z; and by the upper side of the cell that they lie on.  An edge runs from
+// its first corner to its second: along x 0, 2, 4, 6 (2 and 6 downward), along y 1, 3, 5, 7 (3 and 7 downward).
+constexpr unsigned kEdgeX = 0x055u, kEdgeY = 0x0aau, kEdgeZ = 0xf00u;
+constexpr unsigned kEdgeUpX = 0x622u, kEdgeUpY = 0xc44u, kEdgeUpZ = 0x0f0u;
+
+// The vertex on edge e of a cell.
+__device__ __forceinline__ float3 edge_point(const SesEmitShared &sh, int cell, int e) {
+  const float v = sh.at[e][cell];
+  const float x = sh.grid[(kEdgeUpX >> e) & 1u][cell], y = sh.grid[2 + ((kEdgeUpY >> e) & 1u)][cell];
+  const float z = sh.grid[4 + ((kEdgeUpZ >> e) & 1u)][cell];
+  return make_float3((kEdgeX >> e) & 1u ? v : x, (kEdgeY >> e) & 1u ? v : y, (kEdgeZ >> e) & 1u ? v : z);
+}
 
 // Triangles of the groups of CTA blockIdx.x, in cell order.  The groups' crossing cells are taken 256 at a time,
 // one per thread: the eight distances are read once and give the parameter of every crossing edge and the means
@@ -640,7 +680,8 @@ struct SesEmitShared {
 // triangles as one run of floats.
 //
 // Bound by issue (a crossing cell has about five vertices and two triangles) and the triangles' writes.  5.9e6
-// triangles (212 MB): 146 us; 789 us with one thread per triangle finding its cell by binary search over
+// triangles (212 MB): 123 us, with f read from a table of the window's distances and the vertices kept as one
+// coordinate along their edge; 146 us with a root per corner and positions worked out per triangle; 789 us with one thread per triangle finding its cell by binary search over
 // a case byte per cell, recomputing its loop's vertices from the distance plane and storing 36-byte strides.
 __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint16_t *__restrict__ edt,
                                                           const uint32_t *__restrict__ inside, uint32_t n_groups,
@@ -648,8 +689,11 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
                                                           float *__restrict__ tris, long long *__restrict__ labels,
                                                           unsigned long long max_tris) {
   __shared__ SesEmitShared sh;
+  __shared__ float s_f[kSesBitK * kSesBitK + 2];  // f of every distance that a bit-set window has
+  const bool table = G.K <= kSesBitK;
   unsigned long long base = block_base[blockIdx.x];
   if (base >= max_tris) return;
+  if (threadIdx.x <= kSesBitK * kSesBitK + 1) s_f[threadIdx.x] = fmaf(sqrtf((float)threadIdx.x), G.h, -G.p);
   const SesGroup s = ses_group(G, inside, blockIdx.x * (unsigned)kSesGroups + threadIdx.x, n_groups);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   unsigned n_cells;
@@ -675,25 +719,31 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
       n_tri = tc.n_tris;
       const uint16_t *q = edt + ((size_t)k * ny + (size_t)j) * nx + (size_t)i;
       const size_t up = ny * nx;
+      const int d[8] = {q[0], q[1], q[nx + 1], q[nx], q[up], q[up + 1], q[up + nx + 1], q[up + nx]};
       float f[8];
-      f[0] = (float)q[0];
-      f[1] = (float)q[1];
-      f[2] = (float)q[nx + 1];
-      f[3] = (float)q[nx];
-      f[4] = (float)q[up];
-      f[5] = (float)q[up + 1];
-      f[6] = (float)q[up + nx + 1];
-      f[7] = (float)q[up + nx];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) f[c] = fmaf(sqrtf(f[c]), G.h, -G.p);
+      for (int c = 0; c < 8; ++c) f[c] = table ? s_f[d[c]] : fmaf(sqrtf((float)d[c]), G.h, -G.p);
+      float g[6];
+      g[0] = fmaf(G.h, (float)i, G.ox);
+      g[1] = fmaf(G.h, (float)(i + 1), G.ox);
+      g[2] = fmaf(G.h, (float)j, G.oy);
+      g[3] = fmaf(G.h, (float)(j + 1), G.oy);
+      g[4] = fmaf(G.h, (float)k, G.oz);
+      g[5] = fmaf(G.h, (float)(k + 1), G.oz);
+#pragma unroll
+      for (int c = 0; c < 6; ++c) sh.grid[c][tid] = g[c];
       constexpr int ea[12] = {0, 1, 2, 3, 4, 5, 6, 7, 0, 1, 2, 3};
       constexpr int eb[12] = {1, 2, 3, 0, 5, 6, 7, 4, 4, 5, 6, 7};
 #pragma unroll
       for (int e = 0; e < 12; ++e) {
         if (((cs >> ea[e]) ^ (cs >> eb[e])) & 1u) {
+          // X_a + t (X_b - X_a) along the edge's axis, t = f_a / (f_a - f_b)
           const float fa = f[ea[e]], fb = f[eb[e]];
-          const float t = fa == fb ? 0.5f : fa / (fa - fb);
-          sh.t[e][tid] = fminf(fmaxf(t, 0.0f), 1.0f);
+          const float t = fminf(fmaxf(fa == fb ? 0.5f : fa / (fa - fb), 0.0f), 1.0f);
+          const int axis = e >= 8 ? 4 : ((e & 1) ? 2 : 0);
+          const bool down = e < 8 && (e & 2);
+          const float xa = down ? g[axis + 1] : g[axis], xb = down ? g[axis] : g[axis + 1];
+          sh.at[e][tid] = fmaf(t, xb - xa, xa);
         }
       }
       for (int l = 0, at = 0; l < tc.n_loops; at += tc.len[l], ++l) {
@@ -702,7 +752,7 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
         float3 M = make_float3(0.0f, 0.0f, 0.0f);
         for (int v = 0; v < len; ++v) {
           const int e = tc.edge[at + v];
-          const float3 p = edge_point(G, i, j, k, e, sh.t[e][tid]);
+          const float3 p = edge_point(sh, tid, e);
           M.x += p.x;
           M.y += p.y;
           M.z += p.z;
@@ -723,21 +773,20 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
       const unsigned live = min(min(32u, total - q0), (unsigned)min(max_tris - (base + q0), 32ull));
       if (lane < live) {
         const int cell = sh.cell_of[q];
-        const int i = sh.ci[cell], j = sh.cj[cell], k = sh.ck[cell];
         const unsigned code = g_ses_case[sh.cs[cell]].tri[q - sh.off[cell]];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
           const int e = (int)((code >> (4 * v)) & 15u);
           float3 p;
           if (e < 12)
-            p = edge_point(G, i, j, k, e, sh.t[e][cell]);
+            p = edge_point(sh, cell, e);
           else
             p = make_float3(sh.mean[3 * (e - 12)][cell], sh.mean[3 * (e - 12) + 1][cell], sh.mean[3 * (e - 12) + 2][cell]);
           sh.stage[wid][9 * lane + 3 * v] = p.x;
           sh.stage[wid][9 * lane + 3 * v + 1] = p.y;
           sh.stage[wid][9 * lane + 3 * v + 2] = p.z;
           if (labels) {
-            const long long cell_id = ((long long)k * (G.ny - 1) + j) * (G.nx - 1) + i;
+            const long long cell_id = ((long long)sh.ck[cell] * (G.ny - 1) + sh.cj[cell]) * (G.nx - 1) + sh.ci[cell];
             labels[(base + q) * 3 + v] = cell_id * 16 + e;
           }
         }

@@ -29,6 +29,23 @@ def test_ses_window_sizes_at_tile_edges(dims, K):
     check_same(gpu_ses(x, origin, h, d, probe), oracle.ses(x, origin, h, d, probe=probe), "K=%d %s" % (K, dims))
 
 
+@pytest.mark.parametrize("shift", [0.0, 3000.0, 60000.0])
+def test_ses_interior_far_from_the_origin(shift):
+    """The FP32 filter of the interior widens with the coordinates until the exact test decides every chord's ends;
+    radii that put points exactly on a sphere (grid-aligned centres, R a multiple of the spacing) are decided alike."""
+    rng = np.random.default_rng(5)
+    x = np.empty((60, 4), np.float32)
+    x[:, :3] = np.round(rng.uniform(0, 12, (60, 3)) * 2) / 2 + shift
+    x[:30, :3] += rng.uniform(-0.3, 0.3, (30, 3)).astype(np.float32)
+    x[:, 3] = rng.choice([0.5, 1.0, 1.5, 1.7], 60)
+    origin, d = np.full(3, shift - 4.0, np.float32), np.array((41, 41, 41), np.int32)
+    ref = oracle.ses(x, origin, np.float32(0.5), d, probe=1.5)
+    g = gpu_ses(x, origin, 0.5, d, 1.5)
+    np.testing.assert_array_equal(g["sas"], ref.sas)
+    np.testing.assert_array_equal(g["edt2"], ref.edt2)
+    np.testing.assert_array_equal(g["labels"], ref.edges)
+
+
 def test_ses_count_then_emit():
     """The two-call form: no surface before the first count or after a plain call; partial and repeated writes; the
     distances also go to the caller's plane."""
