@@ -285,9 +285,10 @@ static vtx_status prepare(vtx_ctx *c, const Geometry &g, bool soft, long long st
     else
       c->err.clear();
   }
-  // covered-pixel list of the two-pass resolve (32-bit entries: only when every pixel index fits)
+  // covered-pixel list of the two-pass resolve (32-bit indices: only when every pixel index fits, with room for a
+  // grid's stride past the last one)
   c->cov_ok = false;
-  if (!soft && n_img * g.pix_per_img < 4294967295LL) {
+  if (!soft && n_img * g.pix_per_img < 4294967296LL - (1LL << 24)) {
     if (ensure(c, c->covlist, sizeof(uint32_t) * (size_t)(n_img * g.pix_per_img), "covered pixels") == VTX_OK &&
         ensure(c, c->covmask, sizeof(uint32_t) * (size_t)(n_img * g.pix_per_img / 32 + 8), "coverage bits") == VTX_OK)
       c->cov_ok = true;

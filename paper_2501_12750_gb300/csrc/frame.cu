@@ -1794,12 +1794,22 @@ constexpr int kSsaoGroup = VTX_SSAO_GROUP;  // SSAO samples whose neighbour keys
 #define VTX_RESOLVE_2PASS 1
 #endif
 
-// A depth-key difference as float: the 32-bit conversion when it fits (the same rounding as the 64-bit one).
-__device__ __forceinline__ float key_diff_f(long long d) {
-  if (d >= -2147483647LL && d <= 2147483647LL) return __int2float_rn((int)d);
-  return ll_to_float_wide(d);
+// The difference a - b of two depth keys (the upper words of packed keys) as float: the magnitude fits 32 bits and
+// rounding to nearest is symmetric, so one unsigned conversion gives what a 64-bit signed one would.
+__device__ __forceinline__ float key_diff_f(uint32_t a, uint32_t b) {
+  const bool ge = a >= b;
+  const float f = __uint2float_rn(ge ? a - b : b - a);
+  return ge ? f : -f;
 }
 
+// Bound by issue: the winner's set-up and 16 neighbour samples a pixel.  With 32-bit indices in place of three 64-bit
+// divisions a pixel and a single image's view constants as immediate operands: close 4K view 480 -> 467 us,
+// ball-and-stick frame 292 -> 278 us, batch of 32 images 885 -> 872 us.
+//
+// ONE: a single image (its view constants are then compile-time indexed kernel parameters).  Key indices within an
+// image fit 32 bits (at most 2^28 pixels), and of a packed key the neighbours are asked for the depth word only: the
+// background's is 0xffffffff, which no primitive's key has.
+template <bool ONE>
 __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadeParams &sh, const float4 *__restrict__ frames,
                                               const uint8_t *__restrict__ elem, const uint2 *__restrict__ bonds,
                                               const ImageState *__restrict__ st,
@@ -1807,11 +1817,11 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
                                               int do_ssao, int img, int px, int py, unsigned long long key, Status *status) {
   const long long ppi = g.pix_per_img;
   {
-    const long long p = (long long)py * g.W + px;
-    const long long q = (long long)img * ppi + p;
+    const long long p = (unsigned)py * (unsigned)g.W + (unsigned)px;
+    const long long q = (ONE ? 0LL : (long long)img * ppi) + p;
     uint32_t id = (uint32_t)key;
-    float *nrm = out.normal + (long long)img * 3 * ppi + p;
-    float *rgb = out.rgb + (long long)img * 3 * ppi + p;
+    float *nrm = out.normal + (ONE ? 0LL : (long long)img * 3 * ppi) + p;
+    float *rgb = out.rgb + (ONE ? 0LL : (long long)img * 3 * ppi) + p;
     // bounds check of the decoded id (a corrupted key): recorded in the status word, drawn as background
     if (id != kNoId && (long long)id >= g.n_atoms + g.n_bonds) {
       atomicOr(&status->overflow, 32u);
@@ -1827,9 +1837,9 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
       if (out.ao) out.ao[q] = 1.0f;
       return;
     }
-    const ViewParams &v = g.views[img % g.n_views];
-    const ImageState s = st[img];
-    const float4 *X = frames + (long long)(img / g.n_views) * g.stride;
+    const ViewParams &v = ONE ? g.views[0] : g.views[img % g.n_views];
+    const ImageState s = st[ONE ? 0 : img];
+    const float4 *X = ONE ? frames : frames + (long long)(img / g.n_views) * g.stride;
     PrimGeom pg = prim_geom(g, v, X, bonds, id, s.zlo, s.S, false);
     const PixRay r = pix_ray(v, px, py);
     float3 o = local_o(pg.su.u0.hi, pg.su.u0.lo, pg.su.v0.hi, pg.su.v0.lo, pg.su.k, pg.su.dz, r);
@@ -1875,13 +1885,13 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
       T.y *= tinv;
       T.z *= tinv;
       float3 B = make_float3(n.y * T.z - n.z * T.y, n.z * T.x - n.x * T.z, n.x * T.y - n.y * T.x);
-      const unsigned long long *Kimg = keys + (long long)img * ppi;
-      const long long kP = (long long)(key >> 32);
+      const uint32_t *Dimg = reinterpret_cast<const uint32_t *>(keys + (ONE ? 0LL : (long long)img * ppi)) + 1;
+      const uint32_t kP = (uint32_t)(key >> 32);
       float occ = 0.0f;
       const float R = sh.ssao_radius;
-      // samples in groups of kSsaoGroup: the group's neighbour-key loads are issued together
+      // samples in groups of kSsaoGroup: the group's neighbour depths are loaded together
       for (int j0 = 0; j0 < sh.ssao_n; j0 += kSsaoGroup) {
-        long long at[kSsaoGroup];
+        int at[kSsaoGroup];
         float dls[kSsaoGroup];
 #pragma unroll
         for (int u = 0; u < kSsaoGroup; ++u) {
@@ -1902,17 +1912,17 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
               const float offy = -fden * (dy - r.b * dl);
               const int ix = px + (int)floorf(0.5f + offx);
               const int iy = py + (int)floorf(0.5f + offy);
-              if (ix >= 0 && iy >= 0 && ix < g.W && iy < g.H) at[u] = (long long)iy * g.W + ix;
+              if ((unsigned)ix < (unsigned)g.W && (unsigned)iy < (unsigned)g.H) at[u] = iy * g.W + ix;
             }
           }
         }
-        unsigned long long kf[kSsaoGroup];
+        uint32_t kf[kSsaoGroup];
 #pragma unroll
-        for (int u = 0; u < kSsaoGroup; ++u) kf[u] = at[u] >= 0 ? Kimg[at[u]] : kBgKey;
+        for (int u = 0; u < kSsaoGroup; ++u) kf[u] = at[u] >= 0 ? Dimg[2 * (size_t)at[u]] : 0xffffffffu;
 #pragma unroll
         for (int u = 0; u < kSsaoGroup; ++u) {
-          if ((uint32_t)kf[u] == kNoId) continue;
-          const float dzf = key_diff_f((long long)(kf[u] >> 32) - kP) * s.invS;  // z_f - t
+          if (kf[u] == 0xffffffffu) continue;
+          const float dzf = key_diff_f(kf[u], kP) * s.invS;  // z_f - t
           if (dzf <= dls[u] - sh.ssao_bias) {
             const float adz = fabsf(dzf);
             occ += adz <= R ? 1.0f : R / adz;
@@ -1924,16 +1934,16 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
     float3 col = make_float3(c.x * aof, c.y * aof, c.z * aof);
     if (sh.outline_depth > 0.0f) {
       // front side of a depth discontinuity: a 4-neighbour is background or deeper by more than outline_depth
-      const unsigned long long *Kimg = keys + (long long)img * ppi;
-      const long long kP = (long long)(key >> 32);
+      const uint32_t *Dimg = reinterpret_cast<const uint32_t *>(keys + (ONE ? 0LL : (long long)img * ppi)) + 1;
+      const uint32_t kP = (uint32_t)(key >> 32);
       const int nx[4] = {px - 1, px + 1, px, px};
       const int ny[4] = {py, py, py - 1, py + 1};
       bool edge = false;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        if (nx[u] < 0 || ny[u] < 0 || nx[u] >= g.W || ny[u] >= g.H) continue;
-        const unsigned long long kq = Kimg[(long long)ny[u] * g.W + nx[u]];
-        if ((uint32_t)kq == kNoId || key_diff_f((long long)(kq >> 32) - kP) * s.invS > sh.outline_depth) edge = true;
+        if ((unsigned)nx[u] >= (unsigned)g.W || (unsigned)ny[u] >= (unsigned)g.H) continue;
+        const uint32_t kq = Dimg[2 * (size_t)(ny[u] * g.W + nx[u])];
+        if (kq == 0xffffffffu || key_diff_f(kq, kP) * s.invS > sh.outline_depth) edge = true;
       }
       if (edge) col = make_float3(sh.outline_color[0], sh.outline_color[1], sh.outline_color[2]);
     }
@@ -1979,7 +1989,7 @@ __global__ __launch_bounds__(256, VTX_RESOLVE_MINB) void k_resolve(Geometry g, S
     k1 = k2;
     k2 = k3;
     const int py = py0 + 8 * i;
-    if (py < g.H) resolve_pixel(g, sh, frames, elem, bonds, st, keys, out, do_ssao, img, px, py, key, status);
+    if (py < g.H) resolve_pixel<false>(g, sh, frames, elem, bonds, st, keys, out, do_ssao, img, px, py, key, status);
   }
 }
 
@@ -1995,21 +2005,23 @@ __global__ __launch_bounds__(256, VTX_RESOLVE_MINB) void k_resolve(Geometry g, S
 // the 1,024-image trajectory batch (6 % coverage) is ~7 % slower in this
 // stage.  A shared work queue interleaving both kinds and a plain two-pass
 // form were measured too and were slower on the 4K frame.
+// Pixel indices of a launch fit 32 bits (the list is only made when they do).
 template <bool VEC>
 __global__ __launch_bounds__(256) void k_resolve_list(Geometry g, const unsigned long long *__restrict__ keys,
                                                       uint32_t *__restrict__ cov, uint32_t *__restrict__ mask,
                                                       Status *status) {
   pdl_enter();
-  const long long total = g.pix_per_img * g.n_img;
+  const uint32_t total = (uint32_t)(g.pix_per_img * g.n_img);
   const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
   constexpr int P = VEC ? 4 : 1;
-  const long long n_units = total / P;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long n_iter = (n_units + stride - 1) / stride;
-  for (long long it = 0; it < n_iter; ++it) {  // uniform trip count: every lane reaches the warp votes
-    const long long u = it * stride + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t n_units = total / P;
+  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t n_iter = (n_units + stride - 1) / stride;
+  for (uint32_t it = 0; it < n_iter; ++it) {  // uniform trip count: every lane reaches the warp votes
+    const uint32_t u = it * stride + blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = u < n_units;
-    const long long q0 = u * P;
+    const uint32_t q0 = u * P;
     unsigned covered = 0u;
     if (live) {
       if (VEC) {
@@ -2022,59 +2034,66 @@ __global__ __launch_bounds__(256) void k_resolve_list(Geometry g, const unsigned
       }
     }
     // coverage bits of the warp's 32 units (one word per pixel of a unit), for the background CTAs
+    unsigned m[P], warp_total = 0u, before = 0u;
 #pragma unroll
     for (int v = 0; v < P; ++v) {
-      const unsigned m = __ballot_sync(0xffffffffu, (covered >> v) & 1u);
-      if (lane == 0 && live) mask[(u >> 5) * P + v] = m;
+      m[v] = __ballot_sync(0xffffffffu, (covered >> v) & 1u);
+      warp_total += (unsigned)__popc(m[v]);
+      before += (unsigned)__popc(m[v] & lt);
     }
-    const int n_mine = __popc(covered);
-    int incl = n_mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
+    if (lane == 0 && live) {
+      if constexpr (VEC)
+        *reinterpret_cast<uint4 *>(mask + (u >> 5) * 4) = make_uint4(m[0], m[1], m[2], m[3]);
+      else
+        mask[u >> 5] = m[0];
     }
-    const int warp_total = __shfl_sync(0xffffffffu, incl, 31);
-    if (warp_total == 0) continue;
+    if (warp_total == 0u) continue;
     unsigned base = 0u;
-    if (lane == 31) base = atomicAdd(&status->n_cov, (unsigned)warp_total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    unsigned at = base + (unsigned)(incl - n_mine);
+    if (lane == 0) base = atomicAdd(&status->n_cov, warp_total);
+    unsigned at = __shfl_sync(0xffffffffu, base, 0) + before;
 #pragma unroll
     for (int v = 0; v < P; ++v)
-      if (covered & (1u << v)) cov[at++] = (uint32_t)(q0 + v);
+      if (covered & (1u << v)) cov[at++] = q0 + v;
   }
 }
 
-template <bool VEC>
+template <bool VEC, bool ONE>
 __global__ __launch_bounds__(256, VTX_RESOLVE_MINB) void k_resolve_split(
     Geometry g, ShadeParams sh, const float4 *__restrict__ frames, const uint8_t *__restrict__ elem,
     const uint2 *__restrict__ bonds, const ImageState *__restrict__ st, const unsigned long long *__restrict__ keys,
     Outputs out, int do_ssao, const uint32_t *__restrict__ cov, const uint32_t *__restrict__ mask,
     Status *status, int n_shade) {
   pdl_enter();
-  const long long ppi = g.pix_per_img;
+  const uint32_t ppi = (uint32_t)g.pix_per_img;
   if ((int)blockIdx.x < n_shade) {
     const unsigned n = status->n_cov;
     for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (unsigned)n_shade * blockDim.x) {
-      const long long q = cov[e];
-      const int img = (int)(q / ppi);
-      const long long p = q - (long long)img * ppi;
-      const int py = (int)(p / g.W), px = (int)(p - (long long)py * g.W);
-      resolve_pixel(g, sh, frames, elem, bonds, st, keys, out, do_ssao, img, px, py, keys[q], status);
+      const uint32_t q = cov[e];
+      const uint32_t img = ONE ? 0u : q / ppi, p = ONE ? q : q - img * ppi;
+      const uint32_t py = p / (unsigned)g.W, px = p - py * (unsigned)g.W;
+      resolve_pixel<ONE>(g, sh, frames, elem, bonds, st, keys, out, do_ssao, (int)img, (int)px, (int)py, keys[q],
+                         status);
     }
     return;
   }
   constexpr int P = VEC ? 4 : 1;
-  const long long n_units = ppi * g.n_img / P;
+  const uint32_t n_units = (uint32_t)(g.pix_per_img * g.n_img) / P;
   const float inf = __int_as_float(0x7f800000);
-  for (long long u = (long long)(blockIdx.x - n_shade) * blockDim.x + threadIdx.x; u < n_units;
-       u += (long long)(gridDim.x - n_shade) * blockDim.x) {
-    const long long q0 = u * P;
+  const uint32_t stride = (gridDim.x - n_shade) * blockDim.x;
+  const uint32_t n_iter = (n_units + stride - 1) / stride;
+  uint32_t u = (blockIdx.x - n_shade) * blockDim.x + threadIdx.x;
+  for (uint32_t it = 0; it < n_iter; ++it, u += stride) {
+    if (u >= n_units) break;
+    const uint32_t q0 = u * P;
     unsigned covered = 0u;  // from the list pass's bits (1 bit per pixel) instead of the 8-byte keys
-#pragma unroll
-    for (int v = 0; v < P; ++v) covered |= ((mask[(u >> 5) * P + v] >> (u & 31)) & 1u) << v;
-    const long long img = q0 / ppi, p = q0 - img * ppi;
+    if constexpr (VEC) {
+      const uint4 m = *reinterpret_cast<const uint4 *>(mask + (u >> 5) * 4);
+      covered = ((m.x >> (u & 31)) & 1u) | ((m.y >> (u & 31)) & 1u) << 1 | ((m.z >> (u & 31)) & 1u) << 2 |
+                ((m.w >> (u & 31)) & 1u) << 3;
+    } else {
+      covered = (mask[u >> 5] >> (u & 31)) & 1u;
+    }
+    const size_t img = ONE ? 0 : q0 / ppi, p = ONE ? q0 : q0 - (uint32_t)img * ppi;
     float *nrm = out.normal + img * 3 * ppi + p;
     float *rgb = out.rgb + img * 3 * ppi + p;
     if (VEC && covered == 0u) {
@@ -2083,10 +2102,10 @@ __global__ __launch_bounds__(256, VTX_RESOLVE_MINB) void k_resolve_split(
       *reinterpret_cast<uint4 *>(out.id + q0) = make_uint4(kNoId, kNoId, kNoId, kNoId);
       *reinterpret_cast<float4 *>(nrm) = z4;
       *reinterpret_cast<float4 *>(nrm + ppi) = z4;
-      *reinterpret_cast<float4 *>(nrm + 2 * ppi) = z4;
+      *reinterpret_cast<float4 *>(nrm + 2 * (size_t)ppi) = z4;
       *reinterpret_cast<float4 *>(rgb) = make_float4(sh.bg[0], sh.bg[0], sh.bg[0], sh.bg[0]);
       *reinterpret_cast<float4 *>(rgb + ppi) = make_float4(sh.bg[1], sh.bg[1], sh.bg[1], sh.bg[1]);
-      *reinterpret_cast<float4 *>(rgb + 2 * ppi) = make_float4(sh.bg[2], sh.bg[2], sh.bg[2], sh.bg[2]);
+      *reinterpret_cast<float4 *>(rgb + 2 * (size_t)ppi) = make_float4(sh.bg[2], sh.bg[2], sh.bg[2], sh.bg[2]);
       if (out.ao) *reinterpret_cast<float4 *>(out.ao + q0) = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
     } else {
 #pragma unroll
@@ -2094,16 +2113,15 @@ __global__ __launch_bounds__(256, VTX_RESOLVE_MINB) void k_resolve_split(
         if (covered & (1u << v)) continue;
         out.depth[q0 + v] = inf;
         out.id[q0 + v] = kNoId;
-        nrm[v] = nrm[ppi + v] = nrm[2 * ppi + v] = 0.0f;
+        nrm[v] = nrm[ppi + v] = nrm[2 * (size_t)ppi + v] = 0.0f;
         rgb[v] = sh.bg[0];
         rgb[ppi + v] = sh.bg[1];
-        rgb[2 * ppi + v] = sh.bg[2];
+        rgb[2 * (size_t)ppi + v] = sh.bg[2];
         if (out.ao) out.ao[q0 + v] = 1.0f;
       }
     }
   }
 }
-
 
 // ------------------------------------------------------------ launchers --
 
@@ -2313,17 +2331,13 @@ cudaError_t run_frame_pipeline(const Geometry &g, const ShadeParams &sh, const S
     // shading CTAs first (they start at once and stay resident), background CTAs behind them
     const int n_shade = VTX_SHADE_PER_SM * sms;
     const int gb = (int)(want < 8LL * sms ? (want > 0 ? want : 1) : 8LL * sms);
-    if (vec) {
-      launch_pdl(k_resolve_list<true>, gl, 256, 0, st, g, s.keys, s.cov_list, s.cov_mask, s.status);
-      ev_rec(evs, 6, st);
-      launch_pdl(k_resolve_split<true>, n_shade + gb, 256, 0, st, g, sh, Xr, sc.elem, sc.bonds, s.state, s.keys, out,
-                                                            ssao ? 1 : 0, s.cov_list, s.cov_mask, s.status, n_shade);
-    } else {
-      launch_pdl(k_resolve_list<false>, gl, 256, 0, st, g, s.keys, s.cov_list, s.cov_mask, s.status);
-      ev_rec(evs, 6, st);
-      launch_pdl(k_resolve_split<false>, n_shade + gb, 256, 0, st, g, sh, Xr, sc.elem, sc.bonds, s.state, s.keys, out,
-                                                             ssao ? 1 : 0, s.cov_list, s.cov_mask, s.status, n_shade);
-    }
+    const auto list = vec ? k_resolve_list<true> : k_resolve_list<false>;
+    const auto shade = g.n_img == 1 ? (vec ? k_resolve_split<true, true> : k_resolve_split<false, true>)
+                                    : (vec ? k_resolve_split<true, false> : k_resolve_split<false, false>);
+    launch_pdl(list, gl, 256, 0, st, g, s.keys, s.cov_list, s.cov_mask, s.status);
+    ev_rec(evs, 6, st);
+    launch_pdl(shade, n_shade + gb, 256, 0, st, g, sh, Xr, sc.elem, sc.bonds, s.state, s.keys, out, ssao ? 1 : 0,
+               s.cov_list, s.cov_mask, s.status, n_shade);
   } else {
     dim3 grid((g.W + 31) / 32, (g.H + 31) / 32, g.n_img);
     launch_pdl(k_resolve, grid, 256, 0, st, g, sh, Xr, sc.elem, sc.bonds, s.state, s.keys, out, ssao ? 1 : 0,

@@ -300,7 +300,6 @@ struct Setup {
 // 64-bit one to a separate, rarely called function, so that the common path
 // never issues it (a ternary would let the compiler evaluate both sides).
 static __device__ __noinline__ long long float_to_ll_wide(float x) { return llrintf(fminf(fmaxf(x, -4.0e18f), 4.0e18f)); }
-static __device__ __noinline__ float ll_to_float_wide(long long d) { return (float)d; }
 
 // rint(x) for an integer-valued x (a float that already holds an integer)
 __device__ __forceinline__ long long float_to_ll(float x) {
