@@ -125,7 +125,8 @@ struct __align__(16) PrimRec {
   int key_hi;                // depth key of zr, high word (the key may leave [0, 2^32) for near-eye primitives)
   uint32_t id;               // primitive id
   float hl;                  // cylinder half length; 0 for spheres
-  float ax, ay, az, pad;     // cylinder axis (internal frame)
+  float ax, ay, az;          // cylinder axis (internal frame)
+  uint32_t plain;            // 1: a sphere whose hits take the short form of the key (splat_plain)
 };
 
 // Sphere radius of an atom record in the current representation.
@@ -387,12 +388,16 @@ __device__ __forceinline__ bool cylinder_local(float3 o, const PixRay &r, float3
   float3 op = make_float3(fmaf(-oa, A.x, o.x), fmaf(-oa, A.y, o.y), fmaf(-oa, A.z, o.z));
   float a2 = fmaf(up.x, up.x, fmaf(up.y, up.y, __fmul_rn(up.z, up.z)));
   float b2 = fmaf(op.x, up.x, fmaf(op.y, up.y, __fmul_rn(op.z, up.z)));
-  float c2 = fmaf(-rb, rb, fmaf(op.x, op.x, fmaf(op.y, op.y, __fmul_rn(op.z, op.z))));
+  const float opop = fmaf(op.x, op.x, fmaf(op.y, op.y, __fmul_rn(op.z, op.z)));
+  float c2 = fmaf(-rb, rb, opop);
   const float rb2 = __fmul_rn(rb, rb);
   float best = __int_as_float(0x7f800000);
   kind = 0;
   if (a2 > 1e-12f) {
     float disc = fmaf(b2, b2, __fmul_rn(-a2, c2));
+    // The ray misses the infinite cylinder by more than any rounding: at every s, |op + s up|^2 - rb^2 >= -disc / a2,
+    // here above 9e-6 (|op|^2 + rb^2), so neither cap test below could accept (their |q|^2 is good to 4e-7).
+    if (disc < -1e-5f * fmaf(b2, b2, a2 * (opop + rb2))) return false;
     if (disc >= 0.0f) {
       float s1 = __fdiv_rn(__fsub_rn(-b2, sqrtf(disc)), a2);
       float ax = fmaf(s1, ua, oa);
@@ -587,6 +592,28 @@ __device__ __forceinline__ bool lean_box(const ViewParams &v, int W, int H, floa
   const float t = v.hc * rho * fmaf(2.0f * rho, rho, 1.0f);
   const float hx = fmaf(t, fmaf(fabsf(mx), rho, fmaf(0.5f * mx, mx, 1.0f)), v.e0);
   const float hy = fmaf(t, fmaf(fabsf(my), rho, fmaf(0.5f * my, my, 1.0f)), v.e0);
+  const float ux = fmaf(v.f, mx, v.cxm), uy = fmaf(-v.f, my, v.cym);
+  b.x0 = (int)fminf(fmaxf(ceilf(ux - hx), 0.0f), (float)W);
+  b.x1 = (int)fmaxf(fminf(floorf(ux + hx), (float)(W - 1)), -1.0f);
+  b.y0 = (int)fminf(fmaxf(ceilf(uy - hy), 0.0f), (float)H);
+  b.y1 = (int)fmaxf(fminf(floorf(uy + hy), (float)(H - 1)), -1.0f);
+  return b.x0 <= b.x1 && b.y0 <= b.y1;
+}
+
+// Candidate pixel box of a capped cylinder (centre vx, vy, vz known to err, unit axis A, half length hl, radius rb,
+// bounding radius Rb).  A point of it is C + tau A + w, |tau| <= hl, |w| <= rb, so with m = vx / vz its projected
+// slope differs from m by (tau (A.x - m A.z) + w.x - m w.z) / z, at most (hl |A.x - m A.z| + rb sqrt(1 + m^2)) /
+// (vz - hl |A.z| - rb); likewise in y.  rb is widened by the error of the centre and the axis.  Near the eye plane:
+// the bounding sphere's box.
+__device__ __forceinline__ bool cylinder_box(const ViewParams &v, int W, int H, float vx, float vy, float vz, float err,
+                                             float3 A, float hl, float rb, float Rb, PixBox &b) {
+  const float Rm = Rb + err;
+  if (!(vz > 8.0f * Rm && hl > 0.0f)) return lean_box(v, W, H, vx, vy, vz, Rm, b);
+  const float rz = rcp_approx(vz), rm = rb + 2.0f * err + 1e-5f * Rm;
+  const float mx = vx * rz, my = vy * rz;
+  const float t = v.hc * rcp_approx(vz - hl * fabsf(A.z) - rm) * 1.00001f;
+  const float hx = fmaf(t, fmaf(hl, fabsf(fmaf(-mx, A.z, A.x)), rm * fmaf(0.5f * mx, mx, 1.0f)), v.e0);
+  const float hy = fmaf(t, fmaf(hl, fabsf(fmaf(-my, A.z, A.y)), rm * fmaf(0.5f * my, my, 1.0f)), v.e0);
   const float ux = fmaf(v.f, mx, v.cxm), uy = fmaf(-v.f, my, v.cym);
   b.x0 = (int)fminf(fmaxf(ceilf(ux - hx), 0.0f), (float)W);
   b.x1 = (int)fmaxf(fminf(floorf(ux + hx), (float)(W - 1)), -1.0f);
