@@ -592,10 +592,11 @@ static void set_representation(Geometry &g, const vtx_settings *s) {
   g.clip_on = (s->clip_plane[0] != 0.0f || s->clip_plane[1] != 0.0f || s->clip_plane[2] != 0.0f) ? 1 : 0;
 }
 
-// Library-default direct-splat threshold (splat_max_px = 0): sparse frames (at most one primitive per 8
-// pixels) bin all but the smallest primitives for the tile raster (4 px), crowded ones splat boxes of up to
-// 16 px directly.  Measured with the autotuner: the 1e5-atom 1080p frame is fastest at 4 (0.082 -> 0.078
-// ms), the 1e8-atom 4K frame and the 500k-atom trajectory images at 16.  Every threshold gives the same planes.
+// Library-default direct-splat threshold (splat_max_px = 0) where the survivors' sizes are not known to setup (batches,
+// frames with bonds): sparse images (at most one primitive per 8 pixels) bin all but the smallest primitives for the
+// tile raster (4 px), crowded ones splat boxes of up to 16 px directly.  Measured with the autotuner: the
+// 500k-atom trajectory images are fastest at 16; a ball-and-stick frame (60,000 atoms at 1080p) takes 232 us at 4,
+// 240 at 16 and 309 at 256, as cylinders are dear to splat.  Every threshold gives the same planes.
 static int default_splat(long long prims_per_img, long long pix_per_img) {
   return prims_per_img * 8 <= pix_per_img ? 4 : 16;
 }
@@ -612,6 +613,7 @@ static vtx_status render_once(vtx_ctx *c, const vtx_settings *s, const vtx_outpu
   g.n_atoms = c->n_atoms;
   g.n_bonds = (s->mode == VTX_MODE_BALL_AND_STICK || s->mode == VTX_MODE_STICKS) ? c->n_bonds : 0;
   g.splat_max = s->splat_max_px ? s->splat_max_px : default_splat(g.n_atoms + g.n_bonds, g.pix_per_img);
+  g.splat_auto = s->splat_max_px == 0 && g.n_bonds == 0;  // single frames of spheres: chosen in setup (splat_choice)
   g.surv_cap = c->n_atoms + g.n_bonds + cull_survivor_slack(c->n_atoms);
   // no occlusion pass for a single frame: measured on the 1e8-atom 4K frame (whose set-up is 0.07 ms of
   // 0.43) it cost more than it saved (2,331 -> 1,959 frames/s, with the bounds then in a plane of their own):

@@ -81,6 +81,9 @@ __global__ __launch_bounds__(256) void k_clear(ImageState *st, int n_img, Status
     s.invS = 0.0f;
     s.occl = 0u;
     s.n_vis = 0u;
+    s.rho_bits = 0u;
+    s.rho2 = 0.0f;
+    s.n_rho = 0u;
     st[tid] = s;
   }
   if (tid == 0) {
@@ -373,6 +376,8 @@ __global__ __launch_bounds__(kCullThreads, kCullCtasPerSm) void k_cull_direct(Ge
   uint32_t slab = kNoId;
   int used = kSlab;
   float zlo = __int_as_float(0x7f800000), zhi = 0.0f;
+  float rmax = 0.0f, rsum = 0.0f;  // of every fourth atom's R / z, if it survives: the largest, the sum of the squares
+  unsigned rcnt = 0u;              // and their number
   for (long long a0 = (long long)blockIdx.x * CH; a0 < n; a0 += (long long)gridDim.x * CH) {
     float4 a[kCullPT];
 #pragma unroll
@@ -388,7 +393,8 @@ __global__ __launch_bounds__(kCullThreads, kCullCtasPerSm) void k_cull_direct(Ge
       view_f32x2(vp, make_float2(p.x, q.x), make_float2(p.y, q.y), make_float2(p.z, q.z), vx, vy, vz, err);
       const float2 Rm = __fadd2_rn(r, err);
       bool k0, k1;
-      cull_lean_x2(vp, vx, vy, vz, Rm, k0, k1);
+      float size0;
+      cull_lean_x2(vp, vx, vy, vz, Rm, k0, k1, size0);
       k0 = k0 && p.w >= 0.0f;
       k1 = k1 && q.w >= 0.0f;
       if (!PLAIN) {
@@ -398,6 +404,11 @@ __global__ __launch_bounds__(kCullThreads, kCullCtasPerSm) void k_cull_direct(Ge
       if (k0) {
         zlo = fminf(zlo, vz.x - Rm.x);
         zhi = fmaxf(zhi, vz.x + Rm.x);
+        if (j == 0) {
+          rmax = fmaxf(rmax, size0);
+          rsum = fmaf(size0, size0, rsum);
+          ++rcnt;
+        }
       }
       if (k1) {
         zlo = fminf(zlo, vz.y - Rm.y);
@@ -415,10 +426,41 @@ __global__ __launch_bounds__(kCullThreads, kCullCtasPerSm) void k_cull_direct(Ge
   if (slab != kNoId)
     for (int i = used + lane; i < kSlab; i += 32)
       if ((long long)slab + i < cap) surv[slab + i] = kNoId;
+  // one set of atomics per CTA: thousands of warps' on one address would queue for longer than a small frame's cull
   warp_minmax(zlo, zhi);
-  if (lane == 0 && zhi > 0.0f) {
-    atomicMin(&st[0].zlo_bits, __float_as_uint(fmaxf(zlo, 0.0f)));
-    atomicMax(&st[0].zhi_bits, __float_as_uint(zhi));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rsum += __shfl_xor_sync(0xffffffffu, rsum, o);
+  rcnt = __reduce_add_sync(0xffffffffu, rcnt);
+  rmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rmax)));
+  __shared__ float s_zlo[kCullThreads / 32], s_zhi[kCullThreads / 32], s_rmax[kCullThreads / 32],
+      s_rsum[kCullThreads / 32];
+  __shared__ unsigned s_rcnt[kCullThreads / 32];
+  if (lane == 0) {
+    const int w = threadIdx.x >> 5;
+    s_zlo[w] = zlo;
+    s_zhi[w] = zhi;
+    s_rmax[w] = rmax;
+    s_rsum[w] = rsum;
+    s_rcnt[w] = rcnt;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kCullThreads / 32; ++w) {
+      zlo = fminf(zlo, s_zlo[w]);
+      zhi = fmaxf(zhi, s_zhi[w]);
+      rmax = fmaxf(rmax, s_rmax[w]);
+      rsum += s_rsum[w];
+      rcnt += s_rcnt[w];
+    }
+    if (zhi > 0.0f) {
+      atomicMin(&st[0].zlo_bits, __float_as_uint(fmaxf(zlo, 0.0f)));
+      atomicMax(&st[0].zhi_bits, __float_as_uint(zhi));
+    }
+    if (rcnt) {
+      atomicMax(&st[0].rho_bits, __float_as_uint(rmax));
+      atomicAdd(&st[0].rho2, rsum);
+      atomicAdd(&st[0].n_rho, rcnt);
+    }
   }
 }
 
@@ -495,7 +537,8 @@ __global__ __launch_bounds__(kCullThreads, 4) void k_cull_multi(Geometry g, cons
         view_f32x2(vp, make_float2(p.x, q.x), make_float2(p.y, q.y), make_float2(p.z, q.z), vx, vy, vz, err);
         const float2 Rm = __fadd2_rn(r, err);
         bool k0, k1;
-        cull_lean_x2(vp, vx, vy, vz, Rm, k0, k1);
+        float size0;
+        cull_lean_x2(vp, vx, vy, vz, Rm, k0, k1, size0);
         k0 = k0 && in0;
         k1 = k1 && in1;
         if (k0) {
@@ -683,10 +726,11 @@ __device__ __forceinline__ bool prim_hit(const PrimGeom &p, float3 o, const PixR
 // Ray-cast primitive p at every pixel of its candidate box, merging hits into the key plane K (one lane).
 // One flat loop over the box's pixels: the lanes of a warp, whose boxes differ in shape, then run for the
 // largest box's pixel count rather than for the most rows times the most columns.
+// Of the box's rows, the lane takes the sub-th and every (1 << shift)-th after it.
 __device__ __forceinline__ void splat_box(const Geometry &g, const ViewParams &v, const PrimGeom &p, const PixBox &box,
-                                          float S, uint32_t id, unsigned long long *K) {
-  const int npix = (box.x1 - box.x0 + 1) * (box.y1 - box.y0 + 1);
-  int px = box.x0, py = box.y0;
+                                          float S, uint32_t id, unsigned long long *K, int sub, int shift) {
+  const int npix = (box.x1 - box.x0 + 1) * ((box.y1 - box.y0 - sub + (1 << shift)) >> shift);
+  int px = box.x0, py = box.y0 + sub;
   for (int i = 0; i < npix; ++i) {
     PixRay r = pix_ray(v, px, py);
     float3 o = local_o(p.su.u0.hi, p.su.u0.lo, p.su.v0.hi, p.su.v0.lo, p.su.k, p.su.dz, r);
@@ -697,7 +741,7 @@ __device__ __forceinline__ void splat_box(const Geometry &g, const ViewParams &v
       atomicMin(K + (long long)py * g.W + px, pack_key(p.su.keyc, sh, S, id));
     if (++px > box.x1) {
       px = box.x0;
-      ++py;
+      py += 1 << shift;
     }
   }
 }
@@ -720,15 +764,17 @@ __device__ __forceinline__ bool splat_plain(const ViewParams &v, const PrimGeom 
 // image's view constants as immediate operands, the close 4K view of 1.1e7 atoms went from 544 to 480 us and a
 // batch of 32 images of 500,000 atoms from 942 to 885 us.
 __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams &v, const PrimGeom &p,
-                                             const PixBox &box, float S, uint32_t id, unsigned long long *K) {
-  const int w = box.x1 - box.x0 + 1, npix = w * (box.y1 - box.y0 + 1);
+                                             const PixBox &box, float S, uint32_t id, unsigned long long *K, int sub,
+                                             int shift) {
+  const int w = box.x1 - box.x0 + 1, npix = w * ((box.y1 - box.y0 - sub + (1 << shift)) >> shift);
   const float x0 = (float)box.x0 + 0.5f, x1 = (float)box.x1 + 0.5f;
-  float2 c = make_float2(x0, (float)box.y0 + 0.5f);  // the pixel centre
+  const float dy = (float)(1 << shift);
+  float2 c = make_float2(x0, (float)(box.y0 + sub) + 0.5f);  // the pixel centre
   const float2 mc = make_float2(-v.cx, -v.cy), mh = make_float2(-p.su.u0.hi, -p.su.v0.hi);
   const float2 ml = make_float2(-p.su.u0.lo, -p.su.v0.lo);
   const uint32_t kc = (uint32_t)(unsigned long long)p.su.keyc;
-  const int skip = g.W - w + 1;  // from a row's last pixel to the next row's first
-  unsigned long long *k = K + (long long)box.y0 * g.W + box.x0;
+  const int skip = (g.W << shift) - w + 1;  // from a row's last pixel to the next row's first
+  unsigned long long *k = K + (long long)(box.y0 + sub) * g.W + box.x0;
   for (int i = 0; i < npix; ++i) {
     const float2 ab = __fmul2_rn(__fadd2_rn(c, mc), bc2(v.inv_f));                                // (a, -b)
     const float2 o = __fmul2_rn(bc2(p.su.k), __fadd2_rn(__fadd2_rn(c, mh), ml));                  // (o.x, -o.y)
@@ -743,9 +789,32 @@ __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams
     }
     const bool wrap = c.x == x1;
     c.x = wrap ? x0 : c.x + 1.0f;
-    c.y = wrap ? c.y + 1.0f : c.y;
+    c.y = wrap ? c.y + dy : c.y;
     k += wrap ? skip : 1;
   }
+}
+
+// The library-default splat threshold of an image from its survivors' projected sizes, and how many lanes share a
+// survivor (1 << shift).  With the survivors' mean box (2 f R / z + 1.2)^2 (from the cull's sample) and W their number
+// times it, the splat's pixel tests:
+//   every box splatted (up to 256 pixels) when the mean box is at most 30 pixels, or when W <= 1.6e7 and the largest
+//     radius is at most 6 pixels: the tile raster then has next to nothing to do;
+//   else only boxes of up to 4 pixels, the others rasterised.  Large spheres are cheaper there, and a mixture of both
+//     is dearer than either.
+// Measured (frame, all splatted against 4 pixels): 2,000 atoms at 256x256 20 / 33 us, 3e4 at 720p 38 / 52, 1e5 at
+// 1080p (mean box 61) 57 / 71, 2e5 at 1080p (42) 68 / 86, 5e5 at 1080p (26) 81 / 139, 1.1e7-atom close view (10)
+// 400 / 582; but 3e5 at 1440p (54, W = 1.6e7) 108 / 111, 1e6 at 4K (54) 296 / 265, 6e4 at 4K (289) 183 / 141.
+// Sharing pays while the survivors alone leave lanes idle: 2,000 atoms 37 -> 20 us at 8 lanes, 3e4 53 -> 38 at 8, 1e5
+// 61 -> 57 at 4 (66 at 8); 2e5 68 -> 73 at 4.
+struct SplatChoice {
+  int splat_max, shift;
+};
+__device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const ViewParams &v, const ImageState &s) {
+  if (!g.splat_auto) return {g.splat_max, 0};
+  const float n = 4.0f * (float)s.n_rho;  // survivors (n_surv counts the slabs' unused slots too)
+  const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
+  if (!(mean <= 30.0f || (mean * n <= 1.6e7f && v.f * __uint_as_float(s.rho_bits) <= 6.0f))) return {4, 0};
+  return {256, n <= 49152.0f ? 3 : (n <= 163840.0f ? 2 : 0)};
 }
 
 // Setup occupancy: 4 CTAs per SM (63 registers, a few bytes spilled) and 8
@@ -785,14 +854,17 @@ __global__ __launch_bounds__(256, VTX_SETUP_MINB) void k_setup(Geometry g, const
   const uint32_t *sv = (kept_list ? kept : surv) + (long long)img * g.surv_cap;
   unsigned long long *K = keys + (long long)img * g.pix_per_img;
   const int lane = threadIdx.x & 31;
-  const long long stride = (long long)gridDim.x * blockDim.x;
+  // with few survivors, 1 << shift neighbouring lanes share one: each does its set-up and splats its own rows
+  const SplatChoice choice = ONE ? splat_choice(g, v, s) : SplatChoice{g.splat_max, 0};
+  const int shift = choice.shift, sub = lane & ((1 << shift) - 1);
+  const long long stride = (long long)(gridDim.x * blockDim.x) >> shift;
   // two-stage prefetch: the id two iterations ahead, the atom record one ahead
-  const long long k0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long k0 = (long long)(blockIdx.x * blockDim.x + threadIdx.x) >> shift;
   const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   uint32_t id_cur = k0 < n ? sv[k0] : 0u;
   uint32_t id_nxt = k0 + stride < n ? sv[k0 + stride] : 0u;
   float4 a_cur = (k0 < n && (long long)id_cur < g.n_atoms) ? X[id_cur] : zero4;
-  for (long long k = k0; k - lane < n; k += stride) {  // the same trip count for the lanes of a warp
+  for (long long k = k0; k - (lane >> shift) < n; k += stride) {  // the same trip count for the lanes of a warp
     const float4 a_nxt = (k + stride < n && (long long)id_nxt < g.n_atoms) ? X[id_nxt] : zero4;
     const uint32_t id_nn = k + 2 * stride < n ? sv[k + 2 * stride] : 0u;
     bool binned = false;
@@ -821,12 +893,12 @@ __global__ __launch_bounds__(256, VTX_SETUP_MINB) void k_setup(Geometry g, const
       }
       if (any) {
         const long long npx = (long long)(box.x1 - box.x0 + 1) * (long long)(box.y1 - box.y0 + 1);
-        if (!SOFT && npx <= g.splat_max) {
+        if (!SOFT && npx <= choice.splat_max) {
           if (p.hl == 0.0f && splat_plain(v, p, s.S))
-            splat_sphere(g, v, p, box, s.S, id, K);
+            splat_sphere(g, v, p, box, s.S, id, K, sub, shift);
           else
-            splat_box(g, v, p, box, s.S, id, K);
-        } else {
+            splat_box(g, v, p, box, s.S, id, K, sub, shift);
+        } else if (sub == 0) {
           binned = true;
           rec.u0h = p.su.u0.hi;
           rec.u0l = p.su.u0.lo;
@@ -2162,7 +2234,8 @@ static inline void ev_rec(StageEvents *e, int i, cudaStream_t st) {
 // unchanged; the launch latency and prologue of each kernel overlap the
 // previous kernel's tail.
 template <typename... P, typename... A>
-static cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+static cudaError_t launch_kernel(bool overlap, void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                                 A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
@@ -2172,8 +2245,12 @@ static cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+static cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  return launch_kernel(true, k, grid, block, smem, st, args...);
 }
 
 #ifndef VTX_CLEAR_MEMSET
@@ -2223,14 +2300,14 @@ cudaError_t run_binning(const Geometry &g, const Scene &sc, const Scratch &s, cu
     if (g.n_views == 1 && g.n_frames == 1 && sc.counts == nullptr && !g.soft) {
       const int b1 = (int)cull_one_ctas(g.n_atoms);
       const bool plain = g.mode == 0 && !g.clip_on;
-      if (sc.stage && plain)
-        launch_pdl(k_cull_direct<true, true>, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, sc.stage);
-      else if (sc.stage)
-        launch_pdl(k_cull_direct<false, true>, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, sc.stage);
-      else if (plain)
-        launch_pdl(k_cull_direct<true, false>, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, nullptr);
-      else
-        launch_pdl(k_cull_direct<false, false>, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, nullptr);
+      // A large cull starts only when the clear has ended: placed early, its CTAs (one wave of persistent ones) and
+      // set-up's behind them end up where they slow the stream (1e8 atoms at 4K 479 -> 416 us, 1.1e7-atom
+      // close view 452 -> 405 us; any one of clear, cull and set-up without overlap does it).  Below that the
+      // launch latency saved is worth more (1.07e6 atoms at 8K 458 / 461 us, 2,000 atoms 20.4 / 21.9 us).
+      const bool overlap = g.n_atoms < (4LL << 20);
+      const auto cull = sc.stage ? (plain ? k_cull_direct<true, true> : k_cull_direct<false, true>)
+                                 : (plain ? k_cull_direct<true, false> : k_cull_direct<false, false>);
+      launch_kernel(overlap, cull, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, sc.stage);
     } else if (!g.soft && g.n_views <= 4 && g.surv_cap >= per_frame + cull_multi_slack(per_frame, g.n_frames)) {
       // a batch (frames x up to 4 views): the barrier-free multi-view cull
       const dim3 gm(cull_multi_ctas(per_frame, g.n_frames), g.n_frames);

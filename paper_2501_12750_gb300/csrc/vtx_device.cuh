@@ -63,6 +63,7 @@ struct Geometry {
   float clip[4];         // clip plane (n, d); clip_on = n != 0
   int clip_on;
   int splat_max;         // max candidate pixels for the direct splat path
+  int splat_auto;        // 1: setup picks the splat threshold from the survivors' sizes (splat_choice), not splat_max
   int dbg_first_wait;    // test hook: polls allowed for the multi-view cull's first stage wait (-1: normal limit)
   int soft;              // 1 = soft-edge binning (dilated bounds, no splat, every survivor binned)
   int occl;              // 1 = occlusion pass allowed: survivors proven hidden by FP32 depth bounds skip setup
@@ -99,6 +100,10 @@ struct ImageState {
   float zlo, S, invS;     // key = (depth - zlo) * S
   unsigned int occl;      // 1: this image runs the occlusion pass (many survivors per pixel)
   unsigned int n_vis;     // occlusion pass: survivors its test could not prove hidden (the kept list)
+  unsigned int rho_bits;  // single-view cull, over a sample of the survivors (every fourth atom's): atomicMax of
+                          // R / z (float bits; 1 near the eye plane),
+  float rho2;             // the sum of its squares
+  unsigned int n_rho;     // and the sample's size
 };
 
 // Launch-wide status (device memory, read back by the host).
@@ -561,8 +566,9 @@ __device__ __forceinline__ void view_f32x2(const ViewParams &v, float2 x, float2
   err = make_float2(4e-7f * (fabsf(dx.x) + fabsf(dy.x) + fabsf(dz.x)), 4e-7f * (fabsf(dx.y) + fabsf(dy.y) + fabsf(dz.y)));
 }
 
+// size0: the first atom's R / z, or 1 when it comes within 8 radii of the eye plane.
 __device__ __forceinline__ void cull_lean_x2(const ViewParams &v, float2 vx, float2 vy, float2 vz, float2 Rm, bool &k0,
-                                             bool &k1) {
+                                             bool &k1, float &size0) {
   const float2 front = __fadd2_rn(vz, Rm);
   const float2 r8 = __fmul2_rn(bc2(8.0f), Rm);
   const float2 rz = make_float2(rcp_approx(vz.x), rcp_approx(vz.y));
@@ -576,8 +582,10 @@ __device__ __forceinline__ void cull_lean_x2(const ViewParams &v, float2 vx, flo
   const float2 nx = make_float2(fminf(fmaxf(rintf(ux.x), 0.0f), v.wm1), fminf(fmaxf(rintf(ux.y), 0.0f), v.wm1));
   const float2 ny = make_float2(fminf(fmaxf(rintf(uy.x), 0.0f), v.hm1), fminf(fmaxf(rintf(uy.y), 0.0f), v.hm1));
   const float2 ex = __fadd2_rn(ux, make_float2(-nx.x, -nx.y)), ey = __fadd2_rn(uy, make_float2(-ny.x, -ny.y));
-  k0 = front.x >= v.znear && (!(vz.x > r8.x) || (fabsf(ex.x) <= hx.x && fabsf(ey.x) <= hy.x));
-  k1 = front.y >= v.znear && (!(vz.y > r8.y) || (fabsf(ex.y) <= hx.y && fabsf(ey.y) <= hy.y));
+  const bool far0 = vz.x > r8.x, far1 = vz.y > r8.y;
+  k0 = front.x >= v.znear && (!far0 || (fabsf(ex.x) <= hx.x && fabsf(ey.x) <= hy.x));
+  k1 = front.y >= v.znear && (!far1 || (fabsf(ex.y) <= hx.y && fabsf(ey.y) <= hy.y));
+  size0 = far0 ? rho.x : 1.0f;
 }
 
 // Candidate pixel box of a sphere from the cull_lean bound (the exact
