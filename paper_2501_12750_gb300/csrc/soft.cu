@@ -15,9 +15,10 @@
 // sorts its list by (centre depth key, id) in shared memory (bucket pass plus
 // per-bucket insertion sort; in global memory for lists longer than shared
 // memory holds) and writes it back, then each warp walks the sorted list on
-// its own, staging 32 entries at a time with their per-sphere constants
-// (f / z_c, 1 / r and a bound on rho^2 that rejects most entries before any
-// square root or division).  The forward can leave per pixel its final
+// its own, staging 32 entries at a time -- those that can reach its pixels, in
+// pairs -- with their per-sphere constants (f / z_c, 1 / r and a bound on rho^2
+// that rejects most before any square root or division), and takes a pair per
+// step on the paired FP32 pipes.  The forward can leave per pixel its final
 // transmittance and last contributor (the state).  The backward either
 // reuses the forward's sorted lists (warps taking (tile, block) items from a
 // queue) or rebuilds them; it takes the last contributor and final
@@ -25,8 +26,8 @@
 // them, then walks back to front with the carry
 // R_i = alpha_{i+1} c_{i+1} + (1 - alpha_{i+1}) R_{i+1}, recovering T_i from
 // T_{i+1} / (1 - alpha_i) (alpha <= 0.99 keeps this safe), and accumulates
-// d/d(x, y, z, r) per sphere as a warp sum (a six-shuffle reduce-scatter)
-// and one 16-byte FP32 atomic per sphere and warp.
+// d/d(x, y, z, r) per sphere as a warp sum (one reduce-scatter of nine
+// shuffles per pair) and one 16-byte FP32 atomic per sphere and warp.
 #include "vtx_internal.h"
 
 namespace vtx {
@@ -39,45 +40,37 @@ constexpr int kSoftNT = 256;
 constexpr float kTStop = 1e-4f;
 constexpr float kAMax = 0.99f;
 
-// A tile entry as the per-pixel loop reads it from shared memory: the record's
-// projection terms plus the per-sphere constants of the soft terms, computed
-// once per entry when a warp stages it instead of once per pixel.
-struct __align__(16) SoftPrim {
-  float u0h, u0l, v0h, v0l;   // projected reference point (pixels), double-float
-  float k, dz, zr, rad;       // A per pixel at zr, zr - centre depth, reference depth, radius
-  float fz, inv_rad, eta, rej2;  // f / centre depth, 1 / rad, 0.05 rad, bound on rho^2 of a used sphere
-  float rpx2;                 // rej2 / k^2 (px^2) when dz = 0, else +inf: the pixel-distance pre-test
-  float pad[3];
+// The entries of a warp's window as its pixel loop reads them: pairs of consecutive kept entries (a, b), every field
+// of both side by side, so that a 16-byte read gives two fields of the pair ready for the paired FP32 pipes.  A field
+// of entry e (0 or 1) of pair p is at float 2 (field) + e of pair p's seven 16-byte words.
+enum SoftField {
+  kFU0h, kFU0l,      // projected reference point x (pixels), double-float, negated
+  kFV0h, kFV0l,      // and y
+  kFK, kFDz,         // A per pixel at zr; zr - centre depth
+  kFZr, kFRad,       // reference depth; radius
+  kFFz, kFInvRad,    // f / centre depth; 1 / radius
+  kFEta, kFRej2,     // 0.05 radius; bound on rho^2 of a used sphere
+  kFRpx2, kFPos,     // rej2 / k^2 (px^2) when dz = 0, else +inf: the pixel-distance pre-test; list position (int bits)
+  kSoftFields
 };
-static_assert(sizeof(SoftPrim) == 64, "SoftPrim is four 16-byte words");
-static_assert(kSoftNT * sizeof(SoftPrim) >= kSoftCap * sizeof(uint16_t), "the record windows hold the sort's offsets");
+static_assert(kSoftFields == 14, "seven 16-byte words");
+constexpr int kPairWords = kSoftFields / 2;  // 112 bytes: pairs start 28 banks apart, so staging stores conflict 2-way
+constexpr int kWindowBytes = 2048;           // per warp: 16 pairs and 32 atom ids
+static_assert(16 * kPairWords * 16 + 32 * 4 <= kWindowBytes, "a window");
+static_assert((kSoftNT / 32) * kWindowBytes >= kSoftCap * (int)sizeof(uint16_t), "the windows hold the sort's offsets");
 
-constexpr size_t kSoftSmem = kSoftCap * sizeof(unsigned long long) + kSoftNT * sizeof(SoftPrim);
+constexpr size_t kSoftSmem = kSoftCap * sizeof(unsigned long long) + (kSoftNT / 32) * kWindowBytes;
 
-__device__ __forceinline__ SoftPrim soft_prim(const PrimRec &p, float f) {
-  SoftPrim s;
-  s.u0h = p.u0h;
-  s.u0l = p.u0l;
-  s.v0h = p.v0h;
-  s.v0l = p.v0l;
-  s.k = p.k;
-  s.dz = p.dz;
-  s.zr = p.zr;
-  s.rad = p.rad;
-  s.fz = f / (p.zr - p.dz);
-  s.inv_rad = 1.0f / p.rad;
-  s.eta = 0.05f * p.rad;
-  // delta >= -4 px needs sqrt(rho^2) <= rad + 4 / fz; the bound is widened by
-  // 0.05 % so that rounding never drops a sphere the exact test keeps.
-  const float reach = p.rad + 4.0f / s.fz;
-  s.rej2 = reach * reach * 1.001f + 1e-6f;
-  // with dz = 0 the offset is o = k (dx, -dy, 0) and rho^2 >= |o|^2 / |u|^2 (Cauchy-Schwarz on its x, y part),
-  // so d^2 > rej2 |u|^2 / k^2 (d: pixel distance to the projected centre) rejects the sphere; the 0.1 % in
-  // rej2 covers the FP32 rounding of this quotient
-  s.rpx2 = p.dz == 0.0f ? s.rej2 / (p.k * p.k) : __int_as_float(0x7f800000);
-  s.pad[0] = s.pad[1] = s.pad[2] = 0.0f;
-  return s;
-}
+struct SoftWindow {
+  float4 *pair;     // [16][kPairWords]
+  uint32_t *id;     // [32] atom of each kept entry
+  __device__ __forceinline__ explicit SoftWindow(unsigned char *warp_base)
+      : pair(reinterpret_cast<float4 *>(warp_base)),
+        id(reinterpret_cast<uint32_t *>(warp_base + 16 * kPairWords * 16)) {}
+  __device__ __forceinline__ float *slot(int s) const {  // field f of kept entry s at slot(s)[2 f]
+    return reinterpret_cast<float *>(pair + (s >> 1) * kPairWords) + (s & 1);
+  }
+};
 
 // Per-pixel ray constants.
 struct SoftPix {
@@ -93,41 +86,75 @@ __device__ __forceinline__ SoftPix soft_pix(const ViewParams &v, int px, int py)
   return x;
 }
 
-struct SoftTerm {
-  float3 ov;        // ray origin minus centre (internal frame)
-  float sst;        // ray parameter of the closest approach, relative to zr
-  float rho2, rho2s, delta, sg, alpha, m, ism, si, t;
-  float3 n;         // internal frame
+// The soft terms of a pair of spheres for one pixel (x: sphere a, y: sphere b); false where delta < -4 px.
+struct SoftPair {
+  bool ha, hb;
+  int posa, posb;          // list positions
+  float2 ovx, ovy, dz;     // ray origin minus centre (internal frame)
+  float2 sst;              // ray parameter of the closest approach, relative to zr
+  float2 rho2s, irho;      // rho^2 + 1e-12 and its inverse root
+  float2 delta, sg, alpha, m, ism, t, nx, ny, nz;  // n: internal frame
+  float2 fz, inv_rad, eta, rad;
 };
 
-// The soft term of one sphere for one pixel; false when delta < -4 px.
-// nl2s = -log2(e) / sigma, so that exp(-delta / sigma) = 2^(delta nl2s).
-__device__ __forceinline__ bool soft_term(const SoftPrim &p, const SoftPix &x, float nl2s, SoftTerm &o) {
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// nl2s = -log2(e) / sigma, so that exp(-delta / sigma) = 2^(delta nl2s).  Every product-sum is one paired operation;
+// lane for lane they are the operations of one sphere's term.
+__device__ __forceinline__ void soft_pair(const float4 *w, const SoftPix &x, float nl2s, bool act, SoftPair &o) {
   const PixRay &r = x.r;
-  const float ox = __fsub_rn(__fsub_rn(r.pxc, p.u0h), p.u0l);
-  const float oy = __fsub_rn(__fsub_rn(r.pyc, p.v0h), p.v0l);
-  if (fmaf(ox, ox, oy * oy) > p.rpx2 * r.uu) return false;  // pixel-distance pre-test
-  o.ov = make_float3(__fmul_rn(p.k, ox), __fmul_rn(-p.k, oy), p.dz);  // local_o
-  const float ou = fmaf(o.ov.x, r.a, fmaf(o.ov.y, r.b, o.ov.z));
-  const float oo = fmaf(o.ov.x, o.ov.x, fmaf(o.ov.y, o.ov.y, o.ov.z * o.ov.z));
-  o.sst = -ou * x.inv_uu;
-  o.rho2 = fmaxf(fmaf(ou, o.sst, oo), 0.0f);  // |o|^2 - (o.u)^2 / |u|^2
-  if (o.rho2 > p.rej2) return false;
-  o.rho2s = o.rho2 + 1e-12f;
+  const float4 u = w[0], v = w[1], rp = w[6];
+  const float2 ox = __fadd2_rn(__fadd2_rn(bc2(r.pxc), make_float2(u.x, u.y)), make_float2(u.z, u.w));
+  const float2 oyn = __fadd2_rn(__fadd2_rn(make_float2(v.x, v.y), bc2(-r.pyc)), make_float2(v.z, v.w));  // minus oy
+  const float2 d2 = __ffma2_rn(ox, ox, __fmul2_rn(oyn, oyn));
+  const float2 lim = __fmul2_rn(make_float2(rp.x, rp.y), bc2(r.uu));
+  o.ha = act && !(d2.x > lim.x);  // pixel-distance pre-test
+  o.hb = act && !(d2.y > lim.y);
+  if (!(o.ha || o.hb)) return;
+  o.posa = __float_as_int(rp.z);
+  o.posb = __float_as_int(rp.w);
+  const float4 kd = w[2], zr = w[3], fi = w[4], er = w[5];
+  const float2 k = make_float2(kd.x, kd.y);
+  o.dz = make_float2(kd.z, kd.w);
+  o.rad = make_float2(zr.z, zr.w);
+  o.fz = make_float2(fi.x, fi.y);
+  o.inv_rad = make_float2(fi.z, fi.w);
+  o.eta = make_float2(er.x, er.y);
+  o.ovx = __fmul2_rn(k, ox);  // local_o
+  o.ovy = __fmul2_rn(k, oyn);
+  const float2 ou = __ffma2_rn(o.ovx, bc2(r.a), __ffma2_rn(o.ovy, bc2(r.b), o.dz));
+  const float2 oo = __ffma2_rn(o.ovx, o.ovx, __ffma2_rn(o.ovy, o.ovy, __fmul2_rn(o.dz, o.dz)));
+  o.sst = __fmul2_rn(ou, bc2(-x.inv_uu));
+  float2 rho2 = __ffma2_rn(ou, o.sst, oo);  // |o|^2 - (o.u)^2 / |u|^2
+  rho2 = make_float2(fmaxf(rho2.x, 0.0f), fmaxf(rho2.y, 0.0f));
+  o.ha = o.ha && !(rho2.x > er.z);
+  o.hb = o.hb && !(rho2.y > er.w);
+  o.rho2s = __fadd2_rn(rho2, bc2(1e-12f));
   // hardware approximations (relative errors near 1e-7; the outputs' tolerance is 5e-5): sqrt as x rsqrt(x),
   // the sigmoid through ex2.approx and rcp.approx
-  o.delta = (p.rad - o.rho2s * rsqrtf(o.rho2s)) * p.fz;
-  if (!(o.delta >= -4.0f)) return false;
-  o.sg = rcp_approx(1.0f + exp2_approx(o.delta * nl2s));
-  o.alpha = fminf(kAMax, o.sg);
-  o.m = fmaxf(fmaf(p.rad, p.rad, -o.rho2), 0.0f);
-  const float m2 = fmaf(p.eta, p.eta, o.m);
-  o.ism = rsqrtf(m2);
-  o.si = fmaf(-(m2 * o.ism - p.eta), x.inv_un, o.sst);  // smoothed entry, relative to zr
-  o.t = p.zr + o.si;
-  o.n = make_float3(fmaf(o.si, r.a, o.ov.x) * p.inv_rad, fmaf(o.si, r.b, o.ov.y) * p.inv_rad,
-                    (o.ov.z + o.si) * p.inv_rad);
-  return true;
+  o.irho = make_float2(rsqrt_approx(o.rho2s.x), rsqrt_approx(o.rho2s.y));
+  o.delta = __fmul2_rn(__ffma2_rn(neg2(o.rho2s), o.irho, o.rad), o.fz);
+  o.ha = o.ha && o.delta.x >= -4.0f;
+  o.hb = o.hb && o.delta.y >= -4.0f;
+  const float2 ex = __fmul2_rn(o.delta, bc2(nl2s));
+  const float2 den = __fadd2_rn(bc2(1.0f), make_float2(exp2_approx(ex.x), exp2_approx(ex.y)));
+  o.sg = make_float2(rcp_approx(den.x), rcp_approx(den.y));
+  o.alpha = make_float2(fminf(kAMax, o.sg.x), fminf(kAMax, o.sg.y));
+  const float2 m = __ffma2_rn(o.rad, o.rad, neg2(rho2));
+  o.m = make_float2(fmaxf(m.x, 0.0f), fmaxf(m.y, 0.0f));
+  const float2 m2 = __ffma2_rn(o.eta, o.eta, o.m);
+  o.ism = make_float2(rsqrt_approx(m2.x), rsqrt_approx(m2.y));
+  const float2 g = __ffma2_rn(m2, o.ism, neg2(o.eta));
+  const float2 si = __ffma2_rn(neg2(g), bc2(x.inv_un), o.sst);  // smoothed entry, relative to zr
+  o.t = __fadd2_rn(make_float2(zr.x, zr.y), si);
+  o.nx = __fmul2_rn(__ffma2_rn(si, bc2(r.a), o.ovx), o.inv_rad);
+  o.ny = __fmul2_rn(__ffma2_rn(si, bc2(r.b), o.ovy), o.inv_rad);
+  o.nz = __fmul2_rn(__fadd2_rn(o.dz, si), o.inv_rad);
 }
 
 struct SoftTile {
@@ -330,41 +357,81 @@ __device__ __forceinline__ bool soft_load(const Geometry &g, long long gt, unsig
 // disc of that radius misses the bounding rectangle of the active lanes'
 // pixel centres are dropped from the returned mask; the radius is widened
 // (0.01 % plus 1e-3 px plus 2e-7 of the coordinates) to cover FP32 rounding.
-// The record index of entry j of the tile's list (0 past its end); loaded one window ahead of its use.
+// The record index of entry j of the tile's list (0 outside it); loaded two windows ahead of its use, and the record
+// itself brought into L1 one window ahead.
 __device__ __forceinline__ uint32_t soft_rec_index(const Geometry &g, const uint32_t *__restrict__ rec_of,
                                                    const SoftTile &T, int j) {
   return (j >= 0 && j < T.m) ? rec_of[(long long)T.img * g.n_atoms + (uint32_t)T.list[j]] : 0u;
 }
+__device__ __forceinline__ void soft_prefetch(const PrimRec *__restrict__ recs, uint32_t ridx) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(recs + ridx));
+}
 
-__device__ __forceinline__ unsigned soft_stage(const PrimRec *__restrict__ recs, uint32_t ridx, const SoftTile &T,
-                                               int c0, float f, SoftPrim *s_w, unsigned am, float col0, float row0,
-                                               float uu_max) {
+// Stages the window [c0, c0 + 32): the entries that lanes `am` can use (and lists before `end`), in order, as pairs;
+// returns their number.  An odd last entry is paired with one that no pixel accepts.
+__device__ __forceinline__ int soft_stage(const PrimRec *__restrict__ recs, uint32_t ridx, const SoftTile &T, int c0,
+                                          int end, float f, const SoftWindow &W, unsigned am, float col0, float row0,
+                                          float uu_max) {
   const int lane = threadIdx.x & 31;
   const int j = c0 + lane;
   bool keep = false;
-  if (j < T.m) {
-    const SoftPrim sp = soft_prim(recs[ridx], f);
-    s_w[lane] = sp;
+  PrimRec p;
+  float fz = 0.0f, rej2 = 0.0f;
+  if (j < end) {
+    p = recs[ridx];
+    fz = f / (p.zr - p.dz);
+    // delta >= -4 px needs sqrt(rho^2) <= rad + 4 / fz; the bound is widened by
+    // 0.05 % so that rounding never drops a sphere the exact test keeps.
+    const float reach = p.rad + 4.0f / fz;
+    rej2 = reach * reach * 1.001f + 1e-6f;
     const unsigned cols = (am | (am >> 8) | (am >> 16) | (am >> 24)) & 0xffu;
     const unsigned rows = ((am & 0xffu) ? 1u : 0u) | ((am & 0xff00u) ? 2u : 0u) | ((am & 0xff0000u) ? 4u : 0u) |
                           ((am & 0xff000000u) ? 8u : 0u);
     const float rx0 = col0 + (float)(__ffs(cols) - 1), rx1 = col0 + (float)(31 - __clz(cols));
     const float ry0 = row0 + (float)(__ffs(rows) - 1), ry1 = row0 + (float)(31 - __clz(rows));
-    const float cu = sp.u0h + sp.u0l, cv = sp.v0h + sp.v0l;
+    const float cu = p.u0h + p.u0l, cv = p.v0h + p.v0l;
     const float dx = fmaxf(fmaxf(rx0 - cu, cu - rx1), 0.0f);
     const float dy = fmaxf(fmaxf(ry0 - cv, cv - ry1), 0.0f);
-    const float r2 = sp.rej2 * uu_max;  // approximate root and quotient: the 0.01 % widening covers their error
-    const float rt = __fdividef(r2 * rsqrtf(r2), sp.k) * 1.0001f + 1e-3f + 2e-7f * (fabsf(cu) + fabsf(cv));
-    keep = sp.dz != 0.0f || !(dx * dx + dy * dy > rt * rt);
+    const float r2 = rej2 * uu_max;  // approximate root and quotient: the 0.01 % widening covers their error
+    const float rt = __fdividef(r2 * rsqrtf(r2), p.k) * 1.0001f + 1e-3f + 2e-7f * (fabsf(cu) + fabsf(cv));
+    keep = p.dz != 0.0f || !(dx * dx + dy * dy > rt * rt);
   }
-  return __ballot_sync(0xffffffffu, keep);
+  const unsigned m = __ballot_sync(0xffffffffu, keep);
+  const int n = __popc(m);
+  const int at = __popc(m & ((1u << lane) - 1u));
+  if (keep) {
+    float *s = W.slot(at);
+    s[2 * kFU0h] = -p.u0h;
+    s[2 * kFU0l] = -p.u0l;
+    s[2 * kFV0h] = p.v0h;
+    s[2 * kFV0l] = p.v0l;
+    s[2 * kFK] = p.k;
+    s[2 * kFDz] = p.dz;
+    s[2 * kFZr] = p.zr;
+    s[2 * kFRad] = p.rad;
+    s[2 * kFFz] = fz;
+    s[2 * kFInvRad] = 1.0f / p.rad;
+    s[2 * kFEta] = 0.05f * p.rad;
+    s[2 * kFRej2] = rej2;
+    // with dz = 0 the offset is o = k (dx, -dy, 0) and rho^2 >= |o|^2 / |u|^2 (Cauchy-Schwarz on its x, y part),
+    // so d^2 > rej2 |u|^2 / k^2 (d: pixel distance to the projected centre) rejects the sphere; the 0.1 % in
+    // rej2 covers the FP32 rounding of this quotient
+    s[2 * kFRpx2] = p.dz == 0.0f ? rej2 / (p.k * p.k) : __int_as_float(0x7f800000);
+    s[2 * kFPos] = __int_as_float(j);
+    W.id[at] = p.id;
+  }
+  if ((n & 1) && lane < kSoftFields) W.slot(n)[2 * lane] = lane == kFRpx2 ? -1.0f : 0.0f;
+  __syncwarp();
+  return n;
 }
 
 // state (optional, [n_img][H][W]): per pixel the final transmittance (float
 // bits) and 1 + the sorted-list position of its last contributor (0: none),
 // which lets the backward pass start its back-to-front walk directly.
+// Forward CTAs per SM: 3 (80 registers); 20,000 atoms from 16 views at 512x512: forward 284 us at 3, 304 at 4 (spills),
+// 331 at 2.  One entry per step on the scalar pipes took 309 us (4 CTAs).
 #ifndef VTX_SOFT_FWD_MINB
-#define VTX_SOFT_FWD_MINB 4
+#define VTX_SOFT_FWD_MINB 3
 #endif
 // One tile of the forward pass (called by every thread of the CTA).
 __device__ __forceinline__ void soft_fwd_tile(const Geometry &g, long long gt, const PrimRec *__restrict__ recs,
@@ -372,10 +439,11 @@ __device__ __forceinline__ void soft_fwd_tile(const Geometry &g, long long gt, c
                                               unsigned long long cap_entries, const uint32_t *__restrict__ tile_count,
                                               const uint32_t *__restrict__ tile_start, Status *status, float *cov,
                                               float *dep, float *nrm, uint2 *state, unsigned long long *s_e,
-                                              SoftPrim *s_w) {
+                                              unsigned char *s_win) {
   SoftTile T;
   const bool any = soft_load(g, gt, entries, cap_entries, tile_count, tile_start, status, s_e,
-                             reinterpret_cast<uint16_t *>(s_w - (threadIdx.x & ~31)), T, true, false);
+                             reinterpret_cast<uint16_t *>(s_win), T, true, false);
+  const SoftWindow W(s_win + (threadIdx.x >> 5) * kWindowBytes);
   const ViewParams &v = g.views[T.img % g.n_views];
   const SoftPix x = soft_pix(v, T.px, T.py);
   const float inv_sigma = 1.0f / g.sigma;
@@ -389,29 +457,42 @@ __device__ __forceinline__ void soft_fwd_tile(const Geometry &g, long long gt, c
   unsigned used = 0u;
   bool done = !T.inside;
   if (any) {
-    uint32_t ridx = soft_rec_index(g, rec_of, T, lane);
+    uint32_t ridx = soft_rec_index(g, rec_of, T, lane), next = soft_rec_index(g, rec_of, T, 32 + lane);
     for (int c0 = 0; c0 < T.m; c0 += 32) {
       const unsigned am = __ballot_sync(0xffffffffu, !done);
       if (am == 0u) break;
-      const uint32_t next = soft_rec_index(g, rec_of, T, c0 + 32 + lane);  // the next window's, in flight now
-      const unsigned keep = soft_stage(recs, ridx, T, c0, v.f, s_w, am, col0, row0, uu_max);
+      const uint32_t next2 = soft_rec_index(g, rec_of, T, c0 + 64 + lane);  // in flight during this window
+      soft_prefetch(recs, next);
+      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, col0, row0, uu_max);
       ridx = next;
-      __syncwarp();
-      for (unsigned b = keep; b != 0u; b &= b - 1u) {
-        if (done) continue;
-        const int q = __ffs(b) - 1;
-        SoftTerm o;
-        if (!soft_term(s_w[q], x, nl2s, o)) continue;
-        const float w = o.alpha * Tr;
-        A += w;
-        D = fmaf(w, o.t, D);
-        N0 = fmaf(w, o.n.x, N0);
-        N1 = fmaf(w, o.n.y, N1);
-        N2 = fmaf(-w, o.n.z, N2);
-        Tr *= 1.0f - o.alpha;
-        last = c0 + q;
-        ++used;
-        if (Tr < kTStop) done = true;
+      next = next2;
+      for (int q = 0; q < n; q += 2) {
+        SoftPair o;
+        soft_pair(W.pair + (q >> 1) * kPairWords, x, nl2s, !done, o);
+        if (o.ha) {
+          const float w = o.alpha.x * Tr;
+          A += w;
+          D = fmaf(w, o.t.x, D);
+          N0 = fmaf(w, o.nx.x, N0);
+          N1 = fmaf(w, o.ny.x, N1);
+          N2 = fmaf(-w, o.nz.x, N2);
+          Tr *= 1.0f - o.alpha.x;
+          last = o.posa;
+          ++used;
+          if (Tr < kTStop) done = true;
+        }
+        if (o.hb && !done) {
+          const float w = o.alpha.y * Tr;
+          A += w;
+          D = fmaf(w, o.t.y, D);
+          N0 = fmaf(w, o.nx.y, N0);
+          N1 = fmaf(w, o.ny.y, N1);
+          N2 = fmaf(-w, o.nz.y, N2);
+          Tr *= 1.0f - o.alpha.y;
+          last = o.posb;
+          ++used;
+          if (Tr < kTStop) done = true;
+        }
       }
       __syncwarp();
     }
@@ -448,45 +529,39 @@ __global__ __launch_bounds__(kSoftNT, VTX_SOFT_FWD_MINB) void k_soft_fwd(Geometr
                                                       float *cov, float *dep, float *nrm, uint2 *state) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long *s_e = reinterpret_cast<unsigned long long *>(smem);
-  SoftPrim *s_w = reinterpret_cast<SoftPrim *>(smem + kSoftCap * sizeof(unsigned long long)) + (threadIdx.x & ~31);
+  unsigned char *s_win = smem + kSoftCap * sizeof(unsigned long long);
   // every tile, longest list first when the scan listed them all (empty tiles last), else in index order
   const long long gt = tile_list ? (long long)tile_list[blockIdx.x] : (long long)blockIdx.x;
   soft_fwd_tile(g, gt, recs, rec_of, entries, cap_entries, tile_count, tile_start, status, cov, dep, nrm, state, s_e,
-                s_w);
+                s_win);
 }
 
-// Sum of four per-lane values over the warp, scattered: lanes 0, 8, 16 and 24
-// receive the sums of a0, a1, a2 and a3 (six shuffles instead of twenty).
-__device__ __forceinline__ float warp_sum4_scatter(float a0, float a1, float a2, float a3, int lane) {
-  const bool hi16 = (lane & 16) != 0;
-  float k0 = hi16 ? a2 : a0, k1 = hi16 ? a3 : a1;
-  const float s0 = hi16 ? a0 : a2, s1 = hi16 ? a1 : a3;
-  k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-  k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-  const bool hi8 = (lane & 8) != 0;
-  float k = hi8 ? k1 : k0;
-  k += __shfl_xor_sync(0xffffffffu, hi8 ? k0 : k1, 8);
-  k += __shfl_xor_sync(0xffffffffu, k, 4);
-  k += __shfl_xor_sync(0xffffffffu, k, 2);
-  k += __shfl_xor_sync(0xffffffffu, k, 1);
-  return k;
+// Sums over the warp of four per-lane values of sphere a and four of sphere b, scattered: lanes 0, 4, 8, 12 receive
+// a's sums in order and lanes 16, 20, 24, 28 b's (nine shuffles).
+__device__ __forceinline__ float warp_sum8_scatter(const float2 (&v)[4], int lane) {
+  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
+  float k[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    k[c] = h16 ? v[c].y : v[c].x;
+    k[c] += __shfl_xor_sync(0xffffffffu, h16 ? v[c].x : v[c].y, 16);
+  }
+  float p0 = h8 ? k[2] : k[0], p1 = h8 ? k[3] : k[1];
+  p0 += __shfl_xor_sync(0xffffffffu, h8 ? k[0] : k[2], 8);
+  p1 += __shfl_xor_sync(0xffffffffu, h8 ? k[1] : k[3], 8);
+  float s = h4 ? p1 : p0;
+  s += __shfl_xor_sync(0xffffffffu, h4 ? p0 : p1, 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
 }
-
-// One tile of the backward pass (called by every thread of the CTA).
-__device__ __forceinline__ void soft_bwd_tile(const Geometry &g, long long gt, const PrimRec *__restrict__ recs,
-                                              const uint32_t *__restrict__ rec_of, unsigned long long *entries,
-                                              unsigned long long cap_entries, const uint32_t *__restrict__ tile_count,
-                                              const uint32_t *__restrict__ tile_start, Status *status,
-                                              const float *gcov, const float *gdep, const float *gnrm,
-                                              const uint2 *__restrict__ state, float *grad, unsigned long long *s_e,
-                                              SoftPrim *s_w, bool presorted);
 
 // The backward of one warp: its 8x4 pixel block wblk of tile T, whose sorted list T.list is in shared or
-// global memory; s_w is the warp's 32-entry window.
+// global memory; W is the warp's window.
 __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile &T, int wblk,
                                               const PrimRec *__restrict__ recs, const uint32_t *__restrict__ rec_of,
                                               const float *gcov, const float *gdep, const float *gnrm,
-                                              const uint2 *__restrict__ state, float *grad, SoftPrim *s_w) {
+                                              const uint2 *__restrict__ state, float *grad, const SoftWindow &W) {
   const ViewParams &v = g.views[T.img % g.n_views];
   const SoftPix x = soft_pix(v, T.px, T.py);
   const PixRay &r = x.r;
@@ -523,100 +598,128 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
     done = true;
   }
   const int lane = threadIdx.x & 31;
-  uint32_t ridx = soft_rec_index(g, rec_of, T, lane);  // lane stages entry c0 + lane for the whole warp
-  for (int c0 = 0; c0 < T.m && !__all_sync(0xffffffffu, done); c0 += 32) {
-    const unsigned am = __ballot_sync(0xffffffffu, !done);
-    if (am == 0u) break;
-    const uint32_t next = soft_rec_index(g, rec_of, T, c0 + 32 + lane);
-    const unsigned keep = soft_stage(recs, ridx, T, c0, v.f, s_w, am, col0, row0, uu_max);
-    ridx = next;
-    __syncwarp();
-    for (unsigned b = keep; b != 0u; b &= b - 1u) {
-      if (done) continue;
-      const int q = __ffs(b) - 1;
-      SoftTerm o;
-      if (!soft_term(s_w[q], x, nl2s, o)) continue;
-      Tr *= 1.0f - o.alpha;
-      last = c0 + q;
-      if (Tr < kTStop) done = true;
+  if (!__all_sync(0xffffffffu, done)) {
+    uint32_t ridx = soft_rec_index(g, rec_of, T, lane), next = soft_rec_index(g, rec_of, T, 32 + lane);
+    for (int c0 = 0; c0 < T.m; c0 += 32) {
+      const unsigned am = __ballot_sync(0xffffffffu, !done);
+      if (am == 0u) break;
+      const uint32_t next2 = soft_rec_index(g, rec_of, T, c0 + 64 + lane);
+      soft_prefetch(recs, next);
+      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, col0, row0, uu_max);
+      ridx = next;
+      next = next2;
+      for (int q = 0; q < n; q += 2) {
+        SoftPair o;
+        soft_pair(W.pair + (q >> 1) * kPairWords, x, nl2s, !done, o);
+        if (o.ha) {
+          Tr *= 1.0f - o.alpha.x;
+          last = o.posa;
+          if (Tr < kTStop) done = true;
+        }
+        if (o.hb && !done) {
+          Tr *= 1.0f - o.alpha.y;
+          last = o.posb;
+          if (Tr < kTStop) done = true;
+        }
+      }
+      __syncwarp();
     }
-    __syncwarp();
   }
   const int wlast = __reduce_max_sync(0xffffffffu, last);
   if (wlast < 0) return;
-  // pass 2: back to front; per-sphere sums leave the warp as one 16-byte atomic
+  // pass 2: back to front, a pair per step, its later sphere first; per-sphere sums leave the warp as one 16-byte
+  // atomic
   const float ugn0 = fmaf(r.a, gN.x, fmaf(r.b, gN.y, gN.z));
   float R = 0.0f, Tc = Tr;
-  ridx = soft_rec_index(g, rec_of, T, (wlast / 32) * 32 + lane);
-  for (int c0 = (wlast / 32) * 32; c0 >= 0; c0 -= 32) {
+  const int w0 = (wlast / 32) * 32;
+  uint32_t ridx = soft_rec_index(g, rec_of, T, w0 + lane), prev = soft_rec_index(g, rec_of, T, w0 - 32 + lane);
+  for (int c0 = w0; c0 >= 0; c0 -= 32) {
     const unsigned am = __ballot_sync(0xffffffffu, last >= c0);
-    const uint32_t prev = soft_rec_index(g, rec_of, T, c0 - 32 + lane);  // the previous window's, in flight now
-    if (am == 0u) {
-      ridx = prev;
-      continue;
-    }
-    __syncwarp();
-    unsigned keep = soft_stage(recs, ridx, T, c0, v.f, s_w, am, col0, row0, uu_max);
+    const uint32_t prev2 = soft_rec_index(g, rec_of, T, c0 - 64 + lane);  // in flight during this window
+    soft_prefetch(recs, prev);
+    const uint32_t cur = ridx;
     ridx = prev;
-    if (wlast - c0 < 31) keep &= (2u << (wlast - c0)) - 1u;
-    __syncwarp();
-    while (keep != 0u) {
-      const int q = 31 - __clz(keep);
-      keep &= ~(1u << q);
-      const SoftPrim &pr = s_w[q];
-      float gx = 0.0f, gy = 0.0f, gz = 0.0f, grr = 0.0f;
-      SoftTerm o;
-      if (c0 + q <= last && soft_term(pr, x, nl2s, o)) {
-        const float Ti = Tc / (1.0f - o.alpha);
-        const float w = o.alpha * Ti;
-        const float ci = gA + gD * o.t + gN.x * o.n.x + gN.y * o.n.y + gN.z * o.n.z;
-        const float dalpha = Ti * (ci - R);
-        R = o.alpha * ci + (1.0f - o.alpha) * R;
-        Tc = Ti;
-        const float dadd = o.sg < kAMax ? o.sg * (1.0f - o.sg) * inv_sigma : 0.0f;
-        const float dd = dalpha * dadd;
-        // closest-approach offset q = C - (o + s u), |q|^2 = rho^2
-        const float3 qv = make_float3(-fmaf(o.sst, r.a, o.ov.x), -fmaf(o.sst, r.b, o.ov.y), -(o.ov.z + o.sst));
-        const float ddf = dd * pr.fz;
-        const float isq = rsqrtf(o.rho2s);
-        // delta(C, r)
-        gx = -ddf * qv.x * isq;
-        gy = -ddf * qv.y * isq;
-        gz = -ddf * qv.z * isq - ddf * o.delta * v.inv_f;  // d delta / d zc = -delta / zc = -delta fz / f
-        grr = ddf;
-        // t_i(C, r) and n_i = (t_i u - C) / r
-        float c2 = 0.0f, dg_dr = 0.0f;
-        if (o.m > 0.0f) {
-          c2 = -o.ism * x.inv_un;                       // 2 (dg / drho^2) / |u|
-          dg_dr = fmaf(0.05f, pr.eta, pr.rad) * o.ism - 0.05f;
+    prev = prev2;
+    if (am == 0u) continue;
+    const int n = soft_stage(recs, cur, T, c0, wlast + 1, v.f, W, am, col0, row0, uu_max);
+    for (int q = (n - 1) & ~1; q >= 0; q -= 2) {
+      const float4 *pw = W.pair + (q >> 1) * kPairWords;
+      float2 gr[4];  // d/d(x, y, z) in the internal frame and d/dr, of spheres a and b
+      bool nz = false;
+      SoftPair o;
+      soft_pair(pw, x, nl2s, c0 <= last, o);
+      o.ha = o.ha && o.posa <= last;
+      o.hb = o.hb && o.posb <= last;
+      if (o.ha || o.hb) {
+        // c_i, then back to front through the pair: b, then a
+        float2 ci = __ffma2_rn(bc2(gD), o.t, bc2(gA));
+        const float2 gn = __ffma2_rn(bc2(gN.x), o.nx, __ffma2_rn(bc2(gN.y), o.ny, __fmul2_rn(bc2(gN.z), o.nz)));
+        ci = __fadd2_rn(ci, gn);
+        float2 w = make_float2(0.0f, 0.0f), dal = w;
+        if (o.hb) {
+          const float Ti = Tc / (1.0f - o.alpha.y);
+          w.y = o.alpha.y * Ti;
+          dal.y = Ti * (ci.y - R);
+          R = o.alpha.y * ci.y + (1.0f - o.alpha.y) * R;
+          Tc = Ti;
         }
-        const float dtx = fmaf(r.a, x.inv_uu, -c2 * qv.x);
-        const float dty = fmaf(r.b, x.inv_uu, -c2 * qv.y);
-        const float dtz = x.inv_uu - c2 * qv.z;
-        const float dtr = -dg_dr * x.inv_un;
-        const float ut = w * gD;
-        const float ugn = w * ugn0;
-        const float inv = pr.inv_rad;
-        gx += ut * dtx + (dtx * ugn - w * gN.x) * inv;
-        gy += ut * dty + (dty * ugn - w * gN.y) * inv;
-        gz += ut * dtz + (dtz * ugn - w * gN.z) * inv;
-        grr += ut * dtr + (ugn * dtr - w * (gN.x * o.n.x + gN.y * o.n.y + gN.z * o.n.z)) * inv;
+        if (o.ha) {
+          const float Ti = Tc / (1.0f - o.alpha.x);
+          w.x = o.alpha.x * Ti;
+          dal.x = Ti * (ci.x - R);
+          R = o.alpha.x * ci.x + (1.0f - o.alpha.x) * R;
+          Tc = Ti;
+        }
+        float2 dadd = __fmul2_rn(__fmul2_rn(o.sg, __fadd2_rn(bc2(1.0f), neg2(o.sg))), bc2(inv_sigma));
+        dadd = make_float2(o.sg.x < kAMax ? dadd.x : 0.0f, o.sg.y < kAMax ? dadd.y : 0.0f);
+        const float2 ddf = __fmul2_rn(__fmul2_rn(dal, dadd), o.fz);
+        // closest-approach offset minus q = (o + s u) - C, |q|^2 = rho^2
+        const float2 qx = __ffma2_rn(o.sst, bc2(r.a), o.ovx), qy = __ffma2_rn(o.sst, bc2(r.b), o.ovy);
+        const float2 qz = __fadd2_rn(o.dz, o.sst);
+        // delta(C, r): d delta / dC = minus q's offset over rho, d delta / d zc = -delta / zc = -delta fz / f
+        const float2 dq = __fmul2_rn(ddf, o.irho);
+        gr[0] = __fmul2_rn(dq, qx);
+        gr[1] = __fmul2_rn(dq, qy);
+        gr[2] = __ffma2_rn(dq, qz, __fmul2_rn(__fmul2_rn(neg2(ddf), o.delta), bc2(v.inv_f)));
+        gr[3] = ddf;
+        // t_i(C, r) and n_i = (t_i u - C) / r
+        const float2 c2 = make_float2(o.m.x > 0.0f ? -o.ism.x * x.inv_un : 0.0f,
+                                      o.m.y > 0.0f ? -o.ism.y * x.inv_un : 0.0f);  // 2 (dg / drho^2) / |u|
+        float2 dg = __ffma2_rn(__ffma2_rn(bc2(0.05f), o.eta, o.rad), o.ism, bc2(-0.05f));
+        dg = make_float2(o.m.x > 0.0f ? dg.x : 0.0f, o.m.y > 0.0f ? dg.y : 0.0f);
+        const float2 dtx = __ffma2_rn(c2, qx, bc2(r.a * x.inv_uu)), dty = __ffma2_rn(c2, qy, bc2(r.b * x.inv_uu));
+        const float2 dtz = __ffma2_rn(c2, qz, bc2(x.inv_uu)), dtr = __fmul2_rn(neg2(dg), bc2(x.inv_un));
+        const float2 ut = __fmul2_rn(w, bc2(gD));
+        // through the depth and the normal alike: (w gD + w (u.gN) / r) dt, and -w gN / r for the centre itself
+        const float2 wr = __fmul2_rn(w, o.inv_rad), s = __ffma2_rn(wr, bc2(ugn0), ut), mwr = neg2(wr);
+        gr[0] = __fadd2_rn(gr[0], __ffma2_rn(s, dtx, __fmul2_rn(mwr, bc2(gN.x))));
+        gr[1] = __fadd2_rn(gr[1], __ffma2_rn(s, dty, __fmul2_rn(mwr, bc2(gN.y))));
+        gr[2] = __fadd2_rn(gr[2], __ffma2_rn(s, dtz, __fmul2_rn(mwr, bc2(gN.z))));
+        gr[3] = __fadd2_rn(gr[3], __ffma2_rn(s, dtr, __fmul2_rn(mwr, gn)));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) gr[c] = make_float2(o.ha ? gr[c].x : 0.0f, o.hb ? gr[c].y : 0.0f);
+        nz = gr[0].x != 0.0f || gr[1].x != 0.0f || gr[2].x != 0.0f || gr[3].x != 0.0f || gr[0].y != 0.0f ||
+             gr[1].y != 0.0f || gr[2].y != 0.0f || gr[3].y != 0.0f;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) gr[c] = make_float2(0.0f, 0.0f);
       }
-      const bool nz = gx != 0.0f || gy != 0.0f || gz != 0.0f || grr != 0.0f;
       if (__any_sync(0xffffffffu, nz)) {
-        const float sum = warp_sum4_scatter(gx, gy, gz, grr, lane);
-        const float sy = __shfl_sync(0xffffffffu, sum, 8);
-        const float sz = __shfl_sync(0xffffffffu, sum, 16);
-        const float sr = __shfl_sync(0xffffffffu, sum, 24);
-        if (lane == 0) {
-          const uint32_t id = (uint32_t)T.list[c0 + q];
+        const float sum = warp_sum8_scatter(gr, lane);
+        const float sy = __shfl_down_sync(0xffffffffu, sum, 4);
+        const float sz = __shfl_down_sync(0xffffffffu, sum, 8);
+        const float sr = __shfl_down_sync(0xffffffffu, sum, 12);
+        const int e = q + (lane >> 4);
+        if ((lane & 15) == 0 && e < n) {
           const float4 wv = make_float4(v.R[0] * sum + v.U[0] * sy + v.F[0] * sz,
                                         v.R[1] * sum + v.U[1] * sy + v.F[1] * sz,
                                         v.R[2] * sum + v.U[2] * sy + v.F[2] * sz, sr);
-          atomicAdd(reinterpret_cast<float4 *>(grad) + id, wv);
+          if (wv.x != 0.0f || wv.y != 0.0f || wv.z != 0.0f || wv.w != 0.0f)
+            atomicAdd(reinterpret_cast<float4 *>(grad) + W.id[e], wv);
         }
       }
     }
+    __syncwarp();  // every lane is done with the window before it is refilled
   }
 }
 
@@ -626,12 +729,13 @@ __device__ __forceinline__ void soft_bwd_tile(const Geometry &g, long long gt, c
                                               const uint32_t *__restrict__ tile_start, Status *status,
                                               const float *gcov, const float *gdep, const float *gnrm,
                                               const uint2 *__restrict__ state, float *grad, unsigned long long *s_e,
-                                              SoftPrim *s_w, bool presorted) {
+                                              unsigned char *s_win, bool presorted) {
   SoftTile T;
   if (!soft_load(g, gt, entries, cap_entries, tile_count, tile_start, status, s_e,
-                 reinterpret_cast<uint16_t *>(s_w - (threadIdx.x & ~31)), T, false, presorted))
+                 reinterpret_cast<uint16_t *>(s_win), T, false, presorted))
     return;
-  soft_bwd_walk(g, T, (int)(threadIdx.x >> 5), recs, rec_of, gcov, gdep, gnrm, state, grad, s_w);
+  const int wid = (int)(threadIdx.x >> 5);
+  soft_bwd_walk(g, T, wid, recs, rec_of, gcov, gdep, gnrm, state, grad, SoftWindow(s_win + wid * kWindowBytes));
 }
 
 // Persistent backward over the non-empty tiles (as the forward).
@@ -646,7 +750,7 @@ __global__ __launch_bounds__(kSoftNT) void k_soft_bwd(Geometry g, const PrimRec 
                                                       const uint2 *__restrict__ state, float *grad, int presorted) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned long long *s_e = reinterpret_cast<unsigned long long *>(smem);
-  SoftPrim *s_w = reinterpret_cast<SoftPrim *>(smem + kSoftCap * sizeof(unsigned long long)) + (threadIdx.x & ~31);
+  unsigned char *s_win = smem + kSoftCap * sizeof(unsigned long long);
   __shared__ uint32_t s_li;
   const uint32_t n_list = status->n_list;
   for (;;) {
@@ -655,7 +759,7 @@ __global__ __launch_bounds__(kSoftNT) void k_soft_bwd(Geometry g, const PrimRec 
     const uint32_t li = s_li;
     if (li >= n_list) break;
     soft_bwd_tile(g, tile_list[li], recs, rec_of, entries, cap_entries, tile_count, tile_start, status, gcov, gdep,
-                  gnrm, state, grad, s_e, s_w, presorted != 0);
+                  gnrm, state, grad, s_e, s_win, presorted != 0);
     __syncthreads();
   }
 }
@@ -664,7 +768,13 @@ __global__ __launch_bounds__(kSoftNT) void k_soft_bwd(Geometry g, const PrimRec 
 // items from a queue -- the non-empty tiles longest first, eight blocks each -- and walks the tile's list in
 // global memory on its own.  No step needs the whole tile, so there is no block barrier: a warp that finishes
 // its block early takes the next item instead of waiting for the tile's slowest warp.
-__global__ __launch_bounds__(kSoftNT, 4) void k_soft_bwd_warps(Geometry g, const PrimRec *__restrict__ recs,
+// Bound by issue and, on small problems, by each warp's chain of pairs.  Two CTAs per SM (120 registers, nothing
+// spilled): 20,000 atoms from 16 views at 512x512 307 us, 1,200 atoms from 2 views at 200x136 138 us; 3 CTAs 310 / 161,
+// 4 CTAs 368 / 181.  One entry per step, its atom id read from the list in global memory, took 362 / 179 us.
+#ifndef VTX_SOFT_BWD_MINB
+#define VTX_SOFT_BWD_MINB 2
+#endif
+__global__ __launch_bounds__(kSoftNT, VTX_SOFT_BWD_MINB) void k_soft_bwd_warps(Geometry g, const PrimRec *__restrict__ recs,
                                                             const uint32_t *__restrict__ rec_of,
                                                             const unsigned long long *__restrict__ entries,
                                                             unsigned long long cap_entries,
@@ -673,8 +783,8 @@ __global__ __launch_bounds__(kSoftNT, 4) void k_soft_bwd_warps(Geometry g, const
                                                             const uint32_t *__restrict__ tile_list, Status *status,
                                                             const float *gcov, const float *gdep, const float *gnrm,
                                                             const uint2 *__restrict__ state, float *grad) {
-  __shared__ SoftPrim s_win[kSoftNT];  // a 32-entry window per warp
-  SoftPrim *s_w = s_win + (threadIdx.x & ~31);
+  __shared__ __align__(16) unsigned char s_win[(kSoftNT / 32) * kWindowBytes];  // a window per warp
+  const SoftWindow W(s_win + (threadIdx.x >> 5) * kWindowBytes);
   const int lane = threadIdx.x & 31;
   const uint32_t n_items = status->n_list * 8u;
   for (;;) {
@@ -698,7 +808,7 @@ __global__ __launch_bounds__(kSoftNT, 4) void k_soft_bwd_warps(Geometry g, const
     else if ((unsigned long long)T.start + cnt > cap_entries) cnt = (uint32_t)(cap_entries - T.start);
     T.m = (int)cnt;
     T.list = entries + T.start;
-    if (cnt > 0) soft_bwd_walk(g, T, wblk, recs, rec_of, gcov, gdep, gnrm, state, grad, s_w);
+    if (cnt > 0) soft_bwd_walk(g, T, wblk, recs, rec_of, gcov, gdep, gnrm, state, grad, W);
     __syncwarp();
   }
 }
@@ -722,8 +832,8 @@ cudaError_t run_soft_pipeline(const Geometry &g, const Scene &sc, const Scratch 
     if (e != cudaSuccess) return e;
   }
   const long long n_tiles = (long long)g.n_img * g.tiles_per_img;
-  // persistent backward CTAs: as many as fit at once (4 per SM), never more than there are tiles
-  const long long most = 4LL * sm_count();
+  // persistent backward CTAs: as many as fit at once, never more than there are tiles
+  const long long most = (long long)VTX_SOFT_BWD_MINB * sm_count();
   const unsigned grid = (unsigned)(n_tiles < most ? (n_tiles > 0 ? n_tiles : 1) : most);
   if (grad == nullptr) {
     k_soft_fwd<<<(unsigned)n_tiles, kSoftNT, kSoftSmem, st>>>(g, s.recs, s.rec_of, s.entries, s.cap_entries,
