@@ -814,7 +814,8 @@ __device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const Vie
   const float n = 4.0f * (float)s.n_rho;  // survivors (n_surv counts the slabs' unused slots too)
   const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
   if (!(mean <= 30.0f || (mean * n <= 1.6e7f && v.f * __uint_as_float(s.rho_bits) <= 6.0f))) return {4, 0};
-  return {256, n <= 49152.0f ? 3 : (n <= 163840.0f ? 2 : 0)};
+  const float held = fmaxf(n, 0.5f * (float)s.n_surv);  // a sparse view's slabs are mostly unused slots: each costs a step
+  return {256, held <= 49152.0f ? 3 : (held <= 163840.0f ? 2 : 0)};
 }
 
 // Setup occupancy: 4 CTAs per SM (63 registers, a few bytes spilled) and 8
