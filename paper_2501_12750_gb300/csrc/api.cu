@@ -46,7 +46,7 @@ struct vtx_ctx {
   vtx_camera cam;
   bool has_cam = false;
   // scratch
-  Buf keys, surv, state, tcount, tstart, tcursor, tlist, bsums, recs, recimg, recbox, recof, entries, status, counts, hostin_x,
+  Buf keys, surv, state, tcount, tstart, tcursor, tlist, recs, recimg, recbox, recof, entries, status, counts, hostin_x,
       hostin_e, hostout, covlist, covmask, stage, defer;
   bool cov_ok = false;  // the covered-pixel list of the last prepared launch fits (two-pass resolve)
   bool occl_ok = false;  // the occlusion pass's buffers of the last prepared launch fit
@@ -259,8 +259,7 @@ static vtx_status prepare(vtx_ctx *c, const Geometry &g, bool soft, long long st
   if ((st = ensure(c, c->tcount, sizeof(uint32_t) * (size_t)(n_tiles + 1), "tile counts"))) return st;
   if ((st = ensure(c, c->tstart, sizeof(uint32_t) * (size_t)(n_tiles + 1), "tile starts"))) return st;
   if ((st = ensure(c, c->tcursor, sizeof(uint32_t) * (size_t)(n_tiles + 1), "tile cursors"))) return st;
-  if ((st = ensure(c, c->tlist, sizeof(uint32_t) * (size_t)(n_tiles + 1), "tile list"))) return st;
-  if ((st = ensure(c, c->bsums, sizeof(unsigned long long) * (size_t)(n_tiles / 4096 + 4), "scan blocks"))) return st;
+  if ((st = ensure(c, c->tlist, sizeof(uint32_t) * (size_t)tile_list_slots(n_tiles), "tile list"))) return st;
   if (c->cap_rec == 0) {
     long long est = n_img * g.stride / 8;
     est = est < (1 << 16) ? (1 << 16) : (est > (1 << 22) ? (1 << 22) : est);
@@ -306,7 +305,6 @@ static Scratch scratch_of(vtx_ctx *c) {
   s.tile_count = (uint32_t *)c->tcount.p;
   s.tile_start = (uint32_t *)c->tstart.p;
   s.tile_cursor = (uint32_t *)c->tcursor.p;
-  s.block_sums = (uint32_t *)c->bsums.p;
   s.tile_list = (uint32_t *)c->tlist.p;
   s.recs = (PrimRec *)c->recs.p;
   s.rec_img = (uint32_t *)c->recimg.p;
@@ -458,7 +456,7 @@ vtx_status vtx_destroy(vtx_ctx *c) {
   cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   Buf *bufs[] = {&c->keys,   &c->surv,   &c->state,  &c->tcount,   &c->tstart,   &c->tcursor,  &c->tlist,
-                 &c->bsums,  &c->recs,   &c->recimg, &c->recbox,   &c->recof,    &c->entries,  &c->status,
+                 &c->recs,   &c->recimg, &c->recbox,   &c->recof,    &c->entries,  &c->status,
                  &c->counts, &c->hostin_x, &c->hostin_e, &c->hostout, &c->covlist, &c->covmask, &c->stage, &c->defer, &c->ses_bits, &c->ses_a, &c->ses_b,
                  &c->ses_edt, &c->ses_blk, &c->ses_base, &c->ses_total, &c->ses_bbox, &c->ses_in};
   for (Buf *b : bufs)

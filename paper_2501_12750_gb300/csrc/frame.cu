@@ -21,8 +21,8 @@
 //        write bound keys (FP32 upper bounds of their entry depth, as keys)
 //        at the pixels they certainly cover; setup then takes only the
 //        survivors that these keys do not hide at every pixel of their boxes;
-//   k_scan_*     exclusive scan of the per-tile counts (counting sort by tile),
-//        listing the non-empty tiles longest first;
+//   k_ranges     gives every tile with binned primitives its range of the entry
+//        array (counting sort by tile) and lists those tiles longest first;
 //   k_scatter    writes (min depth key << 32 | record) entries per tile;
 //   k_raster     resident CTAs take tiles from a queue: each orders its tile's
 //        entries front to back by depth bucket in shared memory (one-pass
@@ -48,7 +48,6 @@ constexpr int kChunk = 1024;                         // atoms per stage (16 KB)
 constexpr int kPerThread = kChunk / kCullThreads;
 constexpr size_t kCullSmem = (size_t)kStages * kChunk * sizeof(float4);
 constexpr uint32_t kWaitLimit = 1u << 24;            // polls before a wait is declared failed
-constexpr int kScanItems = 4096;  // tiles per scan block (1024 threads x 4)
 
 int sm_count() {
   static int n = 0;
@@ -95,6 +94,7 @@ __global__ __launch_bounds__(256) void k_clear(ImageState *st, int n_img, Status
     status->n_list = 0u;
     status->n_cov = 0u;
   }
+  if (tid < kTileClasses) status->cls[tid] = 0u;
   for (long long i = tid; i < n_tiles; i += stride) tile_count[i] = 0u;
   // keys: 16-byte stores over the (256-byte aligned) buffer, then the odd tail
   const ulonglong2 bg2 = make_ulonglong2(kBgKey, kBgKey);
@@ -1221,223 +1221,76 @@ __global__ __launch_bounds__(256) void k_occl_test(Geometry g, const float4 *__r
   }
 }
 
-// ----------------------------------------------------------------- scan --
+// --------------------------------------------------------------- ranges --
 
-__device__ __forceinline__ unsigned long long block_exclusive_scan_1024(unsigned long long v,
-                                                                         unsigned long long *s_warp,
-                                                                         unsigned long long &total) {
+// Every non-empty tile gets a range of the entry array (start and cursor) and a place in the tile list.  Where a tile's
+// range lies does not matter, only that it is its own: a CTA sums its tiles' counts, reserves their total with
+// one atomic and hands out the parts, so no CTA needs another's result (a scan over all tiles needs one CTA, or
+// three launches).  The list is in classes of equal bit length of the count, longest first (TileOrder): a CTA reserves
+// its tiles' places with one atomic per class that it has; pitch 0 keeps a single list.  The order within a class,
+// like that of the ranges, affects only scheduling.
+//
+// Latency-bound (8,160 tiles: 8 CTAs).  8,160 tiles (1080p) 4.3 us against 9.5 us for the one-CTA scan; 16,384 tiles
+// (16 views at 512x512) 6.9 us against 17 us; 129,600 empty tiles (8K) 2.6 us against 13 us for the three kernels.
+constexpr int kRangeThreads = 1024;
+
+__global__ __launch_bounds__(kRangeThreads) void k_ranges(const uint32_t *__restrict__ cnt, long long n,
+                                                          uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
+                                                          uint32_t *__restrict__ list, long long pitch, Status *status,
+                                                          unsigned long long cap_entries) {
+  pdl_enter();
+  if (status->n_rec == 0u) return;  // every tile is empty: the list stays as the set-up kernel left it, empty
+  __shared__ unsigned s_cls[kTileClasses], s_cbase[kTileClasses];
+  __shared__ unsigned long long s_wsum[32], s_base;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned long long x = v;
+  const long long i = (long long)blockIdx.x * kRangeThreads + threadIdx.x;
+  const unsigned c = i < n ? cnt[i] : 0u;
+  unsigned long long x = c;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) s_warp[wid] = x;
+  if (lane == 31) s_wsum[wid] = x;
+  if (threadIdx.x < kTileClasses) s_cls[threadIdx.x] = 0u;
   __syncthreads();
+  const int cls = c ? (pitch ? __clz((int)c) : 0) : -1;
+  const unsigned peers = __match_any_sync(0xffffffffu, cls);
+  const int leader = __ffs(peers) - 1;
+  unsigned slot = 0u;
+  if (cls >= 0 && lane == leader) slot = atomicAdd(&s_cls[cls], (unsigned)__popc(peers));
+  slot = __shfl_sync(0xffffffffu, slot, leader) + (unsigned)__popc(peers & ((1u << lane) - 1u));
   if (wid == 0) {
-    unsigned long long w = lane < (int)(blockDim.x >> 5) ? s_warp[lane] : 0ull;
+    unsigned long long w = s_wsum[lane];
+    const unsigned long long own = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    s_warp[lane] = w;
-  }
-  __syncthreads();
-  unsigned long long off = wid > 0 ? s_warp[wid - 1] : 0ull;
-  total = s_warp[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return off + x - v;
-}
-
-// Per-block exclusive scan of 4,096 tile counts; block totals to block_sums.
-__global__ __launch_bounds__(1024) void k_scan_blocks(const uint32_t *__restrict__ cnt, long long n,
-                                                      uint32_t *__restrict__ start, unsigned long long *block_sums) {
-  pdl_enter();
-  __shared__ unsigned long long s_warp[32];
-  const long long base = (long long)blockIdx.x * kScanItems + (long long)threadIdx.x * 4;
-  uint32_t c[4];
-  unsigned long long sum = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    c[j] = base + j < n ? cnt[base + j] : 0u;
-    sum += c[j];
-  }
-  unsigned long long total;
-  unsigned long long ex = block_exclusive_scan_1024(sum, s_warp, total);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (base + j < n) start[base + j] = (uint32_t)(ex > 0xffffffffull ? 0xffffffffull : ex);
-    ex += c[j];
-  }
-  if (threadIdx.x == 0) block_sums[blockIdx.x] = total;
-}
-
-constexpr int kScanRounds = 32;                                 // values per lane in the one-CTA scan
-static_assert(kScanSingleMax == 32LL * 32 * kScanRounds, "32 warps x 32 lanes x rounds");
-
-// Exclusive scan of every tile count in one CTA (up to 1024 R tiles), listing
-// the non-empty tiles for the raster stage on the way.  Warp w owns the
-// contiguous segment [w S, (w+1) S), S = 32 R; each lane loads its R values
-// up front (coalesced rows of 32), warps scan their rows with shuffles, and
-// one pass over the 32 warp totals links the segments.  The launch picks the
-// smallest R in {8, 16, 32} that covers the tiles: a 1080p frame's 8,160
-// tiles take 8 rounds instead of the 32 a 4K frame needs.  The list is ordered
-// longest first by classes of equal bit length of the count (a counting sort
-// on the count's leading zeros), so that the kernels walking it start the
-// longest tiles first and the short ones fill in behind them; the order
-// within a class, like the order of the lists themselves, affects only
-// scheduling.
-template <int R>
-__global__ __launch_bounds__(1024) void k_scan_single(const uint32_t *__restrict__ cnt, long long n,
-                                                      uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
-                                                      uint32_t *__restrict__ list, Status *status,
-                                                      unsigned long long cap_entries, int skip_if_empty,
-                                                      int list_empty) {
-  pdl_enter();
-  // hard edges: with no binned record every tile is empty; the raster reads
-  // only the tile list (left empty by the set-up kernel) and the scatter has
-  // nothing to place, so the scan has nothing to do
-  if (skip_if_empty && status->n_rec == 0u) return;
-  __shared__ unsigned long long s_wsum[32];
-  // [0, 32): tiles per class (leading zeros of the count), then the class cursors; [32]: non-empty tiles;
-  // [33]: cursor of the empty tiles, listed after all others when list_empty is set
-  __shared__ unsigned int s_cls[34];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long long seg = (long long)wid * 32 * R;
-  if (threadIdx.x < 34) s_cls[threadIdx.x] = 0u;
-  uint32_t v[R];
-  unsigned long long wsum = 0;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const long long i = seg + r * 32 + lane;
-    v[r] = i < n ? cnt[i] : 0u;
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r) wsum += v[r];
-  __syncthreads();  // class counters cleared
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int c = v[r] ? __clz(v[r]) : -1;
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    if (c >= 0 && lane == __ffs(peers) - 1) atomicAdd(&s_cls[c], (unsigned)__popc(peers));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
-  if (lane == 0) s_wsum[wid] = wsum;
-  __syncthreads();
-  if (wid == 0) {
-    unsigned long long x = s_wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    s_wsum[lane] = x - s_wsum[lane];  // exclusive
+    s_wsum[lane] = w - own;
     if (lane == 31) {
-      status->n_entries = x;
-      start[n] = (uint32_t)(x > cap_entries ? cap_entries : x);
-      if (x > cap_entries) atomicOr(&status->overflow, 4u);
-    }
-  } else if (wid == 1) {
-    // class c starts after every class with fewer leading zeros (longer counts); s_cls[32] = tiles listed
-    const unsigned c = s_cls[lane];
-    unsigned y = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, y, o);
-      if (lane >= o) y += t;
-    }
-    s_cls[lane] = y - c;
-    if (lane == 31) {
-      s_cls[32] = y;
-      s_cls[33] = y;
+      const unsigned long long b = w ? atomicAdd(&status->n_entries, w) : 0ull;
+      if (b + w > cap_entries) atomicOr(&status->overflow, 4u);
+      s_base = b;
     }
   }
   __syncthreads();
-  unsigned long long carry = s_wsum[wid];
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    unsigned long long x = v[r];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    const unsigned long long ex = carry + x - v[r];
-    const long long i = seg + r * 32 + lane;
-    const bool ne = i < n && v[r] > 0u;
-    if (i < n) {
-      const uint32_t w = (uint32_t)(ex > cap_entries ? cap_entries : ex);
-      start[i] = w;
-      cursor[i] = w;
-    }
-    const int c = ne ? __clz(v[r]) : (list_empty && i < n ? 33 : -1);
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    const int leader = __ffs(peers) - 1;
-    unsigned base = 0u;
-    if (c >= 0 && lane == leader) base = atomicAdd(&s_cls[c], (unsigned)__popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (c >= 0) list[base + __popc(peers & ((1u << lane) - 1u))] = (uint32_t)i;
-    carry += __shfl_sync(0xffffffffu, x, 31);
+  if (wid == 1) {
+    const unsigned m = s_cls[lane];
+    unsigned b = 0u;
+    if (m) b = atomicAdd(pitch ? &status->cls[lane] : &status->n_list, m);
+    s_cbase[lane] = b;
+    const unsigned all = __reduce_add_sync(0xffffffffu, m);
+    if (pitch && lane == 0 && all) atomicAdd(&status->n_list, all);
   }
-  if (threadIdx.x == 0) status->n_list = s_cls[32];
-}
-
-// Scan of the block totals (one CTA, loops when there are more than 1,024 blocks).
-__global__ __launch_bounds__(1024) void k_scan_top(unsigned long long *block_sums, int nb, Status *status,
-                                                   unsigned long long cap_entries) {
-  pdl_enter();
-  __shared__ unsigned long long s_warp[32];
-  unsigned long long carry = 0;
-  for (int b0 = 0; b0 < nb; b0 += 1024) {
-    int i = b0 + threadIdx.x;
-    unsigned long long v = i < nb ? block_sums[i] : 0ull;
-    unsigned long long total;
-    unsigned long long ex = block_exclusive_scan_1024(v, s_warp, total);
-    if (i < nb) block_sums[i] = carry + ex;
-    carry += total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    block_sums[nb] = carry;
-    status->n_entries = carry;
-    if (carry > cap_entries) atomicOr(&status->overflow, 4u);
-  }
-}
-
-__global__ __launch_bounds__(1024) void k_scan_add(uint32_t *__restrict__ start, uint32_t *__restrict__ cursor,
-                                                   long long n, const unsigned long long *__restrict__ block_sums,
-                                                   unsigned long long cap_entries, const uint32_t *__restrict__ cnt,
-                                                   uint32_t *__restrict__ list, Status *status) {
-  pdl_enter();
-  const long long base = (long long)blockIdx.x * kScanItems + (long long)threadIdx.x * 4;
-  const unsigned long long off = block_sums[blockIdx.x];
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    long long i = base + j;
-    bool ne = false;
-    if (i < n) {
-      unsigned long long v = off + start[i];
-      uint32_t w = (uint32_t)(v > cap_entries ? cap_entries : v);
-      start[i] = w;
-      cursor[i] = w;
-      ne = cnt[i] > 0u;
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, ne);
-    if (m) {
-      const int leader = __ffs(m) - 1;
-      unsigned b = 0u;
-      if (lane == leader) b = atomicAdd(&status->n_list, (unsigned)__popc(m));
-      b = __shfl_sync(0xffffffffu, b, leader);
-      if (ne) list[b + __popc(m & ((1u << lane) - 1u))] = (uint32_t)i;
-    }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    unsigned long long tot = block_sums[gridDim.x];
-    start[n] = (uint32_t)(tot > cap_entries ? cap_entries : tot);
+  __syncthreads();
+  if (i < n) {
+    const unsigned long long ex = s_base + s_wsum[wid] + (x - c);
+    const uint32_t w = (uint32_t)(ex > cap_entries ? cap_entries : ex);
+    start[i] = w;
+    cursor[i] = w;
+    if (cls >= 0) list[(long long)cls * pitch + s_cbase[cls] + slot] = (uint32_t)i;
   }
 }
 
@@ -1770,7 +1623,8 @@ __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__
                                                    const uint32_t *__restrict__ tile_count,
                                                    const uint32_t *__restrict__ tile_start,
                                                    const ImageState *__restrict__ st, unsigned long long *keys,
-                                                   const uint32_t *__restrict__ tile_list, Status *status) {
+                                                   const uint32_t *__restrict__ tile_list, long long pitch,
+                                                   Status *status) {
   pdl_enter();
   constexpr int NT = TW * TH;
   static_assert(NT % 32 == 0, "whole warps per tile");
@@ -1787,13 +1641,15 @@ __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__
   const int wid = (int)(threadIdx.x >> 5);
   const int lx = 8 * (wid % (TW / 8)) + (lane & 7), ly = 4 * (wid / (TW / 8)) + (lane >> 3);
   const uint32_t n_list = status->n_list;
+  if (n_list == 0u) return;
+  const TileOrder order(status, pitch);
   for (;;) {
     __syncthreads();  // every thread has read the previous tile's index
     if (threadIdx.x == 0) s_li = atomicAdd(&status->tile_next, 1u);
     __syncthreads();
     const uint32_t li = s_li;
     if (li >= n_list) break;
-    const long long gt = tile_list[li];
+    const long long gt = order.tile(tile_list, pitch, li);
     const int img = (int)(gt / g.tiles_per_img);
     const int t = (int)(gt % g.tiles_per_img);
     uint32_t cnt = tile_count[gt];
@@ -2227,33 +2083,6 @@ static inline void ev_rec(StageEvents *e, int i, cudaStream_t st) {
   if (e && e->ev && i < e->n && ((e->mask >> i) & 1u)) cudaEventRecord(e->ev[i], st);
 }
 
-// Kernels of a frame are launched with programmatic stream serialisation:
-// a kernel may be scheduled while its predecessor drains, and every kernel
-// opens with pdl_enter(), which waits for the predecessor grid to complete
-// (and its writes to be visible) before any memory access, then lets its
-// successor start launching.  The stream order of all memory effects is
-// unchanged; the launch latency and prologue of each kernel overlap the
-// previous kernel's tail.
-template <typename... P, typename... A>
-static cudaError_t launch_kernel(bool overlap, void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
-                                 A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
-}
-template <typename... P, typename... A>
-static cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
-  return launch_kernel(true, k, grid, block, smem, st, args...);
-}
-
 #ifndef VTX_CLEAR_MEMSET
 #define VTX_CLEAR_MEMSET 1  // clear a batch's key planes with a memset instead of the clear kernel's stores
 #endif
@@ -2359,25 +2188,8 @@ cudaError_t run_binning(const Geometry &g, const Scene &sc, const Scratch &s, cu
   }
   ev_rec(evs, 2, st);
   {
-    if (n_tiles <= kScanSingleMax) {
-      const int skip = soft ? 0 : 1;
-      if (n_tiles <= 1024LL * 8)
-        launch_pdl(k_scan_single<8>, 1, 1024, 0, st, s.tile_count, n_tiles, s.tile_start, s.tile_cursor, s.tile_list,
-                                             s.status, s.cap_entries, skip, 1 - skip);
-      else if (n_tiles <= 1024LL * 16)
-        launch_pdl(k_scan_single<16>, 1, 1024, 0, st, s.tile_count, n_tiles, s.tile_start, s.tile_cursor, s.tile_list,
-                                              s.status, s.cap_entries, skip, 1 - skip);
-      else
-        launch_pdl(k_scan_single<kScanRounds>, 1, 1024, 0, st, s.tile_count, n_tiles, s.tile_start, s.tile_cursor,
-                                                       s.tile_list, s.status, s.cap_entries, skip, 1 - skip);
-    } else {
-      int nb = (int)((n_tiles + kScanItems - 1) / kScanItems);
-      unsigned long long *bs = reinterpret_cast<unsigned long long *>(s.block_sums);
-      launch_pdl(k_scan_blocks, nb, 1024, 0, st, s.tile_count, n_tiles, s.tile_start, bs);
-      launch_pdl(k_scan_top, 1, 1024, 0, st, bs, nb, s.status, s.cap_entries);
-      launch_pdl(k_scan_add, nb, 1024, 0, st, s.tile_start, s.tile_cursor, n_tiles, bs, s.cap_entries, s.tile_count,
-                                      s.tile_list, s.status);
-    }
+    launch_pdl(k_ranges, (unsigned)((n_tiles + kRangeThreads - 1) / kRangeThreads), kRangeThreads, 0, st, s.tile_count,
+               n_tiles, s.tile_start, s.tile_cursor, s.tile_list, tile_pitch(n_tiles), s.status, s.cap_entries);
   }
   ev_rec(evs, 3, st);
   if (soft)
@@ -2414,13 +2226,13 @@ cudaError_t run_frame_pipeline(const Geometry &g, const ShadeParams &sh, const S
   const unsigned rgrid = (unsigned)(n_tiles < resident ? (n_tiles > 0 ? n_tiles : 1) : resident);
   if (shape == 0)
     launch_pdl(k_raster<16, 16>, rgrid, 256, raster_smem<256>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, s.status);
+               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
   else if (shape == 1)
     launch_pdl(k_raster<32, 8>, rgrid, 256, raster_smem<256>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, s.status);
+               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
   else
     launch_pdl(k_raster<8, 8>, rgrid, 64, raster_smem<64>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, s.status);
+               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
   ev_rec(evs, 5, st);
   if (sc.dbg_corrupt_key && s.keys) cudaMemsetAsync(s.keys, 0x7f, sizeof(unsigned long long), st);  // test hook
   if (VTX_RESOLVE_2PASS && s.cov_list) {

@@ -11,23 +11,26 @@
 //   w_i = alpha_i T_i, T_{i+1} = T_i (1 - alpha_i), stop once T < 1e-4;
 //   coverage = sum w_i, depth = sum w_i t_i, normal = sum w_i n_i.
 // Binning (cull with 4 px dilation, precise setup, per-tile counting sort)
-// is shared with the hard-edge path; each tile CTA (tiles longest first)
-// sorts its list by (centre depth key, id) in shared memory (bucket pass plus
-// per-bucket insertion sort; in global memory for lists longer than shared
-// memory holds) and writes it back, then each warp walks the sorted list on
-// its own, staging 32 entries at a time -- those that can reach its pixels, in
-// pairs -- with their per-sphere constants (f / z_c, 1 / r and a bound on rho^2
-// that rejects most before any square root or division), and takes a pair per
-// step on the paired FP32 pipes.  The forward can leave per pixel its final
-// transmittance and last contributor (the state).  The backward either
-// reuses the forward's sorted lists (warps taking (tile, block) items from a
-// queue) or rebuilds them; it takes the last contributor and final
-// transmittance from the state, or re-walks each pixel front to back for
-// them, then walks back to front with the carry
-// R_i = alpha_{i+1} c_{i+1} + (1 - alpha_{i+1}) R_{i+1}, recovering T_i from
-// T_{i+1} / (1 - alpha_i) (alpha <= 0.99 keeps this safe), and accumulates
-// d/d(x, y, z, r) per sphere as a warp sum (one reduce-scatter of nine
-// shuffles per pair) and one 16-byte FP32 atomic per sphere and warp.
+// is shared with the hard-edge path.  Then
+//   k_soft_sort  one CTA per non-empty tile orders its list by (centre depth
+//        key, id) in shared memory (bucket pass plus per-bucket insertion sort;
+//        in global memory for lists longer than shared memory holds) and
+//        writes it back; other CTAs fill the planes of the empty tiles;
+//   k_soft_fwd   each warp takes (tile, 8x4 block) items from a queue, longest
+//        lists first, and walks the sorted list on its own, staging 32 entries
+//        at a time -- those that can reach its pixels, in pairs -- with their
+//        per-sphere constants (f / z_c, 1 / r and a bound on rho^2 that rejects
+//        most before any square root or division), and takes a pair per step
+//        on the paired FP32 pipes.  It can leave per pixel its final
+//        transmittance and last contributor (the state);
+//   k_soft_bwd   likewise over the forward's sorted lists or rebuilt ones: it
+//        takes the last contributor and final transmittance from the state, or
+//        re-walks each pixel front to back for them, then walks back to front
+//        with the carry R_i = alpha_{i+1} c_{i+1} + (1 - alpha_{i+1}) R_{i+1},
+//        recovering T_i from T_{i+1} / (1 - alpha_i) (alpha <= 0.99 keeps this
+//        safe), and accumulates d/d(x, y, z, r) per sphere as a warp sum (one
+//        reduce-scatter of nine shuffles per pair) and one 16-byte FP32 atomic
+//        per sphere and warp.
 #include "vtx_internal.h"
 
 namespace vtx {
@@ -57,9 +60,6 @@ static_assert(kSoftFields == 14, "seven 16-byte words");
 constexpr int kPairWords = kSoftFields / 2;  // 112 bytes: pairs start 28 banks apart, so staging stores conflict 2-way
 constexpr int kWindowBytes = 2048;           // per warp: 16 pairs and 32 atom ids
 static_assert(16 * kPairWords * 16 + 32 * 4 <= kWindowBytes, "a window");
-static_assert((kSoftNT / 32) * kWindowBytes >= kSoftCap * (int)sizeof(uint16_t), "the windows hold the sort's offsets");
-
-constexpr size_t kSoftSmem = kSoftCap * sizeof(unsigned long long) + (kSoftNT / 32) * kWindowBytes;
 
 struct SoftWindow {
   float4 *pair;     // [16][kPairWords]
@@ -157,25 +157,57 @@ __device__ __forceinline__ void soft_pair(const float4 *w, const SoftPix &x, flo
   o.nz = __fmul2_rn(__fadd2_rn(o.dz, si), o.inv_rad);
 }
 
+// A warp's share of a tile: an 8x4 pixel block, lane l its pixel (l & 7, l >> 3), and the tile's list.
 struct SoftTile {
   int img, px, py, m;
-  int px0, py0;  // the tile's first column and row
+  float col0, row0;  // centre of the block's first pixel
   bool inside;
-  uint32_t start;
-  const unsigned long long *list;  // the tile's entries in (centre-depth key, id) order: shared or global memory
+  const unsigned long long *list;  // the tile's entries in (centre-depth key, id) order
 };
 
+__device__ __forceinline__ uint32_t soft_count(const uint32_t *__restrict__ tile_count,
+                                               const uint32_t *__restrict__ tile_start, long long gt,
+                                               unsigned long long cap_entries, uint32_t &start) {
+  uint32_t cnt = tile_count[gt];
+  start = tile_start[gt];
+  if ((unsigned long long)start >= cap_entries) cnt = 0;
+  else if ((unsigned long long)start + cnt > cap_entries) cnt = (uint32_t)(cap_entries - start);
+  return cnt;
+}
+
+__device__ __forceinline__ SoftTile soft_block(const Geometry &g, long long gt, int blk,
+                                               const unsigned long long *__restrict__ entries,
+                                               unsigned long long cap_entries, const uint32_t *__restrict__ tile_count,
+                                               const uint32_t *__restrict__ tile_start) {
+  SoftTile T;
+  const int lane = threadIdx.x & 31;
+  T.img = (int)(gt / g.tiles_per_img);
+  const int t = (int)(gt % g.tiles_per_img);
+  const int px0 = (t % g.tiles_x) * 16 + 8 * (blk & 1), py0 = (t / g.tiles_x) * 16 + 4 * (blk >> 1);
+  T.px = px0 + (lane & 7);
+  T.py = py0 + (lane >> 3);
+  T.col0 = (float)px0 + 0.5f;
+  T.row0 = (float)py0 + 0.5f;
+  T.inside = T.px < g.W && T.py < g.H;
+  uint32_t start;
+  T.m = (int)soft_count(tile_count, tile_start, gt, cap_entries, start);
+  T.list = entries + start;
+  return T;
+}
+
 // Exact ascending order of a tile's m entries (centre-depth key << 32 | id)
-// in s_e.  A one-pass counting sort first places the entries into 256 buckets
+// in s_e.  A one-pass counting sort first places the entries into 1024 buckets
 // of the tile's key range by a monotone FP32 map (every key of a bucket is <=
 // every key of a later bucket, and equal keys share a bucket); each thread
-// then insertion-sorts its own bucket.  A tile whose fullest bucket holds more
+// then insertion-sorts its four buckets.  A tile whose fullest bucket holds more
 // than 32 entries is finished by a bitonic sort instead.  src is the list in
 // global memory (read three times, L1 hits after the first); s_off (2 bytes
-// per entry) is scratch.
+// per entry) is scratch.  1024 buckets because the insertion sorts took 60 % of
+// the cycles at 256 (lists of 540 entries on average: fullest bucket 11).
+constexpr int kSoftBuckets = 1024;
 __device__ __forceinline__ void soft_order(const unsigned long long *__restrict__ src, int m,
                                            unsigned long long *s_e, uint16_t *s_off) {
-  constexpr int NB = kSoftNT;  // one bucket per thread
+  constexpr int NB = kSoftBuckets, PER = NB / kSoftNT;
   __shared__ uint32_t s_cnt[NB], s_red[3], s_wt[kSoftNT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   uint32_t lo = 0xffffffffu, hi = 0u;
@@ -186,7 +218,8 @@ __device__ __forceinline__ void soft_order(const unsigned long long *__restrict_
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  s_cnt[threadIdx.x] = 0u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) s_cnt[threadIdx.x * PER + j] = 0u;
   if (threadIdx.x == 0) {
     s_red[0] = 0xffffffffu;
     s_red[1] = 0u;
@@ -206,20 +239,31 @@ __device__ __forceinline__ void soft_order(const unsigned long long *__restrict_
     s_off[i] = (uint16_t)atomicAdd(s_cnt + min(NB - 1, (int)((float)(k - lo) * scale)), 1u);
   }
   __syncthreads();
-  const uint32_t c = s_cnt[threadIdx.x];
-  uint32_t inc = c;
+  uint32_t c[PER], sum = 0u, cm = 0u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    c[j] = s_cnt[threadIdx.x * PER + j];
+    sum += c[j];
+    cm = max(cm, c[j]);
+  }
+  uint32_t inc = sum;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += y;
   }
-  const uint32_t cmax = __reduce_max_sync(0xffffffffu, c);
+  const uint32_t cmax = __reduce_max_sync(0xffffffffu, cm);
   if (lane == 31) s_wt[wid] = inc;
   if (lane == 0) atomicMax(s_red + 2, cmax);
   __syncthreads();
-  uint32_t base = inc - c;
+  uint32_t base = inc - sum;
   for (int w = 0; w < wid; ++w) base += s_wt[w];
-  s_cnt[threadIdx.x] = base;
+  uint32_t at = base;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    s_cnt[threadIdx.x * PER + j] = at;
+    at += c[j];
+  }
   __syncthreads();
   for (int i = threadIdx.x; i < m; i += kSoftNT) {
     const unsigned long long e = src[i];
@@ -229,7 +273,8 @@ __device__ __forceinline__ void soft_order(const unsigned long long *__restrict_
   const bool small = s_red[2] <= 32u;
   __syncthreads();
   if (small) {
-    for (int i = (int)base + 1; i < (int)(base + c); ++i) {
+    // the thread's buckets follow one another, so no entry moves past the start of its own bucket
+    for (int i = (int)base + 1; i < (int)(base + sum); ++i) {
       const unsigned long long x = s_e[i];
       int j = i - 1;
       while (j >= (int)base && s_e[j] > x) {
@@ -302,44 +347,72 @@ __device__ __noinline__ void soft_sort_global(unsigned long long *a, int m) {
   }
 }
 
-// Load and order a tile's entries (shared by forward and backward).  Up to kSoftCap entries are ordered
-// in shared memory; a longer list is ordered in place in the entry array, which the walk then reads.
-// The forward writes the ordered list back to the entry array (store_back), so a backward call on the
-// same lists loads it already ordered (presorted) instead of sorting it again.
-__device__ __forceinline__ bool soft_load(const Geometry &g, long long gt, unsigned long long *entries,
-                                          unsigned long long cap_entries, const uint32_t *tile_count,
-                                          const uint32_t *tile_start, Status *status, unsigned long long *s_e,
-                                          uint16_t *s_off, SoftTile &T, bool store_back, bool presorted) {
-  T.img = (int)(gt / g.tiles_per_img);
-  const int t = (int)(gt % g.tiles_per_img);
-  const int tx = t % g.tiles_x, ty = t / g.tiles_x;
-  T.px0 = tx * 16;
-  T.py0 = ty * 16;
-  // warp w covers the 8x4 block (w & 1, w >> 1) of the tile; lane l its pixel (l & 7, l >> 3)
-  const int w = (int)(threadIdx.x >> 5), l = (int)(threadIdx.x & 31);
-  T.px = T.px0 + 8 * (w & 1) + (l & 7);
-  T.py = T.py0 + 4 * (w >> 1) + (l >> 3);
-  T.inside = T.px < g.W && T.py < g.H;
-  uint32_t cnt = tile_count[gt];
-  T.start = tile_start[gt];
-  if ((unsigned long long)T.start >= cap_entries) cnt = 0;
-  else if ((unsigned long long)T.start + cnt > cap_entries) cnt = (uint32_t)(cap_entries - T.start);
-  if (threadIdx.x == 0) atomicMax(&status->max_list, cnt);
-  T.m = (int)cnt;
-  T.list = s_e;
-  if (cnt == 0) return false;
-  if (cnt > (uint32_t)kSoftCap) {
-    if (!presorted) soft_sort_global(entries + T.start, T.m);
-    T.list = entries + T.start;
-  } else if (presorted) {
-    for (int i = threadIdx.x; i < T.m; i += kSoftNT) s_e[i] = entries[T.start + i];
-    __syncthreads();
+// Zeros (state: full transmittance, no contributor) into the planes of empty tile gt, by one warp: whole 64-byte rows of
+// eight (state: 128-byte rows of four) tile rows per store.  vec: every row starts on a 16-byte boundary and holds a
+// multiple of four pixels.
+__device__ __forceinline__ void soft_fill_tile(const Geometry &g, long long gt, bool vec, float *cov, float *dep,
+                                               float *nrm, uint2 *state) {
+  const int lane = threadIdx.x & 31;
+  const int img = (int)(gt / g.tiles_per_img), t = (int)(gt % g.tiles_per_img);
+  const int px0 = (t % g.tiles_x) * 16, py0 = (t / g.tiles_x) * 16;
+  const long long ppi = g.pix_per_img;
+  float *plane[5] = {cov + img * ppi, dep + img * ppi, nrm + img * 3 * ppi, nrm + (img * 3 + 1) * ppi,
+                     nrm + (img * 3 + 2) * ppi};
+  uint2 *st = state ? state + img * ppi : nullptr;
+  const uint32_t one = __float_as_uint(1.0f);
+  if (vec) {
+    const int px = px0 + 4 * (lane & 3), sx = px0 + 2 * (lane & 7);
+    for (int y = lane >> 2; y < 16; y += 8)
+      if (px < g.W && py0 + y < g.H)
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+          *reinterpret_cast<float4 *>(plane[q] + (long long)(py0 + y) * g.W + px) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (st)
+      for (int y = lane >> 3; y < 16; y += 4)
+        if (sx < g.W && py0 + y < g.H)
+          *reinterpret_cast<uint4 *>(st + (long long)(py0 + y) * g.W + sx) = make_uint4(one, 0u, one, 0u);
   } else {
-    soft_order(entries + T.start, T.m, s_e, s_off);
-    if (store_back)
-      for (int i = threadIdx.x; i < T.m; i += kSoftNT) entries[T.start + i] = s_e[i];
+    const int px = px0 + (lane & 15);
+    for (int y = lane >> 4; y < 16; y += 2) {
+      if (px >= g.W || py0 + y >= g.H) continue;
+      const long long p = (long long)(py0 + y) * g.W + px;
+      for (int q = 0; q < 5; ++q) plane[q][p] = 0.0f;
+      if (st) st[p] = make_uint2(one, 0u);
+    }
   }
-  return true;
+}
+
+// Orders the lists of the n_list non-empty tiles in place, one CTA each, longest first.  With output planes (the forward),
+// every warp of the CTAs behind them fills one tile's planes if it is empty; those past both end at once.
+__global__ __launch_bounds__(kSoftNT) void k_soft_sort(Geometry g, unsigned long long *entries,
+                                                      unsigned long long cap_entries,
+                                                      const uint32_t *__restrict__ tile_count,
+                                                      const uint32_t *__restrict__ tile_start,
+                                                      const uint32_t *__restrict__ tile_list, long long pitch,
+                                                      Status *status, float *cov, float *dep, float *nrm, uint2 *state,
+                                                      int vec) {
+  pdl_enter();
+  __shared__ unsigned long long s_e[kSoftCap];
+  __shared__ uint16_t s_off[kSoftCap];
+  const uint32_t n_list = status->n_list;
+  if (blockIdx.x >= n_list) {
+    const long long gt = (long long)(blockIdx.x - n_list) * (kSoftNT / 32) + (threadIdx.x >> 5);
+    if (cov && gt < (long long)g.n_img * g.tiles_per_img && tile_count[gt] == 0u)
+      soft_fill_tile(g, gt, vec != 0, cov, dep, nrm, state);
+    return;
+  }
+  const TileOrder order(status, pitch);
+  const long long gt = order.tile(tile_list, pitch, blockIdx.x);
+  uint32_t start;
+  const int m = (int)soft_count(tile_count, tile_start, gt, cap_entries, start);
+  if (threadIdx.x == 0) atomicMax(&status->max_list, (unsigned)m);
+  if (m == 0) return;
+  if (m > kSoftCap) {
+    soft_sort_global(entries + start, m);
+    return;
+  }
+  soft_order(entries + start, m, s_e, s_off);
+  for (int i = threadIdx.x; i < m; i += kSoftNT) entries[start + i] = s_e[i];
 }
 
 // Each warp walks the sorted list on its own (no block barrier after the
@@ -428,42 +501,28 @@ __device__ __forceinline__ int soft_stage(const PrimRec *__restrict__ recs, uint
 // state (optional, [n_img][H][W]): per pixel the final transmittance (float
 // bits) and 1 + the sorted-list position of its last contributor (0: none),
 // which lets the backward pass start its back-to-front walk directly.
-// Forward CTAs per SM: 3 (80 registers); 20,000 atoms from 16 views at 512x512: forward 284 us at 3, 304 at 4 (spills),
-// 331 at 2.  One entry per step on the scalar pipes took 309 us (4 CTAs).
-#ifndef VTX_SOFT_FWD_MINB
-#define VTX_SOFT_FWD_MINB 3
-#endif
-// One tile of the forward pass (called by every thread of the CTA).
-__device__ __forceinline__ void soft_fwd_tile(const Geometry &g, long long gt, const PrimRec *__restrict__ recs,
-                                              const uint32_t *__restrict__ rec_of, unsigned long long *entries,
-                                              unsigned long long cap_entries, const uint32_t *__restrict__ tile_count,
-                                              const uint32_t *__restrict__ tile_start, Status *status, float *cov,
-                                              float *dep, float *nrm, uint2 *state, unsigned long long *s_e,
-                                              unsigned char *s_win) {
-  SoftTile T;
-  const bool any = soft_load(g, gt, entries, cap_entries, tile_count, tile_start, status, s_e,
-                             reinterpret_cast<uint16_t *>(s_win), T, true, false);
-  const SoftWindow W(s_win + (threadIdx.x >> 5) * kWindowBytes);
+// The forward of one warp's block.
+__device__ __forceinline__ void soft_fwd_walk(const Geometry &g, const SoftTile &T, const PrimRec *__restrict__ recs,
+                                              const uint32_t *__restrict__ rec_of, Status *status, float *cov,
+                                              float *dep, float *nrm, uint2 *state, const SoftWindow &W) {
   const ViewParams &v = g.views[T.img % g.n_views];
   const SoftPix x = soft_pix(v, T.px, T.py);
   const float inv_sigma = 1.0f / g.sigma;
   const float nl2s = -1.4426950408889634f * inv_sigma;  // exp(-delta / sigma) = 2^(delta nl2s)
   const float uu_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x.r.uu)));
-  const float col0 = (float)(T.px0 + 8 * (int)((threadIdx.x >> 5) & 1)) + 0.5f;
-  const float row0 = (float)(T.py0 + 4 * (int)(threadIdx.x >> 6)) + 0.5f;
   const int lane = threadIdx.x & 31;
   float A = 0.0f, D = 0.0f, N0 = 0.0f, N1 = 0.0f, N2 = 0.0f, Tr = 1.0f;
   int last = -1;
   unsigned used = 0u;
   bool done = !T.inside;
-  if (any) {
+  {
     uint32_t ridx = soft_rec_index(g, rec_of, T, lane), next = soft_rec_index(g, rec_of, T, 32 + lane);
     for (int c0 = 0; c0 < T.m; c0 += 32) {
       const unsigned am = __ballot_sync(0xffffffffu, !done);
       if (am == 0u) break;
       const uint32_t next2 = soft_rec_index(g, rec_of, T, c0 + 64 + lane);  // in flight during this window
       soft_prefetch(recs, next);
-      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, col0, row0, uu_max);
+      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, T.col0, T.row0, uu_max);
       ridx = next;
       next = next2;
       for (int q = 0; q < n; q += 2) {
@@ -515,25 +574,42 @@ __device__ __forceinline__ void soft_fwd_tile(const Geometry &g, long long gt, c
   }
 }
 
-// Forward: one CTA per tile, the empty ones writing their zeros (overlapped with the busy tiles).
-// state (optional, [n_img][H][W]): per pixel the final transmittance (float
-// bits) and 1 + the sorted-list position of its last contributor (0: none),
-// which lets the backward pass start its back-to-front walk directly.
+// Warps take (tile, 8x4 block) items from a queue: the non-empty tiles longest first, eight blocks each.  No step needs
+// the whole tile, so a warp that finishes its block early takes the next item instead of waiting for the tile's
+// slowest warp (a quarter of the time with a CTA per tile, of 20,000 atoms from 16 views), and the sort before it keeps
+// neither its registers nor its shared memory.
+// Forward CTAs per SM: 3 (80 registers).
+//
+// 20,000 atoms from 16 views at 512x512: 136 us after 45 us of sorting and filling, forward call 223 us; 284 us with a CTA per tile that sorted, walked and (empty
+// ones) filled; 309 us with one entry per step on the scalar pipes.
+#ifndef VTX_SOFT_FWD_MINB
+#define VTX_SOFT_FWD_MINB 3
+#endif
 __global__ __launch_bounds__(kSoftNT, VTX_SOFT_FWD_MINB) void k_soft_fwd(Geometry g, const PrimRec *__restrict__ recs,
                                                       const uint32_t *__restrict__ rec_of,
-                                                      unsigned long long *entries,
+                                                      const unsigned long long *__restrict__ entries,
                                                       unsigned long long cap_entries,
                                                       const uint32_t *__restrict__ tile_count,
                                                       const uint32_t *__restrict__ tile_start,
-                                                      const uint32_t *__restrict__ tile_list, Status *status,
-                                                      float *cov, float *dep, float *nrm, uint2 *state) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  unsigned long long *s_e = reinterpret_cast<unsigned long long *>(smem);
-  unsigned char *s_win = smem + kSoftCap * sizeof(unsigned long long);
-  // every tile, longest list first when the scan listed them all (empty tiles last), else in index order
-  const long long gt = tile_list ? (long long)tile_list[blockIdx.x] : (long long)blockIdx.x;
-  soft_fwd_tile(g, gt, recs, rec_of, entries, cap_entries, tile_count, tile_start, status, cov, dep, nrm, state, s_e,
-                s_win);
+                                                      const uint32_t *__restrict__ tile_list, long long pitch,
+                                                      Status *status, float *cov, float *dep, float *nrm,
+                                                      uint2 *state) {
+  pdl_enter();
+  __shared__ __align__(16) unsigned char s_win[(kSoftNT / 32) * kWindowBytes];  // a window per warp
+  const SoftWindow W(s_win + (threadIdx.x >> 5) * kWindowBytes);
+  const int lane = threadIdx.x & 31;
+  const uint32_t n_items = status->n_list * 8u;
+  const TileOrder order(status, pitch);
+  for (;;) {
+    uint32_t item = 0u;
+    if (lane == 0) item = atomicAdd(&status->tile_next, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_items) break;
+    const SoftTile T = soft_block(g, order.tile(tile_list, pitch, item >> 3), (int)(item & 7u), entries, cap_entries,
+                                  tile_count, tile_start);
+    soft_fwd_walk(g, T, recs, rec_of, status, cov, dep, nrm, state, W);
+    __syncwarp();
+  }
 }
 
 // Sums over the warp of four per-lane values of sphere a and four of sphere b, scattered: lanes 0, 4, 8, 12 receive
@@ -556,9 +632,8 @@ __device__ __forceinline__ float warp_sum8_scatter(const float2 (&v)[4], int lan
   return s;
 }
 
-// The backward of one warp: its 8x4 pixel block wblk of tile T, whose sorted list T.list is in shared or
-// global memory; W is the warp's window.
-__device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile &T, int wblk,
+// The backward of one warp's block; W is the warp's window.
+__device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile &T,
                                               const PrimRec *__restrict__ recs, const uint32_t *__restrict__ rec_of,
                                               const float *gcov, const float *gdep, const float *gnrm,
                                               const uint2 *__restrict__ state, float *grad, const SoftWindow &W) {
@@ -584,8 +659,6 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
   // pass 1: front to back, last contributor and final transmittance (read from the forward call's state
   // when it left one)
   const float uu_max = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(r.uu)));
-  const float col0 = (float)(T.px0 + 8 * (wblk & 1)) + 0.5f;
-  const float row0 = (float)(T.py0 + 4 * (wblk >> 1)) + 0.5f;
   float Tr = 1.0f;
   int last = -1;
   bool done = !need;
@@ -605,7 +678,7 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
       if (am == 0u) break;
       const uint32_t next2 = soft_rec_index(g, rec_of, T, c0 + 64 + lane);
       soft_prefetch(recs, next);
-      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, col0, row0, uu_max);
+      const int n = soft_stage(recs, ridx, T, c0, T.m, v.f, W, am, T.col0, T.row0, uu_max);
       ridx = next;
       next = next2;
       for (int q = 0; q < n; q += 2) {
@@ -641,7 +714,7 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
     ridx = prev;
     prev = prev2;
     if (am == 0u) continue;
-    const int n = soft_stage(recs, cur, T, c0, wlast + 1, v.f, W, am, col0, row0, uu_max);
+    const int n = soft_stage(recs, cur, T, c0, wlast + 1, v.f, W, am, T.col0, T.row0, uu_max);
     for (int q = (n - 1) & ~1; q >= 0; q -= 2) {
       const float4 *pw = W.pair + (q >> 1) * kPairWords;
       float2 gr[4];  // d/d(x, y, z) in the internal frame and d/dr, of spheres a and b
@@ -723,92 +796,37 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
   }
 }
 
-__device__ __forceinline__ void soft_bwd_tile(const Geometry &g, long long gt, const PrimRec *__restrict__ recs,
-                                              const uint32_t *__restrict__ rec_of, unsigned long long *entries,
-                                              unsigned long long cap_entries, const uint32_t *__restrict__ tile_count,
-                                              const uint32_t *__restrict__ tile_start, Status *status,
-                                              const float *gcov, const float *gdep, const float *gnrm,
-                                              const uint2 *__restrict__ state, float *grad, unsigned long long *s_e,
-                                              unsigned char *s_win, bool presorted) {
-  SoftTile T;
-  if (!soft_load(g, gt, entries, cap_entries, tile_count, tile_start, status, s_e,
-                 reinterpret_cast<uint16_t *>(s_win), T, false, presorted))
-    return;
-  const int wid = (int)(threadIdx.x >> 5);
-  soft_bwd_walk(g, T, wid, recs, rec_of, gcov, gdep, gnrm, state, grad, SoftWindow(s_win + wid * kWindowBytes));
-}
-
-// Persistent backward over the non-empty tiles (as the forward).
-__global__ __launch_bounds__(kSoftNT) void k_soft_bwd(Geometry g, const PrimRec *__restrict__ recs,
-                                                      const uint32_t *__restrict__ rec_of,
-                                                      unsigned long long *entries,
-                                                      unsigned long long cap_entries,
-                                                      const uint32_t *__restrict__ tile_count,
-                                                      const uint32_t *__restrict__ tile_start,
-                                                      const uint32_t *__restrict__ tile_list, Status *status,
-                                                      const float *gcov, const float *gdep, const float *gnrm,
-                                                      const uint2 *__restrict__ state, float *grad, int presorted) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  unsigned long long *s_e = reinterpret_cast<unsigned long long *>(smem);
-  unsigned char *s_win = smem + kSoftCap * sizeof(unsigned long long);
-  __shared__ uint32_t s_li;
-  const uint32_t n_list = status->n_list;
-  for (;;) {
-    if (threadIdx.x == 0) s_li = atomicAdd(&status->soft_next, 1u);
-    __syncthreads();
-    const uint32_t li = s_li;
-    if (li >= n_list) break;
-    soft_bwd_tile(g, tile_list[li], recs, rec_of, entries, cap_entries, tile_count, tile_start, status, gcov, gdep,
-                  gnrm, state, grad, s_e, s_win, presorted != 0);
-    __syncthreads();
-  }
-}
-
-// Backward on the forward call's lists, already sorted in the entry array: each warp takes (tile, 8x4 block)
-// items from a queue -- the non-empty tiles longest first, eight blocks each -- and walks the tile's list in
-// global memory on its own.  No step needs the whole tile, so there is no block barrier: a warp that finishes
-// its block early takes the next item instead of waiting for the tile's slowest warp.
+// Items and queue as the forward's.
 // Bound by issue and, on small problems, by each warp's chain of pairs.  Two CTAs per SM (120 registers, nothing
 // spilled): 20,000 atoms from 16 views at 512x512 307 us, 1,200 atoms from 2 views at 200x136 138 us; 3 CTAs 310 / 161,
 // 4 CTAs 368 / 181.  One entry per step, its atom id read from the list in global memory, took 362 / 179 us.
 #ifndef VTX_SOFT_BWD_MINB
 #define VTX_SOFT_BWD_MINB 2
 #endif
-__global__ __launch_bounds__(kSoftNT, VTX_SOFT_BWD_MINB) void k_soft_bwd_warps(Geometry g, const PrimRec *__restrict__ recs,
+__global__ __launch_bounds__(kSoftNT, VTX_SOFT_BWD_MINB) void k_soft_bwd(Geometry g, const PrimRec *__restrict__ recs,
                                                             const uint32_t *__restrict__ rec_of,
                                                             const unsigned long long *__restrict__ entries,
                                                             unsigned long long cap_entries,
                                                             const uint32_t *__restrict__ tile_count,
                                                             const uint32_t *__restrict__ tile_start,
-                                                            const uint32_t *__restrict__ tile_list, Status *status,
+                                                            const uint32_t *__restrict__ tile_list, long long pitch,
+                                                            Status *status,
                                                             const float *gcov, const float *gdep, const float *gnrm,
                                                             const uint2 *__restrict__ state, float *grad) {
+  pdl_enter();
   __shared__ __align__(16) unsigned char s_win[(kSoftNT / 32) * kWindowBytes];  // a window per warp
   const SoftWindow W(s_win + (threadIdx.x >> 5) * kWindowBytes);
   const int lane = threadIdx.x & 31;
   const uint32_t n_items = status->n_list * 8u;
+  const TileOrder order(status, pitch);
   for (;;) {
     uint32_t item = 0u;
     if (lane == 0) item = atomicAdd(&status->soft_next, 1u);
     item = __shfl_sync(0xffffffffu, item, 0);
     if (item >= n_items) break;
-    const long long gt = tile_list[item >> 3];
-    const int wblk = (int)(item & 7u);
-    SoftTile T;
-    T.img = (int)(gt / g.tiles_per_img);
-    const int t = (int)(gt % g.tiles_per_img);
-    T.px0 = (t % g.tiles_x) * 16;
-    T.py0 = (t / g.tiles_x) * 16;
-    T.px = T.px0 + 8 * (wblk & 1) + (lane & 7);
-    T.py = T.py0 + 4 * (wblk >> 1) + (lane >> 3);
-    T.inside = T.px < g.W && T.py < g.H;
-    uint32_t cnt = tile_count[gt];
-    T.start = tile_start[gt];
-    if ((unsigned long long)T.start >= cap_entries) cnt = 0;
-    else if ((unsigned long long)T.start + cnt > cap_entries) cnt = (uint32_t)(cap_entries - T.start);
-    T.m = (int)cnt;
-    T.list = entries + T.start;
-    if (cnt > 0) soft_bwd_walk(g, T, wblk, recs, rec_of, gcov, gdep, gnrm, state, grad, W);
+    const SoftTile T = soft_block(g, order.tile(tile_list, pitch, item >> 3), (int)(item & 7u), entries, cap_entries,
+                                  tile_count, tile_start);
+    if (T.m > 0) soft_bwd_walk(g, T, recs, rec_of, gcov, gdep, gnrm, state, grad, W);
     __syncwarp();
   }
 }
@@ -816,12 +834,6 @@ __global__ __launch_bounds__(kSoftNT, VTX_SOFT_BWD_MINB) void k_soft_bwd_warps(G
 cudaError_t run_soft_pipeline(const Geometry &g, const Scene &sc, const Scratch &s, float *cov, float *depth,
                               float *normal, const float *g_cov, const float *g_depth, const float *g_normal,
                               float *grad, uint2 *state, bool reuse_lists, cudaStream_t st, StageEvents *evs) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_soft_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSoftSmem);
-    cudaFuncSetAttribute(k_soft_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSoftSmem);
-    attr = true;
-  }
   const bool reuse = reuse_lists && grad != nullptr;
   if (reuse) {
     // the lists, records and tile order of the forward call are still in place; only the backward's tile
@@ -831,25 +843,26 @@ cudaError_t run_soft_pipeline(const Geometry &g, const Scene &sc, const Scratch 
     cudaError_t e = run_binning(g, sc, s, st, evs, true);
     if (e != cudaSuccess) return e;
   }
-  const long long n_tiles = (long long)g.n_img * g.tiles_per_img;
-  // persistent backward CTAs: as many as fit at once, never more than there are tiles
-  const long long most = (long long)VTX_SOFT_BWD_MINB * sm_count();
-  const unsigned grid = (unsigned)(n_tiles < most ? (n_tiles > 0 ? n_tiles : 1) : most);
-  if (grad == nullptr) {
-    k_soft_fwd<<<(unsigned)n_tiles, kSoftNT, kSoftSmem, st>>>(g, s.recs, s.rec_of, s.entries, s.cap_entries,
-                                                             s.tile_count, s.tile_start,
-                                                             n_tiles <= kScanSingleMax ? s.tile_list : nullptr,
-                                                             s.status, cov, depth, normal, state);
+  const long long n_tiles = (long long)g.n_img * g.tiles_per_img, pitch = tile_pitch(n_tiles);
+  const bool fwd = grad == nullptr;
+  if (!reuse) {
+    const bool vec = fwd && g.W % 4 == 0 &&
+                     ((uintptr_t)cov | (uintptr_t)depth | (uintptr_t)normal | (uintptr_t)state) % 16 == 0;
+    // n_list (at most n_tiles, not known here) sorting CTAs and, forward, a filling warp per tile
+    const long long fill = fwd ? (n_tiles + kSoftNT / 32 - 1) / (kSoftNT / 32) : 0;
+    launch_pdl(k_soft_sort, (unsigned)(n_tiles + fill), kSoftNT, 0, st, g, s.entries, s.cap_entries, s.tile_count,
+               s.tile_start, s.tile_list, pitch, s.status, cov, depth, normal, state, vec ? 1 : 0);
+  }
+  // persistent CTAs: as many as are resident at once, never more than eight items of a tile each
+  const long long most = (long long)(fwd ? VTX_SOFT_FWD_MINB : VTX_SOFT_BWD_MINB) * sm_count();
+  const unsigned grid = (unsigned)(n_tiles < most ? n_tiles : most);
+  if (fwd) {
+    launch_pdl(k_soft_fwd, grid, kSoftNT, 0, st, g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
+               s.tile_start, s.tile_list, pitch, s.status, cov, depth, normal, state);
   } else {
     cudaMemsetAsync(grad, 0, sizeof(float) * 4 * (size_t)g.n_atoms, st);
-    if (reuse)
-      k_soft_bwd_warps<<<(unsigned)most, kSoftNT, 0, st>>>(g, s.recs, s.rec_of, s.entries, s.cap_entries,
-                                                           s.tile_count, s.tile_start, s.tile_list, s.status, g_cov,
-                                                           g_depth, g_normal, state, grad);
-    else
-      k_soft_bwd<<<grid, kSoftNT, kSoftSmem, st>>>(g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
-                                                   s.tile_start, s.tile_list, s.status, g_cov, g_depth, g_normal,
-                                                   state, grad, 0);
+    launch_pdl(k_soft_bwd, grid, kSoftNT, 0, st, g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
+               s.tile_start, s.tile_list, pitch, s.status, g_cov, g_depth, g_normal, state, grad);
   }
   if (evs && evs->ev && evs->n > 5) cudaEventRecord(evs->ev[5], st);
   if (evs && evs->ev && evs->n > 6) cudaEventRecord(evs->ev[6], st);

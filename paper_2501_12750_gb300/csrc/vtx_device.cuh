@@ -31,6 +31,7 @@ constexpr float kKeySpanF = 4294966784.0f;
 constexpr int kMaxViews = 16;
 constexpr int kMaxSsao = 64;
 constexpr int kMaxElem = 32;
+constexpr int kTileClasses = 32;
 
 // ------------------------------------------------------------ parameters --
 
@@ -113,12 +114,37 @@ struct Status {
                                 // 5 a decoded primitive id out of range
   unsigned long long n_entries; // binned (tile, primitive) entries requested
   unsigned int max_list;        // longest tile list seen by the raster stage
-  unsigned int n_list;          // non-empty tiles listed by the scan (raster work list)
+  unsigned int n_list;          // non-empty tiles listed (raster work list)
   unsigned int n_cov;           // covered pixels listed by the resolve's list pass
   unsigned int pad;
   unsigned long long n_terms;   // soft forward: sigmoid terms composited (sum over pixels)
-  unsigned int soft_next;       // soft passes: the next entry of the non-empty tile list to take
-  unsigned int tile_next;       // hard raster: the next entry of the non-empty tile list to take
+  unsigned int soft_next;       // soft backward: the next (tile, block) item of the non-empty tile list to take
+  unsigned int tile_next;       // hard raster: the next entry of that list; soft forward: the next (tile, block) item
+  unsigned int cls[kTileClasses];  // non-empty tiles of each length class (the lists behind TileOrder)
+};
+
+// The non-empty tiles, longest list first: one list of tile indices per class of equal bit length of the count (class c:
+// c leading zeros), `pitch` apart (pitch 0: a single unordered list).  Lane c of every warp holds the number of tiles
+// listed before class c, so that a warp finds the i-th tile with one ballot.  All lanes call both together.
+struct TileOrder {
+  unsigned before;  // lane c: tiles in classes 0 .. c - 1
+  __device__ __forceinline__ TileOrder(const Status *status, long long pitch) {
+    const int lane = threadIdx.x & 31;
+    const unsigned c = pitch ? status->cls[lane] : 0u;
+    unsigned x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    before = x - c;
+  }
+  __device__ __forceinline__ uint32_t tile(const uint32_t *__restrict__ list, long long pitch, uint32_t i) const {
+    if (pitch == 0) return list[i];
+    // the last class that starts at or before i (empty classes before it may start there too)
+    const int c = 31 - __clz((int)__ballot_sync(0xffffffffu, before <= i));
+    return list[(long long)c * pitch + (i - __shfl_sync(0xffffffffu, before, c))];
+  }
 };
 
 // A binned primitive staged through shared memory (64 bytes).  Its tile box

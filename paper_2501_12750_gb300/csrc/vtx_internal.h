@@ -14,9 +14,10 @@ namespace vtx {
 #endif
 constexpr long long kOcclPixels = VTX_OCCL_PIXELS;  // occlusion pass from one survivor per this many pixels
 
-// Tile counts that the one-CTA scan covers (32 warps x 32 lanes x 32 values); more take the three-kernel scan,
-// whose tile list is unordered and holds the non-empty tiles only.
-constexpr long long kScanSingleMax = 32LL * 32 * 32;
+// Distance of the tile list's classes (TileOrder): a list per class for up to 131,072 tiles (16 MB), a single unordered
+// list beyond, where the tiles of many images even out by themselves.
+inline long long tile_pitch(long long n_tiles) { return n_tiles <= (1 << 17) ? n_tiles : 0; }
+inline long long tile_list_slots(long long n_tiles) { return n_tiles <= (1 << 17) ? n_tiles * kTileClasses : n_tiles; }
 
 // Device buffers of one pipeline run (all owned by the context).
 struct Scratch {
@@ -24,11 +25,9 @@ struct Scratch {
   uint32_t *surv;             // [n_img][surv_cap] survivor primitive ids
   ImageState *state;          // [n_img]
   uint32_t *tile_count;       // [n_tiles]
-  uint32_t *tile_start;       // [n_tiles + 1] exclusive prefix (tile_start[n_tiles] = total, clamped)
+  uint32_t *tile_start;       // [n_tiles] first entry of each tile (clamped to the capacity)
   uint32_t *tile_cursor;      // [n_tiles]
-  uint32_t *block_sums;       // [ceil(n_tiles / 4096) + 1]
-  uint32_t *tile_list;        // [n_tiles] indices of the non-empty tiles, longest list first (one-CTA scan);
-                              // the soft path's one-CTA scan lists the empty tiles after them
+  uint32_t *tile_list;        // [tile_list_slots(n_tiles)] the non-empty tiles, in classes (TileOrder)
   PrimRec *recs;              // [cap_rec]
   uint32_t *rec_img;          // [cap_rec] image of each record
   uint2 *rec_box;             // [cap_rec] tile box of each record: (x0 | y0 << 16, x1 | y1 << 16)
@@ -114,6 +113,33 @@ long long ses_blocks(const int32_t dims[3]);
 int ses_window(float probe, float h);
 bool ses_three_pass(float probe, float h);  // the window is too large for the bit-set distance pass
 long long ses_words(const int32_t dims[3]);  // 32-bit words of the interior bits
+
+// Kernels of a frame are launched with programmatic stream serialisation:
+// a kernel may be scheduled while its predecessor drains, and every kernel
+// opens with pdl_enter(), which waits for the predecessor grid to complete
+// (and its writes to be visible) before any memory access, then lets its
+// successor start launching.  The stream order of all memory effects is
+// unchanged; the launch latency and prologue of each kernel overlap the
+// previous kernel's tail.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(bool overlap, void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                                 A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
+  return launch_kernel(true, k, grid, block, smem, st, args...);
+}
 
 int sm_count();
 
