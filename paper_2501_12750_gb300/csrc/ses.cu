@@ -16,7 +16,7 @@
 //   3. SES interior: edt2 >= 1 and edt2 h^2 >= p^2 (FP64; an integer threshold
 //      here, as the product is monotone in edt2), again one bit per point.
 //      Marching cubes in two passes over "groups" of 32 cells of a row: one
-//      counts the triangles of every 256 groups (the last CTA scans the
+//      counts the triangles of every CTA's groups (the last CTA scans the
 //      counts), the other writes them in cell order, so the output order is
 //      deterministic.  The per-case loops come from a table built once on the
 //      host: faces with four crossings cut their inside corners apart, segments
@@ -33,7 +33,6 @@
 namespace vtx {
 
 constexpr int kSesThreads = 256;
-constexpr int kSesGroups = 256;  // groups of 32 cells per CTA of the marching-cubes passes
 constexpr uint16_t kSesInf = 0xffffu;
 
 // Per case: number of loops, their lengths, their edges back to back, and the triangles as three 4-bit vertex
@@ -598,20 +597,22 @@ __device__ __forceinline__ unsigned block_exclusive_sum(unsigned v, unsigned *to
   return before;
 }
 
-// Triangles of every 256 groups (one group per thread, going through its crossing cells), and, in the last CTA to
+// Triangles of every `per_cta` <= 256 groups (one group per thread, going through its crossing cells), and, in the last CTA to
 // finish, their exclusive scan: block_base[b] is the first triangle of CTA b's groups.  *done counts finished CTAs
 // (zero at launch); no CTA waits for another.  3.4e7 points: 27 us, of which most is the table lookups of the
 // crossing cells; 307 us with one thread per four cells reading the distance plane, and 100 us for the scan of
 // its eight times as many counts in a launch of its own.
 __global__ __launch_bounds__(kSesThreads) void k_ses_count(SesGrid G, const uint32_t *__restrict__ inside,
-                                                           uint32_t n_groups, unsigned *__restrict__ block_tris,
+                                                           uint32_t n_groups, unsigned per_cta,
+                                                           unsigned *__restrict__ block_tris,
                                                            unsigned long long *__restrict__ block_base,
                                                            unsigned long long *__restrict__ total, unsigned *done) {
   __shared__ unsigned char s_tris[256];
   __shared__ bool s_last;
   s_tris[threadIdx.x] = g_ses_case[threadIdx.x].n_tris;
   __syncthreads();
-  const SesGroup s = ses_group(G, inside, blockIdx.x * (unsigned)kSesGroups + threadIdx.x, n_groups);
+  const SesGroup s = ses_group(G, inside, blockIdx.x * per_cta + threadIdx.x,
+                               threadIdx.x < per_cta ? n_groups : 0u);
   unsigned n = 0u;
   for (uint32_t m = s.active; m != 0u; m &= m - 1u) n += s_tris[ses_case_of(s, __ffs(m) - 1)];
   unsigned sum;
@@ -685,6 +686,7 @@ __device__ __forceinline__ float3 edge_point(const SesEmitShared &sh, int cell, 
 // a case byte per cell, recomputing its loop's vertices from the distance plane and storing 36-byte strides.
 __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint16_t *__restrict__ edt,
                                                           const uint32_t *__restrict__ inside, uint32_t n_groups,
+                                                          unsigned per_cta,
                                                           const unsigned long long *__restrict__ block_base,
                                                           float *__restrict__ tris, long long *__restrict__ labels,
                                                           unsigned long long max_tris) {
@@ -694,7 +696,8 @@ __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint1
   unsigned long long base = block_base[blockIdx.x];
   if (base >= max_tris) return;
   if (threadIdx.x <= kSesBitK * kSesBitK + 1) s_f[threadIdx.x] = fmaf(sqrtf((float)threadIdx.x), G.h, -G.p);
-  const SesGroup s = ses_group(G, inside, blockIdx.x * (unsigned)kSesGroups + threadIdx.x, n_groups);
+  const SesGroup s = ses_group(G, inside, blockIdx.x * per_cta + threadIdx.x,
+                               threadIdx.x < per_cta ? n_groups : 0u);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   unsigned n_cells;
   unsigned rank = block_exclusive_sum((unsigned)__popc(s.active), &n_cells);
@@ -872,6 +875,14 @@ static long long ses_groups(const int32_t dims[3]) {
   return ((long long)dims[0] + 30) / 32 * (dims[1] - 1) * (dims[2] - 1);
 }
 
+// Groups per CTA of the count and emit passes: 256, or fewer (down to 32) while that leaves less than four CTAs per SM,
+// so that a small grid's cells spread over the chip (1,200 atoms at 0.6 A, 16,000 groups: emit 25 us at 256, 10 at 32).
+static unsigned ses_per_cta(const int32_t dims[3]) {
+  unsigned per = kSesThreads;
+  while (per > 32 && ses_groups(dims) / per < 4LL * sm_count()) per >>= 1;
+  return per;
+}
+
 long long ses_words(const int32_t dims[3]) { return ((long long)dims[0] + 31) / 32 * dims[1] * dims[2]; }
 
 template <int K>
@@ -958,19 +969,22 @@ cudaError_t run_ses_count(const SesLaunch &L, cudaStream_t st) {
   }
   const long long n_blocks = ses_blocks(L.dims);
   unsigned *done = reinterpret_cast<unsigned *>(L.bits + ses_words(L.dims));  // cleared with the bits
-  k_ses_count<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.inside, (uint32_t)ses_groups(L.dims), L.block_tris,
-                                                          L.block_base, L.total, done);
+  k_ses_count<<<(unsigned)n_blocks, kSesThreads, 0, st>>>(G, L.inside, (uint32_t)ses_groups(L.dims),
+                                                          ses_per_cta(L.dims), L.block_tris, L.block_base, L.total, done);
   return cudaGetLastError();
 }
 
 cudaError_t run_ses_emit(const SesLaunch &L, cudaStream_t st) {
   if (L.max_tris == 0) return cudaSuccess;
   k_ses_emit<<<(unsigned)ses_blocks(L.dims), kSesThreads, 0, st>>>(
-      make_grid(L), L.edt2, L.inside, (uint32_t)ses_groups(L.dims), L.block_base, L.tris, L.labels,
+      make_grid(L), L.edt2, L.inside, (uint32_t)ses_groups(L.dims), ses_per_cta(L.dims), L.block_base, L.tris, L.labels,
       (unsigned long long)L.max_tris);
   return cudaGetLastError();
 }
 
-long long ses_blocks(const int32_t dims[3]) { return (ses_groups(dims) + kSesGroups - 1) / kSesGroups; }
+long long ses_blocks(const int32_t dims[3]) {
+  const long long per = ses_per_cta(dims);
+  return (ses_groups(dims) + per - 1) / per;
+}
 
 }  // namespace vtx
