@@ -43,7 +43,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-KERNELS_PER_FRAME = 8  # clear, cull, setup, scan, scatter, raster, resolve list, resolve/shade
+KERNELS_PER_FRAME = 8  # clear, cull, setup, ranges, scatter, raster, resolve list, resolve/shade
 
 
 def parse():
@@ -531,7 +531,7 @@ def ses_extra(vtx, torch, dev, reps=5):
     pts = int(g2.dims[0]) * int(g2.dims[1]) * int(g2.dims[2])
     return {"workload": "1e5 atoms, SES (probe 1.4 A) on a 0.5 A grid, marching cubes", "grid_points": pts,
             "triangles": int(n_tri), "ms": ses_ms, "gpoints_per_s": pts / ses_ms / 1e6,
-            "note": "wall time of the synchronous call (SAS, 3 distance passes, count, scan, emit)"}
+            "note": "wall time of the synchronous call (SAS, distances, count, emit)"}
 
 
 # FP32 operations of one composited soft term (the definition's arithmetic, counted from the formula with an
