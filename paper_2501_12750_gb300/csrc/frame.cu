@@ -672,8 +672,8 @@ struct PrimGeom {
 // SHARED: the branches only find the centre's offset from the eye, and lanes with spheres and lanes with cylinders share
 // the precise set-up (the resolve, whose warps mix them).  Set-up, whose lists hold the atoms before the bonds, keeps it
 // inside the branches: shared there, the close 4K view took 439 us instead of 423.
-// (A bond's axis is a sum whose contraction is the compiler's: the two forms may round it differently, by an ulp; a
-// ball-and-stick frame's planes then differ at a few pixels by rounding, 6e-9 of their norm, and no id does.)
+// A bond's axis, length and bounding radius are spelled as explicit operations, so that both forms give the same bits:
+// the resolve then finds the hit that set-up or the raster found (it has no answer for a ray that misses).
 template <bool SHARED>
 __device__ __forceinline__ PrimGeom prim_geom(const Geometry &g, const ViewParams &v, const float4 *X, const uint2 *bonds,
                                               uint32_t id, float zlo, float S, bool use_box_r,
@@ -700,14 +700,16 @@ __device__ __forceinline__ PrimGeom prim_geom(const Geometry &g, const ViewParam
     dx.hi *= 0.5f; dx.lo *= 0.5f;
     dy.hi *= 0.5f; dy.lo *= 0.5f;
     dz.hi *= 0.5f; dz.lo *= 0.5f;
-    float ex = B.x - A.x, ey = B.y - A.y, ez = B.z - A.z;
-    float L = sqrtf(ex * ex + ey * ey + ez * ez);
-    float inv = 1.0f / L;
-    p.A = make_float3((v.R[0] * ex + v.R[1] * ey + v.R[2] * ez) * inv, (v.U[0] * ex + v.U[1] * ey + v.U[2] * ez) * inv,
-                      (v.F[0] * ex + v.F[1] * ey + v.F[2] * ez) * inv);
+    const float ex = B.x - A.x, ey = B.y - A.y, ez = B.z - A.z;
+    const float L = sqrtf(__fmaf_rn(ez, ez, __fmaf_rn(ex, ex, __fmul_rn(ey, ey))));
+    const float inv = __fdiv_rn(1.0f, L);
+    auto along = [&](const float *w) {
+      return __fmul_rn(__fmaf_rn(w[2], ez, __fmaf_rn(w[0], ex, __fmul_rn(w[1], ey))), inv);
+    };
+    p.A = make_float3(along(v.R), along(v.U), along(v.F));
     p.hl = 0.5f * L;
     p.rad = g.bond_radius;
-    p.Rb = sqrtf(p.hl * p.hl + p.rad * p.rad) * 1.00001f;
+    p.Rb = __fmul_rn(sqrtf(__fmaf_rn(p.hl, p.hl, __fmul_rn(p.rad, p.rad))), 1.00001f);
     if (!SHARED) p.su = precise_setup(v, dx, dy, dz, p.Rb, zlo, S);
     if (use_box_r) {
       float cx = 0.5f * (A.x + B.x), cy = 0.5f * (A.y + B.y), cz = 0.5f * (A.z + B.z);
