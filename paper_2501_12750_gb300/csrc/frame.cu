@@ -2155,14 +2155,9 @@ cudaError_t run_binning(const Geometry &g, const Scene &sc, const Scratch &s, cu
     if (g.n_views == 1 && g.n_frames == 1 && sc.counts == nullptr && !g.soft) {
       const int b1 = (int)cull_one_ctas(g.n_atoms);
       const bool plain = g.mode == 0 && !g.clip_on;
-      // A large cull starts only when the clear has ended: placed early, its CTAs (one wave of persistent ones) and
-      // set-up's behind them end up where they slow the stream (1e8 atoms at 4K 479 -> 416 us, 1.1e7-atom
-      // close view 452 -> 405 us; any one of clear, cull and set-up without overlap does it).  Below that the
-      // launch latency saved is worth more (1.07e6 atoms at 8K 458 / 461 us, 2,000 atoms 20.4 / 21.9 us).
-      const bool overlap = g.n_atoms < (4LL << 20);
       const auto cull = sc.stage ? (plain ? k_cull_direct<true, true> : k_cull_direct<false, true>)
                                  : (plain ? k_cull_direct<true, false> : k_cull_direct<false, false>);
-      launch_kernel(overlap, cull, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, sc.stage);
+      launch_pdl(cull, b1, kCullThreads, 0, st, g, sc.frames, s.state, s.surv, sc.stage);
     } else if (!g.soft && g.n_views <= 4 && g.surv_cap >= per_frame + cull_multi_slack(per_frame, g.n_frames)) {
       // a batch (frames x up to 4 views): the barrier-free multi-view cull
       const dim3 gm(cull_multi_ctas(per_frame, g.n_frames), g.n_frames);

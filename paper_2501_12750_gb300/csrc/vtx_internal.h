@@ -122,8 +122,7 @@ long long ses_words(const int32_t dims[3]);  // 32-bit words of the interior bit
 // unchanged; the launch latency and prologue of each kernel overlap the
 // previous kernel's tail.
 template <typename... P, typename... A>
-cudaError_t launch_kernel(bool overlap, void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
-                                 A... args) {
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
@@ -133,12 +132,8 @@ cudaError_t launch_kernel(bool overlap, void (*k)(P...), dim3 grid, int block, s
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
-}
-template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A... args) {
-  return launch_kernel(true, k, grid, block, smem, st, args...);
 }
 
 int sm_count();
