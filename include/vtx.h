@@ -122,7 +122,7 @@ typedef struct {
  * Rendering settings.  vtx_default_settings() fills the values used by the
  * tests: glossy (Blinn-Phong) ka 0.2, kd 0.7, ks 0.3, shininess 32, light
  * (0.25, 0.5, 1) in view space, white background, no SSAO, 16x16 tiles,
- * direct splat up to 16 candidate pixels (tile_w = 0 lets the library
+ * the library's direct-splat threshold (tile_w = 0 lets the library
  * autotune both), 4 toon bands, SAS probe 1.4 A, no clipping, fog or outline.
  * The paper names these techniques but not their constants.  Order of the
  * per-pixel operations: shade, times AO, outline (replaces the colour), fog.
@@ -444,9 +444,12 @@ vtx_status vtx_stage_times(vtx_ctx *ctx, const char **names, float *ms, int32_t 
  * The tile shape and direct-splat threshold chosen by the autotuner for the
  * most recent render call made with settings.tile_w = 0.  The tuner times all
  * nine combinations of tile shape (16x16, 32x8, 8x8) and threshold (4, 16, 64
- * candidate pixels) on the caller's own frame (a batch: its first four
- * frames) once per class (image size, views, log2 of the primitive count,
- * mode) and reuses the fastest.  The output never depends on the choice.
+ * candidate pixels), and with frames that draw no bonds the library default
+ * (splat_max_px = 0, chosen on the device) at each shape, on the caller's own
+ * frame (a batch: its first four frames) once per class (image size, views,
+ * log2 of the primitive count, mode) and reuses the fastest.  splat_max_px is
+ * the fastest of 4, 16 and 64 at the chosen shape, also where the default was
+ * faster still and is used.  The output never depends on the choice.
  * Returns VTX_ERR_STATE before any tuned call.
  */
 vtx_status vtx_tuned_settings(const vtx_ctx *ctx, int32_t *tile_w, int32_t *tile_h, int32_t *splat_max_px);

@@ -69,10 +69,12 @@ struct vtx_ctx {
   size_t ev_used = 0;
   // graphs
   std::vector<GraphEntry> graphs;
-  // autotuning results: key -> (tile_w, tile_h, splat_max)
+  // autotuning results: key -> tile shape, fastest of the explicit thresholds there, and whether set-up's own choice
+  // was faster still (then used in its place)
   struct Tune {
     long long key[6];
-    int tw, th, splat;
+    int tw = 16, th = 16, splat = 16;
+    bool own = false;
   };
   std::vector<Tune> tunes;
   int last_tw = 0, last_th = 0, last_splat = 0;
@@ -409,7 +411,7 @@ vtx_status vtx_default_settings(vtx_settings *s) {
   s->ssao_bias = 0.025f;
   s->tile_w = 16;
   s->tile_h = 16;
-  s->splat_max_px = 0;  // the library default: by primitives per pixel
+  s->splat_max_px = 0;  // the library default: by the survivors' sizes, or primitives per pixel (default_splat)
   s->shading = VTX_SHADE_GLOSSY;
   s->toon_levels = 4;
   s->probe_radius = 1.4f;
@@ -642,8 +644,11 @@ static vtx_status render_once(vtx_ctx *c, const vtx_settings *s, const vtx_outpu
 // ------------------------------------------------------------ autotuner --
 // Tile shape x direct-splat threshold, chosen by timing every candidate on
 // the caller's own frame (or first frames of a batch) once per problem class.
+// Frames without bonds have a fourth threshold: the one that set-up chooses
+// (0), the only one with lanes shared by few survivors.  For every other call
+// the library default is one of the three.
 static const int kTuneShapes[3][2] = {{16, 16}, {32, 8}, {8, 8}};
-static const int kTuneSplat[3] = {4, 16, 64};
+static const int kTuneSplat[4] = {4, 16, 64, 0};
 
 static int ilog2ll(long long v) {
   int r = 0;
@@ -654,28 +659,33 @@ static int ilog2ll(long long v) {
   return r;
 }
 
-// fn(settings) enqueues one run; returns the milliseconds it took (after a sync), or < 0 on error.
+static void use_tune(vtx_ctx *c, const vtx_ctx::Tune &t, vtx_settings *chosen) {
+  chosen->tile_w = c->last_tw = t.tw;
+  chosen->tile_h = c->last_th = t.th;
+  c->last_splat = t.splat;
+  chosen->splat_max_px = t.own ? 0 : t.splat;
+}
+
+// run(settings) enqueues one run.  own: the threshold that set-up chooses is a candidate.
 template <class Fn>
-static vtx_status tune(vtx_ctx *c, const long long key[6], const vtx_settings *s, vtx_settings *chosen, Fn run) {
+static vtx_status tune(vtx_ctx *c, const long long key[6], const vtx_settings *s, bool own, vtx_settings *chosen, Fn run) {
   *chosen = *s;
   for (auto &t : c->tunes)
     if (std::equal(t.key, t.key + 6, key)) {
-      chosen->tile_w = t.tw;
-      chosen->tile_h = t.th;
-      chosen->splat_max_px = t.splat;
-      c->last_tw = t.tw;
-      c->last_th = t.th;
-      c->last_splat = t.splat;
+      use_tune(c, t, chosen);
       return VTX_OK;
     }
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
+  const int n_splat = own ? 4 : 3;
   float best = 3.4e38f;
-  int bi = 0, bj = 1;
+  vtx_ctx::Tune t;
+  std::copy(key, key + 6, t.key);
   vtx_status st = VTX_OK;
-  for (int i = 0; i < 3 && !st; ++i)
-    for (int j = 0; j < 3 && !st; ++j) {
+  for (int i = 0; i < 3 && !st; ++i) {
+    float ms[4];
+    for (int j = 0; j < n_splat && !st; ++j) {
       vtx_settings cand = *s;
       cand.tile_w = kTuneShapes[i][0];
       cand.tile_h = kTuneShapes[i][1];
@@ -696,29 +706,25 @@ static vtx_status tune(vtx_ctx *c, const long long key[6], const vtx_settings *s
       cudaEventRecord(e1, c->stream);
       if (st) break;
       cudaEventSynchronize(e1);
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      if (ms < best) {
-        best = ms;
-        bi = i;
-        bj = j;
-      }
+      ms[j] = 0.0f;
+      cudaEventElapsedTime(&ms[j], e0, e1);
     }
+    if (st) break;
+    const int j = (int)(std::min_element(ms, ms + 3) - ms);
+    const bool by_setup = own && ms[3] < ms[j];
+    if ((by_setup ? ms[3] : ms[j]) < best) {
+      best = by_setup ? ms[3] : ms[j];
+      t.tw = kTuneShapes[i][0];
+      t.th = kTuneShapes[i][1];
+      t.splat = kTuneSplat[j];
+      t.own = by_setup;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st) return st;
-  vtx_ctx::Tune t;
-  std::copy(key, key + 6, t.key);
-  t.tw = kTuneShapes[bi][0];
-  t.th = kTuneShapes[bi][1];
-  t.splat = kTuneSplat[bj];
   c->tunes.push_back(t);
-  chosen->tile_w = t.tw;
-  chosen->tile_h = t.th;
-  chosen->splat_max_px = t.splat;
-  c->last_tw = t.tw;
-  c->last_th = t.th;
-  c->last_splat = t.splat;
+  use_tune(c, t, chosen);
   return VTX_OK;
 }
 
@@ -741,7 +747,8 @@ vtx_status vtx_render_frame(vtx_ctx *c, const vtx_settings *s, const vtx_outputs
   vtx_settings tuned;
   if (s->tile_w == 0) {
     const long long key[6] = {0, c->cam.width, c->cam.height, 1, ilog2ll(c->n_atoms + c->n_bonds + 1), s->mode};
-    st = tune(c, key, s, &tuned, [&](const vtx_settings *cand) { return render_once(c, cand, out, nullptr); });
+    const bool bonds = (s->mode == VTX_MODE_BALL_AND_STICK || s->mode == VTX_MODE_STICKS) && c->n_bonds > 0;
+    st = tune(c, key, s, !bonds, &tuned, [&](const vtx_settings *cand) { return render_once(c, cand, out, nullptr); });
     if (st) return st;
     s = &tuned;
   }
@@ -927,7 +934,7 @@ vtx_status vtx_render_batch(vtx_ctx *c, const float *frames_xyzr, int64_t frame_
   if (s->tile_w == 0) {  // tune on the first (up to) four frames
     const long long key[6] = {1, cams[0].width, cams[0].height, n_views, ilog2ll(frame_stride + 1), s->mode};
     const int nf = n_frames < 4 ? n_frames : 4;
-    st = tune(c, key, s, &tuned, [&](const vtx_settings *cand) {
+    st = tune(c, key, s, false, &tuned, [&](const vtx_settings *cand) {
       return batch_all(c, frames_xyzr, frame_stride, d_counts, nf, cams, n_views, cand, out, nullptr);
     });
     if (st) return st;

@@ -1,0 +1,44 @@
+"""Asking for autotuning must not end slower than not asking: the library default is one of the candidates.  (With the
+explicit thresholds alone the tuned frame took 1.46 to 1.49 times the default's time on these two.)"""
+import numpy as np
+import pytest
+
+from paper_2501_12750_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,w,h", [(2000, 256, 256), (30000, 1280, 720)])
+def test_tuned_frame_is_no_slower_than_the_default(n, w, h):
+    import torch
+
+    import paper_2501_12750_gb300 as vtx
+    rng = np.random.default_rng(n)
+    box = scenes.box_edge(n)
+    elem = scenes.draw_elements(rng, n)
+    x = scenes.pack_xyzr(scenes.protein_like(rng, n, box), elem)
+    c = np.array([box / 2] * 3)
+    r = vtx.Renderer()
+    r.upload_atoms(torch.from_numpy(x).cuda(), torch.from_numpy(elem).cuda())
+    r.set_camera(scenes.look_at(c + np.array([0.0, 0.0, 3.0 * box]), c, w, h))
+    kernel = scenes.ssao_kernel()
+    out = r.alloc_outputs(w, h)
+
+    def us(settings):
+        times = []
+        r.render_frame(settings, out=out)
+        for _ in range(9):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(40):
+                r.render_frame(settings, out=out)
+            e1.record()
+            e1.synchronize()
+            times.append(e0.elapsed_time(e1) * 25.0)
+        return float(np.median(times))
+
+    default = us(vtx.default_settings(ssao_kernel=kernel))
+    planes = {k: v.clone() for k, v in out.items()}
+    tuned = us(vtx.default_settings(ssao_kernel=kernel, tile_w=0))
+    assert all(torch.equal(out[k], planes[k]) for k in planes)
+    assert tuned < 1.2 * default, (tuned, default)
