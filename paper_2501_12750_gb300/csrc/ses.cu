@@ -242,7 +242,8 @@ __global__ __launch_bounds__(256, 6) void k_ses_sas(SesGrid G, const float4 *__r
     // and of the end's sum, each 2^-24 of numbers <= (|c - o| + R) / h
     const float xc = (c.x - G.ox) * inv_h;
     const float eps = 1e-6f + 4e-7f * (fabsf(xc) + fabsf(Rf) * inv_h);
-    if (!(fabsf(xc) < 1e30f)) M = INFINITY;  // no usable index (1 / h overflows): the exact test decides
+    // no usable index (1 / h overflows) or chord (R^2 does): the exact test decides every point
+    if (!(fabsf(xc) < 1e30f && R2f < 1e30f)) M = INFINITY;
     const float Mh = M * inv_h * 1.001f;
     // row r of the box is (lo[1] + r % ny_box, lo[2] + r / ny_box); this lane takes every (32 parts)-th
     const unsigned ny_box = (unsigned)(hi[1] - lo[1] + 1), step = 32u * (unsigned)parts;
@@ -276,7 +277,9 @@ __global__ __launch_bounds__(256, 6) void k_ses_sas(SesGrid G, const float4 *__r
         if (a != i0 || b != i1) sas_row_exact(G.ox, G.oy, G.oz, G.h, G.p, c, j, k, i0, i1, a, b, row);
       } else if (!(t < -M)) {  // else the whole row is outside
         const float w = sqrtf(fmaxf(t + M, 0.0f)) * 1.000001f * inv_h;
-        const int i0 = max(__float2int_ru(xc - w - eps), lo[0]), i1 = min(__float2int_rd(xc + w + eps), hi[0]);
+        const bool all = !(t + M < INFINITY);
+        const int i0 = all ? lo[0] : max(__float2int_ru(xc - w - eps), lo[0]);
+        const int i1 = all ? hi[0] : min(__float2int_rd(xc + w + eps), hi[0]);
         sas_row_exact(G.ox, G.oy, G.oz, G.h, G.p, c, j, k, i0, i1, 1, 0, row);
       }
       j += step_j;
