@@ -188,17 +188,18 @@ static __device__ __noinline__ void sas_row_exact(float ox, float oy, float oz, 
 
 // SAS interior, one bit per grid point (bit i & 31 of word i >> 5 of a row; wx words a row): one warp per atom
 // (`parts` warps when there are few atoms), lanes over the (j, k) rows of its box.  A row meets the sphere in a
-// chord: with t = R^2 - dy^2 - dz^2 in FP32 and M the bound on the FP32 error of d^2 (coordinates, differences
-// and squares, all at most a few ulps of numbers <= xmax + R + 2h, and of R^2 itself), every point with
-// |dx| <= sqrt(t - M) is inside and none with |dx| > sqrt(t + M) is.  Both lie within M / sqrt(t) of sqrt(t) (t > M),
-// so the chord's ends, as grid indices, are known to within u = (M / sqrt(t) + 2 delta) / h plus the rounding eps of
-// the index arithmetic itself; the points within u of an end (a few in a thousand rows have one), and every point of
-// a row with t <= 4 M, are decided by the exact FP64 test, so every decision equals the FP64 one.  Both
-// bounds are kept near the roundings they stand for: an exact test costs its warp some 300 cycles of the FP64 pipe
-// (four times wider bounds took 262 us instead of 102).  The chord's bits are set with one atomic a word.
+// chord: with t = R^2 - dy^2 - dz^2 in FP32 and M the bound on the FP32 error of t (below), every point with
+// dx^2 <= t - M is inside and none with dx^2 > t + M is.  For t > 4 M both ends lie within M / sqrt(t) of sqrt(t).
+// The ends are compared as grid indices, xc -/+ w with xc = (c.x - o.x) / h and w = sqrt(t) / h, so y and z enter
+// through M alone.  In units of 2^-24 = 6e-8 xc carries 3 |xc| (difference, 1 / h, product), w carries 7 w (rsqrt 2
+// ulps, the two products, 1 / h) and the sums xc -/+ w -/+ u 2 (|xc| + w + u); the ends are therefore known to within
+//   u = 1.001 M / (h sqrt(t)) + eps + 1e-6 w,  eps = 1e-6 + 4e-7 (|xc| + R / h).
+// The points within u of an end (a few in a thousand rows have one), and every point of a row with t <= 4 M, are
+// decided by the exact FP64 test, so every decision equals the FP64 one.  The bounds are kept near the roundings they
+// stand for: an exact test costs its warp some 300 cycles of the FP64 pipe (four times wider bounds took 262 us
+// instead of 102).  The chord's bits are set with one atomic a word.
 //
-// Bound by the row loop's issue and its atomics, not by memory: the bits of 3.4e7 points are 4.6 MB and stay in
-// L2.  1e5 atoms at 0.5 A (3.4e7 points): 102 us; 179 us with both ends of both bounds computed per row over a box
+// 1e5 atoms at 0.5 A (3.4e7 points): 102 us; 179 us with both ends of both bounds computed per row over a box
 // two points wider on each side; 1302 us with a byte per point, each point classified on its own.
 __global__ __launch_bounds__(256, 6) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n, int parts,
                                                     uint32_t *__restrict__ bits) {
