@@ -813,8 +813,13 @@ __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams
 // Measured (frame, all splatted against 4 pixels): 2,000 atoms at 256x256 20 / 33 us, 3e4 at 720p 38 / 52, 1e5 at
 // 1080p (mean box 61) 57 / 71, 2e5 at 1080p (42) 68 / 86, 5e5 at 1080p (26) 81 / 139, 1.1e7-atom close view (10)
 // 400 / 582; but 3e5 at 1440p (54, W = 1.6e7) 108 / 111, 1e6 at 4K (54) 296 / 265, 6e4 at 4K (289) 183 / 141.
-// Sharing pays while the survivors alone leave lanes idle: 2,000 atoms 37 -> 20 us at 8 lanes, 3e4 53 -> 38 at 8, 1e5
-// 61 -> 57 at 4 (66 at 8); 2e5 68 -> 73 at 4.
+// Lanes: sharing pays while the survivors alone leave lanes idle and their boxes are large enough that the splat, which
+// is shared, outweighs the set-up, which every lane repeats: twice the lanes where the survivors number at most 4000,
+// 1900 and 450 times the mean box's pixels, and never when they fill the resident threads (152 SMs x 4 CTAs).  Measured
+// over 137 frames (1,500 to 300,000 atoms, 96x67 to 1920x1344): each within 5 % of its best number of lanes; by the
+// number of survivors alone, frames of small boxes lost up to a third (48,000 atoms at 240x168, mean box 6.4: 27.3 us
+// at 8 lanes, 18.3 at 1; 1.6e5 at 340x237, 6.0: 36 at 4, 22.5 at 1).  At 1, 2, 4, 8 lanes: 4,000 atoms at 480x336 (59)
+// 36 / 28 / 23 / 20.5, 25,000 at 480x336 (21) 22.9 / 21.0 / 20.7 / 23.4, 1e5 at 1080p (61) 60 / 59 / 57 / 66.
 struct SplatChoice {
   int splat_max, shift;
 };
@@ -824,7 +829,8 @@ __device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const Vie
   const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
   if (!(mean <= 30.0f || (mean * n <= 1.6e7f && v.f * __uint_as_float(s.rho_bits) <= 6.0f))) return {4, 0};
   const float held = fmaxf(n, 0.5f * (float)s.n_surv);  // a sparse view's slabs are mostly unused slots: each costs a step
-  return {256, held <= 49152.0f ? 3 : (held <= 163840.0f ? 2 : 0)};
+  if (held > 155648.0f) return {256, 0};
+  return {256, held <= 450.0f * mean ? 3 : (held <= 1900.0f * mean ? 2 : (held <= 4000.0f * mean ? 1 : 0))};
 }
 
 // Setup occupancy: 4 CTAs per SM (63 registers, a few bytes spilled) and 8

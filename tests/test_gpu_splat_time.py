@@ -1,0 +1,45 @@
+"""The library-default splat (threshold and lanes per survivor chosen in set-up) against explicit thresholds, on frames
+where a wrong choice is dear: many spheres of a few pixels, which gain nothing from shared lanes."""
+import numpy as np
+import pytest
+
+from paper_2501_12750_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def us(r, out, settings):
+    import torch
+    times = []
+    r.render_frame(settings, out=out)
+    for _ in range(9):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(40):
+            r.render_frame(settings, out=out)
+        e1.record()
+        e1.synchronize()
+        times.append(e0.elapsed_time(e1) * 25.0)
+    return float(np.median(times))
+
+
+# explicit threshold that is best there; time by the survivors' number alone over the time at that threshold
+@pytest.mark.parametrize("n,w,h,splat", [(48000, 240, 168, 16),    # 1.45
+                                         (160000, 340, 237, 16)])  # 1.55
+def test_default_is_near_the_best_threshold(n, w, h, splat):
+    import torch
+
+    import paper_2501_12750_gb300 as vtx
+    rng = np.random.default_rng(n)
+    box = scenes.box_edge(n)
+    elem = scenes.draw_elements(rng, n)
+    x = scenes.pack_xyzr(scenes.protein_like(rng, n, box), elem)
+    c = np.array([box / 2] * 3)
+    r = vtx.Renderer()
+    r.upload_atoms(torch.from_numpy(x).cuda(), torch.from_numpy(elem).cuda())
+    r.set_camera(scenes.look_at(c + np.array([0.0, 0.0, 3.0 * box]), c, w, h))
+    out = r.alloc_outputs(w, h)
+    r.render_frame(vtx.default_settings(flags=vtx.FLAG_SYNC), out=out)
+    explicit = us(r, out, vtx.default_settings(splat_max_px=splat))
+    default = us(r, out, vtx.default_settings())
+    assert default < 1.15 * explicit, (default, explicit)
