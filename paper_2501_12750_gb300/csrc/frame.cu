@@ -804,15 +804,15 @@ __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams
 }
 
 // The library-default splat threshold of an image from its survivors' projected sizes, and how many lanes share a
-// survivor (1 << shift).  With the survivors' mean box (2 f R / z + 1.2)^2 (from the cull's sample) and W their number
-// times it, the splat's pixel tests:
-//   every box splatted (up to 256 pixels) when the mean box is at most 30 pixels, or when W <= 1.6e7 and the largest
-//     radius is at most 6 pixels: the tile raster then has next to nothing to do;
-//   else only boxes of up to 4 pixels, the others rasterised.  Large spheres are cheaper there, and a mixture of both
-//     is dearer than either.
-// Measured (frame, all splatted against 4 pixels): 2,000 atoms at 256x256 20 / 33 us, 3e4 at 720p 38 / 52, 1e5 at
-// 1080p (mean box 61) 57 / 71, 2e5 at 1080p (42) 68 / 86, 5e5 at 1080p (26) 81 / 139, 1.1e7-atom close view (10)
-// 400 / 582; but 3e5 at 1440p (54, W = 1.6e7) 108 / 111, 1e6 at 4K (54) 296 / 265, 6e4 at 4K (289) 183 / 141.
+// survivor (1 << shift).  With n survivors of mean box m = (2 f R / z + 1.2)^2 pixels (from the cull's sample):
+//   every box splatted (up to 256 pixels) when m <= 30, or when m n <= 1.6e7 (the splat's pixel tests), m^2.5 n <= 6.7e9
+//     and the largest radius is at most 6 pixels: the tile raster then has next to nothing to do;
+//   else only boxes of up to 4 pixels, the others rasterised.  Large spheres are cheaper there (the raster stops behind
+//     the nearest ones, the splat tests every pixel of every box), and a mixture of both is dearer than either.
+// Measured (us a frame, all splatted / 4 pixels; protein-like unless said; number, m): 25,000, 96 38 / 46; 48,000, 92
+// 54 / 57; 1e5, 61 58 / 70; 1.5e5, 65 74 / 76; 2e5, 47 69 / 86; 2.5e5, 48 80 / 95.  Past the second limit: 70,000, 102
+// 70 / 63; 1e5, 104 95 / 77; 1.5e5, 82 103 / 84; 2.5e5, 61 116 / 97.  Past the first: 4e5, 47 124 / 116; 1e6, 54 270 / 249;
+// but 5e5, 32 95 / 141.  Uniform cubes, whose spheres hide each other less, cross later: 2.5e5, 63 112 / 130.
 // Lanes: sharing pays while the survivors alone leave lanes idle and their boxes are large enough that the splat, which
 // is shared, outweighs the set-up, which every lane repeats: twice the lanes where the survivors number at most 4000,
 // 1900 and 450 times the mean box's pixels, and never when they fill the resident threads (152 SMs x 4 CTAs).  Measured
@@ -827,7 +827,9 @@ __device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const Vie
   if (!g.splat_auto) return {g.splat_max, 0};
   const float n = 4.0f * (float)s.n_rho;  // survivors (n_surv counts the slabs' unused slots too)
   const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
-  if (!(mean <= 30.0f || (mean * n <= 1.6e7f && v.f * __uint_as_float(s.rho_bits) <= 6.0f))) return {4, 0};
+  const float tests = mean * n;
+  if (!(mean <= 30.0f || (tests <= 1.6e7f && tests * mean * side <= 6.7e9f && v.f * __uint_as_float(s.rho_bits) <= 6.0f)))
+    return {4, 0};
   const float held = fmaxf(n, 0.5f * (float)s.n_surv);  // a sparse view's slabs are mostly unused slots: each costs a step
   if (held > 155648.0f) return {256, 0};
   return {256, held <= 450.0f * mean ? 3 : (held <= 1900.0f * mean ? 2 : (held <= 4000.0f * mean ? 1 : 0))};
