@@ -403,8 +403,9 @@ vtx_status vtx_ses_fit_grid(vtx_ctx *ctx, const float *xyzr, int64_t n_atoms, fl
  * j) (nx-1) + i; sas (nullable) uint8 and edt2 (nullable) uint16, both
  * [nz][ny][nx].  *n_tris (host) receives the total number of triangles;
  * when it exceeds max_tris only the first max_tris are written and the call
- * returns VTX_ERR_CAPACITY.  Scratch (2.25 bytes per grid point; 6.25 when
- * p / h > 5) is owned by the context.  Synchronises.
+ * returns VTX_ERR_CAPACITY.  Scratch (2 bytes per grid point and 8 per 32
+ * points of a row or part of them; 4 more per point when p / h > 5) is owned
+ * by the context.  Synchronises.
  */
 vtx_status vtx_ses_mesh(vtx_ctx *ctx, const float *xyzr, int64_t n_atoms, const vtx_ses_grid *grid, float *tris,
                         int64_t max_tris, int64_t *labels, uint8_t *sas, uint16_t *edt2, int64_t *n_tris);

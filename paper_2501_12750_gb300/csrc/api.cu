@@ -27,6 +27,7 @@ struct GraphEntry {
 };
 
 constexpr int kNumStages = 8;
+// (scan: the tiles' ranges; resolve: the list of covered pixels)
 const char *kStageNames[kNumStages] = {"clear", "cull", "setup", "scan", "scatter", "raster", "resolve", "shade"};
 
 }  // namespace

@@ -769,9 +769,10 @@ __device__ __forceinline__ bool splat_plain(const ViewParams &v, const PrimGeom 
 // splat_box for a sphere that splat_plain accepts: the same keys, bit for bit, with the x and y parts of every
 // step on the paired FP32 pipes (b and o.y are carried negated, which changes no product), 32-bit key arithmetic
 // and the pixel, its key's address and the row change by selects instead of a conversion and a product a pixel.
-// Setup is bound by issue, and on frames of spheres a few pixels wide most of it is this loop: with the single
-// image's view constants as immediate operands, the close 4K view of 1.1e7 atoms went from 544 to 480 us and a
-// batch of 32 images of 500,000 atoms from 942 to 885 us.
+// Setup is bound by issue (close 4K view of 1.1e7 atoms: 81 % of the issue slots, 25 of 32 lanes, ALU and FMA pipes at
+// 46 and 43 %), and on frames of spheres a few pixels wide most of it is this loop: with the single image's view
+// constants as immediate operands, that frame went from 544 to 480 us and a batch of 32 images of 500,000 atoms from
+// 942 to 885 us.
 __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams &v, const PrimGeom &p,
                                              const PixBox &box, float S, uint32_t id, unsigned long long *K, int sub,
                                              int shift) {
@@ -1074,7 +1075,6 @@ __device__ __forceinline__ void occl_upper_splat(const Geometry &g, const ViewPa
   const int w = box.x1 - box.x0 + 1, npix = w * (box.y1 - box.y0 + 1);
   if (npix > kOcclMaxPixels) return;
   const float rr2 = rr * rr, dU = fmaf(2.0f, del, 1e-4f);
-  // (with the test's records all loaded before the first is tested: batch of 32 images of 500,000 atoms 878 -> 862 us)
   // stepped as splat_sphere's loop: the x and y parts on the paired FP32 pipes (b and w.y negated), the pixel and its
   // key's address by selects
   const float x0 = (float)box.x0 + 0.5f, x1 = (float)box.x1 + 0.5f;
@@ -1226,7 +1226,7 @@ __global__ __launch_bounds__(256) void k_occl_test(Geometry g, const float4 *__r
       id[j] = k < n ? sv[k] : kNoId;
     }
 #pragma unroll
-    for (int j = 0; j < kOcclItems; ++j)  // all records in flight before the first is tested
+    for (int j = 0; j < kOcclItems; ++j)  // all records in flight before the first is tested (batch 878 -> 862 us)
       at[j] = (id[j] != kNoId && (long long)id[j] < g.n_atoms) ? X[id[j]] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int j = 0; j < kOcclItems; ++j) {
@@ -1639,9 +1639,10 @@ __device__ __forceinline__ unsigned long long raster_hit(const PrimRec &p, const
   return (hit && p.zr + s >= znear) ? pack_key(rec_key(p), s, S, p.id) : kBgKey;
 }
 
-// Bound by issue and the slowest warps' dependent hit tests.  8 x 4 pixel blocks per warp, the short key, the
-// cylinders' per-axis reach and their early return: ball-and-stick frame (60,000 atoms at 1080p) 278 -> 232 us,
-// 1e5 atoms at 1080p 74.1 -> 69.1 us, SAS illustration of 30,000 atoms 59.8 -> 54.5 us.
+// Bound by the slowest warp of each tile and its dependent hit tests, and on bonds by issue: ball-and-stick frame
+// (60,000 atoms at 1080p) 109 us at 61 % of the issue slots, 18 of 32 lanes, more warps waiting at the tile's barriers
+// than for anything else; SAS illustration of 30,000 atoms 24 us at 25 % of the slots.  8 x 4 pixel blocks per warp, the
+// short key, the cylinders' per-axis reach and their early return: frames 278 -> 232 us and 59.8 -> 54.5 us.
 //
 // One CTA per tile at a time, the non-empty tiles longest first from a queue (as many CTAs as are resident):
 // the tile's list is ordered by depth bucket with every entry's pixel box; then each warp walks it on its own.
@@ -1785,9 +1786,10 @@ __device__ __forceinline__ float key_diff_f(uint32_t a, uint32_t b) {
   return ge ? f : -f;
 }
 
-// Bound by issue: the winner's set-up and 16 neighbour samples a pixel.  With 32-bit indices in place of three 64-bit
-// divisions a pixel and a single image's view constants as immediate operands: close 4K view 480 -> 467 us,
-// ball-and-stick frame 292 -> 278 us, batch of 32 images 885 -> 872 us.
+// Bound by waiting for the 16 neighbour depths a pixel and by issue (the winner's set-up and the samples' positions): 52
+// to 65 % of the issue slots, warps mostly waiting on the gathers; the batch also writes at half of the DRAM rate.
+// 32-bit indices in place of three 64-bit divisions a pixel, and a single image's view constants as immediate operands:
+// close 4K view 480 -> 467 us, ball-and-stick frame 292 -> 278 us, batch of 32 images 885 -> 872 us.
 //
 // ONE: a single image (its view constants are then compile-time indexed kernel parameters).  Key indices within an
 // image fit 32 bits (at most 2^28 pixels), and of a packed key the neighbours are asked for the depth word only: the
@@ -2120,7 +2122,7 @@ static inline void ev_rec(StageEvents *e, int i, cudaStream_t st) {
 #define VTX_CLEAR_MEMSET 1  // clear a batch's key planes with a memset instead of the clear kernel's stores
 #endif
 
-// Shared binning front end: init, cull, finalize, setup (+splat), scan, scatter.
+// Shared binning front end: clear, cull, setup (+splat), ranges, scatter.
 cudaError_t run_binning(const Geometry &g, const Scene &sc, const Scratch &s, cudaStream_t st, StageEvents *evs,
                         bool soft) {
   const int sms = sm_count();

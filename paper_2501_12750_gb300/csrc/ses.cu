@@ -199,8 +199,9 @@ static __device__ __noinline__ void sas_row_exact(float ox, float oy, float oz, 
 // stand for: an exact test costs its warp some 300 cycles of the FP64 pipe (four times wider bounds took 262 us
 // instead of 102).  The chord's bits are set with one atomic a word.
 //
-// 1e5 atoms at 0.5 A (3.4e7 points): 102 us; 179 us with both ends of both bounds computed per row over a box
-// two points wider on each side; 1302 us with a byte per point, each point classified on its own.
+// Bound by issue (83 % of the slots; FP64 pipe 42 %).  1e5 atoms at 0.5 A (3.4e7 points): 105 us; 179 us with both ends
+// of both bounds computed per row over a box two points wider on each side; 1302 us with a byte per point, each point
+// classified on its own.
 __global__ __launch_bounds__(256, 6) void k_ses_sas(SesGrid G, const float4 *__restrict__ X, long long n, int parts,
                                                     uint32_t *__restrict__ bits) {
   const int lane = threadIdx.x & 31;
@@ -402,9 +403,9 @@ __device__ __forceinline__ void ses_values(uint16_t *s_val, std::integer_sequenc
 // level (the ordinal of its distance) is kept as binary digit planes and spread to one 16-bit value per point at
 // the end.  Points beyond the grid are not outside points.
 //
-// Bound by shared-memory reads and issue (K = 4: 153 reads a word).  3.4e7 points at K = 4: 60 us; the three
-// separable passes over 16-bit planes (one point per thread) take 105 + 2 x 172 us.  K <= 6 because the offsets
-// grow with K^3 (519 at K = 6) and every one is an unrolled instruction.
+// Bound by issue (K = 4: 153 reads and ORs a word; 79 % of the issue slots, ALU 70 %, shared memory 58 %).  3.4e7 points at
+// K = 4: 66 us; the three separable passes over 16-bit planes (one point per thread) take 105 + 2 x 172 us.  K <= 6
+// because the offsets grow with K^3 (519 at K = 6) and every one is an unrolled instruction.
 template <int K>
 __global__ __launch_bounds__(256) void k_ses_levels(SesGrid G, const uint32_t *__restrict__ bits,
                                                     uint16_t *__restrict__ edt2, uint32_t *__restrict__ inside) {
@@ -601,11 +602,11 @@ __device__ __forceinline__ unsigned block_exclusive_sum(unsigned v, unsigned *to
   return before;
 }
 
-// Triangles of every `per_cta` <= 256 groups (one group per thread, going through its crossing cells), and, in the last CTA to
-// finish, their exclusive scan: block_base[b] is the first triangle of CTA b's groups.  *done counts finished CTAs
-// (zero at launch); no CTA waits for another.  3.4e7 points: 27 us, of which most is the table lookups of the
-// crossing cells; 307 us with one thread per four cells reading the distance plane, and 100 us for the scan of
-// its eight times as many counts in a launch of its own.
+// Triangles of every `per_cta` <= 256 groups (one group per thread, going through its crossing cells), and, in the last
+// CTA to finish, their exclusive scan: block_base[b] is the first triangle of CTA b's groups.  *done counts finished
+// CTAs (zero at launch); no CTA waits for another.  3.4e7 points: 27 us, ALU at 64 % with half of the lanes idle
+// (groups differ in crossing cells); 307 us with one thread per four cells reading the distance plane, and 100 us
+// for the scan of its eight times as many counts in a launch of its own.
 __global__ __launch_bounds__(kSesThreads) void k_ses_count(SesGrid G, const uint32_t *__restrict__ inside,
                                                            uint32_t n_groups, unsigned per_cta,
                                                            unsigned *__restrict__ block_tris,
@@ -684,10 +685,11 @@ __device__ __forceinline__ float3 edge_point(const SesEmitShared &sh, int cell, 
 // of the longer loops; then one thread per triangle puts its three vertices together and the warp writes its 32
 // triangles as one run of floats.
 //
-// Bound by issue (a crossing cell has about five vertices and two triangles) and the triangles' writes.  5.9e6
-// triangles (212 MB): 123 us, with f read from a table of the window's distances and the vertices kept as one
-// coordinate along their edge; 146 us with a root per corner and positions worked out per triangle; 789 us with one thread per triangle finding its cell by binary search over
-// a case byte per cell, recomputing its loop's vertices from the distance plane and storing 36-byte strides.
+// Bound by shared memory, issue and the barriers between the steps: L1 63 %, 66 % of the issue slots, 22 of 32 lanes; DRAM
+// 17 %.  5.9e6 triangles (212 MB): 123 us, with f read from a table of the window's distances and the vertices kept
+// as one coordinate along their edge; 146 us with a root per corner and positions worked out per triangle; 789 us with
+// one thread per triangle finding its cell by binary search over a case byte per cell, recomputing its loop's vertices
+// from the distance plane and storing 36-byte strides.
 __global__ __launch_bounds__(kSesThreads) void k_ses_emit(SesGrid G, const uint16_t *__restrict__ edt,
                                                           const uint32_t *__restrict__ inside, uint32_t n_groups,
                                                           unsigned per_cta,

@@ -578,10 +578,11 @@ __device__ __forceinline__ void soft_fwd_walk(const Geometry &g, const SoftTile 
 // the whole tile, so a warp that finishes its block early takes the next item instead of waiting for the tile's
 // slowest warp (a quarter of the time with a CTA per tile, of 20,000 atoms from 16 views), and the sort before it keeps
 // neither its registers nor its shared memory.
-// Forward CTAs per SM: 3 (80 registers).
+// Forward CTAs per SM: 3 (80 registers).  Bound by issue and the pairs' dependent steps (65 % of the issue slots, 21 of 32
+// lanes).
 //
-// 20,000 atoms from 16 views at 512x512: 136 us after 45 us of sorting and filling, forward call 223 us; 284 us with a CTA per tile that sorted, walked and (empty
-// ones) filled; 309 us with one entry per step on the scalar pipes.
+// 20,000 atoms from 16 views at 512x512: 148 us after 47 us of sorting and filling, forward call 223 us; 284 us with a
+// CTA per tile that sorted, walked and (empty ones) filled; 309 us with one entry per step on the scalar pipes.
 #ifndef VTX_SOFT_FWD_MINB
 #define VTX_SOFT_FWD_MINB 3
 #endif
@@ -797,9 +798,10 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
 }
 
 // Items and queue as the forward's.
-// Bound by issue and, on small problems, by each warp's chain of pairs.  Two CTAs per SM (120 registers, nothing
-// spilled): 20,000 atoms from 16 views at 512x512 307 us, 1,200 atoms from 2 views at 200x136 138 us; 3 CTAs 310 / 161,
-// 4 CTAs 368 / 181.  One entry per step, its atom id read from the list in global memory, took 362 / 179 us.
+// Bound by each warp's chain of pairs and by issue (59 % of the slots at 24 % of the warps, 19 of 32 lanes; on small
+// problems 21 % of the slots, the chain alone).  Two CTAs per SM (120 registers, nothing spilled): 20,000 atoms from 16
+// views at 512x512 307 us, 1,200 atoms from 2 views at 200x136 138 us; 3 CTAs 310 / 161, 4 CTAs 368 / 181.  One entry
+// per step, its atom id read from the list in global memory, took 362 / 179 us.
 #ifndef VTX_SOFT_BWD_MINB
 #define VTX_SOFT_BWD_MINB 2
 #endif
