@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2501_12750_gb300 import scenes
+from test_gpu_splat_time import fastest
 
 pytestmark = pytest.mark.gpu
 
@@ -24,21 +25,10 @@ def test_tuned_frame_is_no_slower_than_the_default(n, w, h):
     kernel = scenes.ssao_kernel()
     out = r.alloc_outputs(w, h)
 
-    def us(settings):
-        times = []
-        r.render_frame(settings, out=out)
-        for _ in range(9):
-            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            e0.record()
-            for _ in range(40):
-                r.render_frame(settings, out=out)
-            e1.record()
-            e1.synchronize()
-            times.append(e0.elapsed_time(e1) * 25.0)
-        return float(np.median(times))
-
-    default = us(vtx.default_settings(ssao_kernel=kernel))
+    settings = [vtx.default_settings(ssao_kernel=kernel), vtx.default_settings(ssao_kernel=kernel, tile_w=0)]
+    r.render_frame(settings[0], out=out)
     planes = {k: v.clone() for k, v in out.items()}
-    tuned = us(vtx.default_settings(ssao_kernel=kernel, tile_w=0))
+    r.render_frame(settings[1], out=out)
     assert all(torch.equal(out[k], planes[k]) for k in planes)
+    default, tuned = fastest(r, out, settings)
     assert tuned < 1.2 * default, (tuned, default)

@@ -9,19 +9,22 @@ from paper_2501_12750_gb300 import scenes
 pytestmark = pytest.mark.gpu
 
 
-def us(r, out, settings):
+def fastest(r, out, settings):
+    """Microseconds a frame of each of the settings: the least of eleven runs of 40 frames, taken in turn."""
     import torch
-    times = []
-    r.render_frame(settings, out=out)
-    for _ in range(9):
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        for _ in range(40):
-            r.render_frame(settings, out=out)
-        e1.record()
-        e1.synchronize()
-        times.append(e0.elapsed_time(e1) * 25.0)
-    return float(np.median(times))
+    best = [float("inf")] * len(settings)
+    for s in settings:
+        r.render_frame(s, out=out)
+    for _ in range(11):
+        for i, s in enumerate(settings):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(40):
+                r.render_frame(s, out=out)
+            e1.record()
+            e1.synchronize()
+            best[i] = min(best[i], e0.elapsed_time(e1) * 25.0)
+    return best
 
 
 # explicit threshold that is best there; beside it, the default's time over that threshold's with lanes shared by the
@@ -43,6 +46,5 @@ def test_default_is_near_the_best_threshold(n, w, h, splat):
     r.set_camera(scenes.look_at(c + np.array([0.0, 0.0, 3.0 * box]), c, w, h))
     out = r.alloc_outputs(w, h)
     r.render_frame(vtx.default_settings(flags=vtx.FLAG_SYNC), out=out)
-    explicit = us(r, out, vtx.default_settings(splat_max_px=splat))
-    default = us(r, out, vtx.default_settings())
+    explicit, default = fastest(r, out, [vtx.default_settings(splat_max_px=splat), vtx.default_settings()])
     assert default < 1.15 * explicit, (default, explicit)
