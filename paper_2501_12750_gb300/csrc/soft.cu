@@ -382,37 +382,42 @@ __device__ __forceinline__ void soft_fill_tile(const Geometry &g, long long gt, 
   }
 }
 
-// Orders the lists of the n_list non-empty tiles in place, one CTA each, longest first.  With output planes (the forward),
-// every warp of the CTAs behind them fills one tile's planes if it is empty; those past both end at once.
+// Orders the lists of the n_list non-empty tiles in place: n_sort CTAs take every n_sort-th of them, longest first.  With
+// output planes (the forward), every warp of the CTAs behind them fills one tile's planes if it is empty.  n_sort is
+// bounded (a CTA per tile of the image, most of which ended at once, made a backward that rebuilds the lists of four
+// views at 4096x4096 take 898 us instead of 664, and the forward 1125 instead of 865).
 __global__ __launch_bounds__(kSoftNT) void k_soft_sort(Geometry g, unsigned long long *entries,
                                                       unsigned long long cap_entries,
                                                       const uint32_t *__restrict__ tile_count,
                                                       const uint32_t *__restrict__ tile_start,
                                                       const uint32_t *__restrict__ tile_list, long long pitch,
-                                                      Status *status, float *cov, float *dep, float *nrm, uint2 *state,
-                                                      int vec) {
+                                                      Status *status, unsigned n_sort, float *cov, float *dep, float *nrm,
+                                                      uint2 *state, int vec) {
   pdl_enter();
   __shared__ unsigned long long s_e[kSoftCap];
   __shared__ uint16_t s_off[kSoftCap];
-  const uint32_t n_list = status->n_list;
-  if (blockIdx.x >= n_list) {
-    const long long gt = (long long)(blockIdx.x - n_list) * (kSoftNT / 32) + (threadIdx.x >> 5);
-    if (cov && gt < (long long)g.n_img * g.tiles_per_img && tile_count[gt] == 0u)
+  if (blockIdx.x >= n_sort) {
+    const long long gt = (long long)(blockIdx.x - n_sort) * (kSoftNT / 32) + (threadIdx.x >> 5);
+    if (gt < (long long)g.n_img * g.tiles_per_img && tile_count[gt] == 0u)
       soft_fill_tile(g, gt, vec != 0, cov, dep, nrm, state);
     return;
   }
+  const uint32_t n_list = status->n_list;
   const TileOrder order(status, pitch);
-  const long long gt = order.tile(tile_list, pitch, blockIdx.x);
-  uint32_t start;
-  const int m = (int)soft_count(tile_count, tile_start, gt, cap_entries, start);
-  if (threadIdx.x == 0) atomicMax(&status->max_list, (unsigned)m);
-  if (m == 0) return;
-  if (m > kSoftCap) {
-    soft_sort_global(entries + start, m);
-    return;
+  for (uint32_t li = blockIdx.x; li < n_list; li += n_sort) {
+    const long long gt = order.tile(tile_list, pitch, li);
+    uint32_t start;
+    const int m = (int)soft_count(tile_count, tile_start, gt, cap_entries, start);
+    if (threadIdx.x == 0) atomicMax(&status->max_list, (unsigned)m);
+    if (m == 0) continue;
+    if (m > kSoftCap) {
+      soft_sort_global(entries + start, m);
+      continue;
+    }
+    __syncthreads();  // the previous list has left shared memory
+    soft_order(entries + start, m, s_e, s_off);
+    for (int i = threadIdx.x; i < m; i += kSoftNT) entries[start + i] = s_e[i];
   }
-  soft_order(entries + start, m, s_e, s_off);
-  for (int i = threadIdx.x; i < m; i += kSoftNT) entries[start + i] = s_e[i];
 }
 
 // Each warp walks the sorted list on its own (no block barrier after the
@@ -850,10 +855,12 @@ cudaError_t run_soft_pipeline(const Geometry &g, const Scene &sc, const Scratch 
   if (!reuse) {
     const bool vec = fwd && g.W % 4 == 0 &&
                      ((uintptr_t)cov | (uintptr_t)depth | (uintptr_t)normal | (uintptr_t)state) % 16 == 0;
-    // n_list (at most n_tiles, not known here) sorting CTAs and, forward, a filling warp per tile
+    // sorting CTAs: about three times as many as are resident (44 KB of shared memory each); then, forward, a filling
+    // warp per tile
+    const long long most = 16LL * sm_count(), n_sort = n_tiles < most ? n_tiles : most;
     const long long fill = fwd ? (n_tiles + kSoftNT / 32 - 1) / (kSoftNT / 32) : 0;
-    launch_pdl(k_soft_sort, (unsigned)(n_tiles + fill), kSoftNT, 0, st, g, s.entries, s.cap_entries, s.tile_count,
-               s.tile_start, s.tile_list, pitch, s.status, cov, depth, normal, state, vec ? 1 : 0);
+    launch_pdl(k_soft_sort, (unsigned)(n_sort + fill), kSoftNT, 0, st, g, s.entries, s.cap_entries, s.tile_count,
+               s.tile_start, s.tile_list, pitch, s.status, n_sort, cov, depth, normal, state, vec ? 1 : 0);
   }
   // persistent CTAs: as many as are resident at once, never more than eight items of a tile each
   const long long most = (long long)(fwd ? VTX_SOFT_FWD_MINB : VTX_SOFT_BWD_MINB) * sm_count();

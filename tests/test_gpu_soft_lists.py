@@ -67,14 +67,15 @@ def test_empty_tiles_of_any_width(w, h):
         assert np.abs(nrm[v].cpu().numpy().reshape(3, -1).T[ok] - o.N[ok]).max() <= TOL
 
 
-@pytest.mark.parametrize("w", [1457, 1460])
-def test_single_tile_list(w):
-    """16 views of 92 x 92 tiles: the planes, the state and the gradients of 16 calls of one view each."""
+@pytest.mark.parametrize("w,h,views", [(1457, 1459, 16), (1460, 1459, 16), (1024, 1024, 4)])
+def test_many_tiles(w, h, views):
+    """More than 131,072 tiles (a single list), and more lists than the sorting CTAs take at once: the planes, the state
+    and the gradients of as many calls of one view each."""
     import torch
 
     import paper_2501_12750_gb300 as vtx
-    x, cams = scene(2500, w, 1459, 16, 1.7)
-    assert 16 * (-(-w // 16)) * (-(-1459 // 16)) > 131072
+    x, cams = scene(2500, w, h, views, 1.7)
+    assert (views == 4) == (views * (-(-w // 16)) * (-(-h // 16)) <= 131072)
     x = torch.from_numpy(x).cuda()
     r = vtx.Renderer()
     planes = forward_into_nan(r, x, cams)
@@ -85,7 +86,7 @@ def test_single_tile_list(w):
             (("lists", dict(state=planes[3], reuse_lists=True)), ("rebuilt", dict(state=planes[3])), ("walk", {}))}
     sums = torch.zeros(x.shape, dtype=torch.float64, device="cuda")
     one = vtx.Renderer()
-    for v in range(16):
+    for v in range(views):
         part = forward_into_nan(one, x, cams[v:v + 1])
         for a, b in zip(planes, part):
             assert torch.equal(a[v].view(torch.int32), b[0].view(torch.int32))
