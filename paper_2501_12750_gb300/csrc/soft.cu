@@ -804,13 +804,13 @@ __device__ __forceinline__ void soft_bwd_walk(const Geometry &g, const SoftTile 
 
 // Items and queue as the forward's.
 // Bound by each warp's chain of pairs and by issue (59 % of the slots at 24 % of the warps, 19 of 32 lanes; on small
-// problems 21 % of the slots, the chain alone).  Two CTAs per SM (120 registers, nothing spilled): 20,000 atoms from 16
-// views at 512x512 307 us, 1,200 atoms from 2 views at 200x136 138 us; 3 CTAs 310 / 161, 4 CTAs 368 / 181.  One entry
-// per step, its atom id read from the list in global memory, took 362 / 179 us.
-#ifndef VTX_SOFT_BWD_MINB
-#define VTX_SOFT_BWD_MINB 2
-#endif
-__global__ __launch_bounds__(kSoftNT, VTX_SOFT_BWD_MINB) void k_soft_bwd(Geometry g, const PrimRec *__restrict__ recs,
+// problems 21 % of the slots, the chain alone).  CTAS per SM: two (120 registers, nothing spilled) up to 32,768 tiles,
+// where the chain counts, three (80 registers) above, where items are short and many and their waits count.  At 2 / 3 /
+// 4: 1,000 atoms from 16 views at 256x256 85 / 101 / 114 us, 20,000 from 16 views at 512x512 336 / 331 / 395, at 1024x1024
+// 391 / 361 / 395, 20,000 from 4 views at 4096x4096 489 / 424 / 404, 2,000 from 8 at 2048x2048 156 / 143 / 139.  One
+// entry per step, its atom id read from the list in global memory, took 362 us at 512x512 (348 at 4096x4096).
+template <int CTAS>
+__global__ __launch_bounds__(kSoftNT, CTAS) void k_soft_bwd(Geometry g, const PrimRec *__restrict__ recs,
                                                             const uint32_t *__restrict__ rec_of,
                                                             const unsigned long long *__restrict__ entries,
                                                             unsigned long long cap_entries,
@@ -863,14 +863,15 @@ cudaError_t run_soft_pipeline(const Geometry &g, const Scene &sc, const Scratch 
                s.tile_start, s.tile_list, pitch, s.status, n_sort, cov, depth, normal, state, vec ? 1 : 0);
   }
   // persistent CTAs: as many as are resident at once, never more than eight items of a tile each
-  const long long most = (long long)(fwd ? VTX_SOFT_FWD_MINB : VTX_SOFT_BWD_MINB) * sm_count();
+  const int ctas = fwd ? VTX_SOFT_FWD_MINB : (n_tiles > 32768 ? 3 : 2);
+  const long long most = (long long)ctas * sm_count();
   const unsigned grid = (unsigned)(n_tiles < most ? n_tiles : most);
   if (fwd) {
     launch_pdl(k_soft_fwd, grid, kSoftNT, 0, st, g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
                s.tile_start, s.tile_list, pitch, s.status, cov, depth, normal, state);
   } else {
     cudaMemsetAsync(grad, 0, sizeof(float) * 4 * (size_t)g.n_atoms, st);
-    launch_pdl(k_soft_bwd, grid, kSoftNT, 0, st, g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
+    launch_pdl(ctas == 3 ? k_soft_bwd<3> : k_soft_bwd<2>, grid, kSoftNT, 0, st, g, s.recs, s.rec_of, s.entries, s.cap_entries, s.tile_count,
                s.tile_start, s.tile_list, pitch, s.status, g_cov, g_depth, g_normal, state, grad);
   }
   if (evs && evs->ev && evs->n > 5) cudaEventRecord(evs->ev[5], st);
