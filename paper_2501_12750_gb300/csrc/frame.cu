@@ -1405,12 +1405,12 @@ __global__ __launch_bounds__(256) void k_scatter(Geometry g, const PrimRec *__re
 // after the first).
 constexpr int kRasterBuckets = 256;
 
-template <int TW, int TH>
+template <int TW, int TH, bool BONDS>
 __device__ __forceinline__ uint32_t entry_box(const PrimRec *__restrict__ recs, const ViewParams &v, uint32_t ri,
                                               int tx0, int ty0, float uu_max);
 
 // While placing each entry, the final pass also stores its 16-bit pixel box (entry_box) beside it in s_box.
-template <int TW, int TH>
+template <int TW, int TH, bool BONDS>
 __device__ __forceinline__ void bucket_order(const unsigned long long *__restrict__ src, int m,
                                              unsigned long long *s_e, uint16_t *s_off, uint32_t *s_cnt,
                                              uint32_t *s_lo, uint32_t *s_red, const PrimRec *__restrict__ recs,
@@ -1483,7 +1483,7 @@ __device__ __forceinline__ void bucket_order(const unsigned long long *__restric
     const int b = min(NB - 1, (int)((float)(k - lo) * scale));
     const uint32_t pos = s_cnt[b] + s_off[i];
     s_e[pos] = ((unsigned long long)s_lo[b] << 32) | (e & 0xffffffffull);
-    s_box[pos] = (uint16_t)entry_box<TW, TH>(recs, v, (uint32_t)e, tx0, ty0, uu_tile);
+    s_box[pos] = (uint16_t)entry_box<TW, TH, BONDS>(recs, v, (uint32_t)e, tx0, ty0, uu_tile);
   }
   __syncthreads();
 }
@@ -1506,13 +1506,14 @@ __device__ __forceinline__ float raster_reach(float hl, float rad, float k, floa
   return __fdividef(rb * uu_max * rsqrtf(uu_max), k) * 1.001f + 0.01f + 2e-7f * (fabsf(cu) + fabsf(cv));
 }
 
+template <bool BONDS>
 __device__ __forceinline__ bool raster_keep(const PrimRec &p, unsigned x0, unsigned x1, unsigned y0, unsigned y1,
                                             float uu_max) {
   if (p.dz != 0.0f) return true;
   const float cu = p.u0h + p.u0l, cv = p.v0h + p.v0l;
   const float dx = fmaxf(fmaxf((float)x0 + 0.5f - cu, cu - ((float)x1 + 0.5f)), 0.0f);
   const float dy = fmaxf(fmaxf((float)y0 + 0.5f - cv, cv - ((float)y1 + 0.5f)), 0.0f);
-  const float rt = raster_reach(p.hl, p.rad, p.k, cu, cv, uu_max);
+  const float rt = raster_reach(BONDS ? p.hl : 0.0f, p.rad, p.k, cu, cv, uu_max);
   return !(dx * dx + dy * dy > rt * rt);
 }
 
@@ -1524,7 +1525,7 @@ __device__ __forceinline__ bool raster_keep(const PrimRec &p, unsigned x0, unsig
 // cannot reach any of its still-searching pixels.
 // Capped cylinders away from the eye take the reach of cylinder_box along each axis instead of their
 // bounding sphere's (a 1.5 A bond of radius 0.15 A at a random angle then covers 2.4 times fewer pixels).
-template <int TW, int TH>
+template <int TW, int TH, bool BONDS>
 __device__ __forceinline__ uint32_t entry_box(const PrimRec *__restrict__ recs, const ViewParams &v, uint32_t ri,
                                               int tx0, int ty0, float uu_max) {
   constexpr int XB = TW == 32 ? 5 : (TW == 16 ? 4 : 3), YB = TH == 16 ? 4 : 3;
@@ -1532,12 +1533,12 @@ __device__ __forceinline__ uint32_t entry_box(const PrimRec *__restrict__ recs, 
   const PrimRec *pr = recs + ri;
   const float4 uv = __ldg(reinterpret_cast<const float4 *>(pr));      // u0h, u0l, v0h, v0l
   const float4 zk = __ldg(reinterpret_cast<const float4 *>(pr) + 1);  // zr, k, dz, rad
-  const float hl = __ldg(&pr->hl);
+  const float hl = BONDS ? __ldg(&pr->hl) : 0.0f;
   int x0 = 0, x1 = TW - 1, y0 = 0, y1 = TH - 1;
   if (zk.z == 0.0f) {
     const float cu = uv.x + uv.y, cv = uv.z + uv.w;
     float rx, ry;
-    if (hl != 0.0f && zk.x > 8.0f * (hl + zk.w)) {
+    if (BONDS && hl != 0.0f && zk.x > 8.0f * (hl + zk.w)) {
       const float4 ax = __ldg(reinterpret_cast<const float4 *>(pr) + 3);  // ax, ay, az, plain
       const float mx = (cu - v.cx) * v.inv_f, my = (v.cy - cv) * v.inv_f;
       // zk: reference depth, A per pixel there, 0, radius
@@ -1620,6 +1621,7 @@ __device__ __forceinline__ float tile_uu_max(const ViewParams &v, int tx, int ty
 #endif
 
 // The packed key of record p's hit at pixel ray r, or the background key when the ray misses it.
+template <bool BONDS>
 __device__ __forceinline__ unsigned long long raster_hit(const PrimRec &p, const PixRay &r, float znear, float S) {
   const float3 o = local_o(p.u0h, p.u0l, p.v0h, p.v0l, p.k, p.dz, r);
   float s;
@@ -1629,7 +1631,7 @@ __device__ __forceinline__ unsigned long long raster_hit(const PrimRec &p, const
                ? ((unsigned long long)(p.key_lo + (uint32_t)__float2int_rn(s * S)) << 32) | (unsigned long long)p.id
                : kBgKey;
   }
-  if (p.hl == 0.0f) {
+  if (!BONDS || p.hl == 0.0f) {
     hit = sphere_local(o, r, p.rad, s);
   } else {
     int kind;
@@ -1644,9 +1646,13 @@ __device__ __forceinline__ unsigned long long raster_hit(const PrimRec &p, const
 // than for anything else; SAS illustration of 30,000 atoms 24 us at 25 % of the slots.  8 x 4 pixel blocks per warp, the
 // short key, the cylinders' per-axis reach and their early return: frames 278 -> 232 us and 59.8 -> 54.5 us.
 //
+// BONDS: the frame draws bonds. Without them the cylinders' reach and hit test are left out of every step: frames that
+// look out of the middle of a scene, whose lists of tens of thousands of entries are mostly ordering and boxes, went from
+// 6498 to 5756 us (1e5 atoms at 720p) and 19.2 to 16.8 ms (3e5 at 1080p).
+//
 // One CTA per tile at a time, the non-empty tiles longest first from a queue (as many CTAs as are resident):
 // the tile's list is ordered by depth bucket with every entry's pixel box; then each warp walks it on its own.
-template <int TW, int TH>
+template <int TW, int TH, bool BONDS>
 __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__restrict__ recs,
                                                    const unsigned long long *__restrict__ entries,
                                                    unsigned long long cap_entries,
@@ -1700,7 +1706,7 @@ __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__
     if (threadIdx.x == 0) atomicMax(&status->max_list, cnt);
     for (uint32_t seg = 0; seg < cnt; seg += kListCap) {
       const int m = (int)min((uint32_t)kListCap, cnt - seg);
-      bucket_order<TW, TH>(entries + start + seg, m, s_e, reinterpret_cast<uint16_t *>(s_raw), s_cnt, s_lo, s_red,
+      bucket_order<TW, TH, BONDS>(entries + start + seg, m, s_e, reinterpret_cast<uint16_t *>(s_raw), s_cnt, s_lo, s_red,
                            recs, v, s_box, tx * TW, ty * TH, uu_tile);
       // each warp walks the sorted segment on its own, 32 entries at a time, the next window's records
       // arriving by cp.async while the current one is tested; only the entries whose pixel boxes meet the
@@ -1729,7 +1735,7 @@ __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__
         const PrimRec *win = s_w + wb;
         const unsigned x0 = (unsigned)(tx * TW + rx0), x1 = (unsigned)(tx * TW + rx1);
         const unsigned y0 = (unsigned)(ty * TH + ry0), y1 = (unsigned)(ty * TH + ry1);
-        const bool keep = ((cur >> lane) & 1u) && raster_keep(win[lane], x0, x1, y0, y1, uu_max);
+        const bool keep = ((cur >> lane) & 1u) && raster_keep<BONDS>(win[lane], x0, x1, y0, y1, uu_max);
         const unsigned kept = __ballot_sync(0xffffffffu, keep);
         // two entries per step: their hit tests are independent chains the scheduler can interleave.  The
         // second is tested even when the first's bound would have finished the pixel after the first's
@@ -1744,8 +1750,8 @@ __global__ __launch_bounds__(TW *TH) void k_raster(Geometry g, const PrimRec *__
             done = true;
             continue;
           }
-          const unsigned long long k1 = raster_hit(win[q1], r, v.znear, S);
-          const unsigned long long k2 = (VTX_RASTER_PAIR && q2 >= 0) ? raster_hit(win[q2], r, v.znear, S) : kBgKey;
+          const unsigned long long k1 = raster_hit<BONDS>(win[q1], r, v.znear, S);
+          const unsigned long long k2 = (VTX_RASTER_PAIR && q2 >= 0) ? raster_hit<BONDS>(win[q2], r, v.znear, S) : kBgKey;
           if (!VTX_RASTER_PAIR && q2 >= 0) b |= 1u << q2;  // one entry per step: the second waits for the next
           best = k1 < best ? k1 : best;
           best = k2 < best ? k2 : best;
@@ -2239,30 +2245,32 @@ cudaError_t run_frame_pipeline(const Geometry &g, const ShadeParams &sh, const S
   const float4 *Xr = sc.stage ? sc.stage : sc.frames;  // winners are survivors: staged when staging is on
   const long long n_tiles = (long long)g.n_img * g.tiles_per_img;
   // raster CTAs: as many as are resident at once (the tile queue balances them), never more than tiles
-  static int per_sm[3] = {0, 0, 0};
+  static int per_sm[6] = {0, 0, 0, 0, 0, 0};  // by tile shape: without bonds, with them
   static bool rattr = false;
   if (!rattr) {
-    cudaFuncSetAttribute(k_raster<16, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)raster_smem<256>());
-    cudaFuncSetAttribute(k_raster<32, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)raster_smem<256>());
-    cudaFuncSetAttribute(k_raster<8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)raster_smem<64>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_raster<16, 16>, 256, raster_smem<256>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_raster<32, 8>, 256, raster_smem<256>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], k_raster<8, 8>, 64, raster_smem<64>());
+    const auto ready = [](auto k, int threads, size_t smem, int *n) {
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, threads, smem);
+    };
+    ready(k_raster<16, 16, false>, 256, raster_smem<256>(), &per_sm[0]);
+    ready(k_raster<32, 8, false>, 256, raster_smem<256>(), &per_sm[1]);
+    ready(k_raster<8, 8, false>, 64, raster_smem<64>(), &per_sm[2]);
+    ready(k_raster<16, 16, true>, 256, raster_smem<256>(), &per_sm[3]);
+    ready(k_raster<32, 8, true>, 256, raster_smem<256>(), &per_sm[4]);
+    ready(k_raster<8, 8, true>, 64, raster_smem<64>(), &per_sm[5]);
     for (int &q : per_sm) q = q > 0 ? q : 1;
     rattr = true;
   }
   const int shape = (g.tile_w == 16 && g.tile_h == 16) ? 0 : ((g.tile_w == 32 && g.tile_h == 8) ? 1 : 2);
-  const long long resident = (long long)per_sm[shape] * sm_count();
+  const bool bonds = g.n_bonds > 0;
+  const long long resident = (long long)per_sm[shape + (bonds ? 3 : 0)] * sm_count();
   const unsigned rgrid = (unsigned)(n_tiles < resident ? (n_tiles > 0 ? n_tiles : 1) : resident);
-  if (shape == 0)
-    launch_pdl(k_raster<16, 16>, rgrid, 256, raster_smem<256>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
-  else if (shape == 1)
-    launch_pdl(k_raster<32, 8>, rgrid, 256, raster_smem<256>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
-  else
-    launch_pdl(k_raster<8, 8>, rgrid, 64, raster_smem<64>(), st, g, s.recs, s.entries, s.cap_entries,
-               s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles), s.status);
+  const auto raster = shape == 0   ? (bonds ? k_raster<16, 16, true> : k_raster<16, 16, false>)
+                      : shape == 1 ? (bonds ? k_raster<32, 8, true> : k_raster<32, 8, false>)
+                                   : (bonds ? k_raster<8, 8, true> : k_raster<8, 8, false>);
+  launch_pdl(raster, rgrid, shape == 2 ? 64 : 256, shape == 2 ? raster_smem<64>() : raster_smem<256>(), st, g, s.recs,
+             s.entries, s.cap_entries, s.tile_count, s.tile_start, s.state, s.keys, s.tile_list, tile_pitch(n_tiles),
+             s.status);
   ev_rec(evs, 5, st);
   if (sc.dbg_corrupt_key && s.keys) cudaMemsetAsync(s.keys, 0x7f, sizeof(unsigned long long), st);  // test hook
   if (VTX_RESOLVE_2PASS && s.cov_list) {
