@@ -809,7 +809,12 @@ __device__ __forceinline__ void splat_sphere(const Geometry &g, const ViewParams
 //   every box splatted (up to 256 pixels) when m <= 30, or when m n <= 1.6e7 (the splat's pixel tests), m^2.5 n <= 6.7e9
 //     and the largest radius is at most 6 pixels: the tile raster then has next to nothing to do;
 //   else only boxes of up to 4 pixels, the others rasterised.  Large spheres are cheaper there (the raster stops behind
-//     the nearest ones, the splat tests every pixel of every box), and a mixture of both is dearer than either.
+//     the nearest ones, the splat tests every pixel of every box), and a mixture of both is dearer than either;
+//   but 32 pixels where the largest radius is over 6 pixels and 5 times the root mean square (out of the middle of a cell
+//     or a cloud: a few huge spheres before many small ones): at 4 the tiles' lists fill with small boxes, at 256 single
+//     lanes keep the rest waiting.  At 4 / 16 / 32 / 64 / 256 (us): SAS in a cell, 3e6 atoms at 720p 3,800 / 2,760 / 2,770 /
+//     2,810 / -, 3e5 152 / 115 / 101 / 78 / 97; a cloud of 6e5 202 / 182 / 185 / 200 / 278.  Views of one molecule or from
+//     outside a cell have ratios of 1.5 to 4.
 // Measured (us a frame, all splatted / 4 pixels; protein-like unless said; number, m): 25,000, 96 38 / 46; 48,000, 92
 // 54 / 57; 1e5, 61 58 / 70; 1.5e5, 65 74 / 76; 2e5, 47 69 / 86; 2.5e5, 48 80 / 95.  Past the second limit: 70,000, 102
 // 70 / 63; 1e5, 104 95 / 77; 1.5e5, 82 103 / 84; 2.5e5, 61 116 / 97.  Past the first: 4e5, 47 124 / 116; 1e6, 54 270 / 249;
@@ -828,9 +833,9 @@ __device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const Vie
   if (!g.splat_auto) return {g.splat_max, 0};
   const float n = 4.0f * (float)s.n_rho;  // survivors (n_surv counts the slabs' unused slots too)
   const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
-  const float tests = mean * n;
-  if (!(mean <= 30.0f || (tests <= 1.6e7f && tests * mean * side <= 6.7e9f && v.f * __uint_as_float(s.rho_bits) <= 6.0f)))
-    return {4, 0};
+  const float tests = mean * n, largest = __uint_as_float(s.rho_bits);
+  if (v.f * largest > 6.0f && largest * largest * (float)s.n_rho > 25.0f * s.rho2) return {32, 0};
+  if (!(mean <= 30.0f || (tests <= 1.6e7f && tests * mean * side <= 6.7e9f && v.f * largest <= 6.0f))) return {4, 0};
   const float held = fmaxf(n, 0.5f * (float)s.n_surv);  // a sparse view's slabs are mostly unused slots: each costs a step
   if (held > 155648.0f) return {256, 0};
   return {256, held <= 450.0f * mean ? 3 : (held <= 1900.0f * mean ? 2 : (held <= 4000.0f * mean ? 1 : 0))};
