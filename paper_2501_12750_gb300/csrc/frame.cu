@@ -1648,7 +1648,7 @@ __device__ __forceinline__ unsigned long long raster_hit(const PrimRec &p, const
 
 // Bound by the slowest warp of each tile and its dependent hit tests, and on bonds by issue: ball-and-stick frame
 // (60,000 atoms at 1080p) 109 us at 61 % of the issue slots, 18 of 32 lanes, more warps waiting at the tile's barriers
-// than for anything else; SAS illustration of 30,000 atoms 24 us at 25 % of the slots.  8 x 4 pixel blocks per warp, the
+// than for anything else; SAS illustration of 30,000 atoms 24 us at 23 % of the slots.  8 x 4 pixel blocks per warp, the
 // short key, the cylinders' per-axis reach and their early return: frames 278 -> 232 us and 59.8 -> 54.5 us.
 //
 // BONDS: the frame draws bonds. Without them the cylinders' reach and hit test are left out of every step: frames that

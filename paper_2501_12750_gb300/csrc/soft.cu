@@ -586,7 +586,7 @@ __device__ __forceinline__ void soft_fwd_walk(const Geometry &g, const SoftTile 
 // Forward CTAs per SM: 3 (80 registers).  Bound by issue and the pairs' dependent steps (65 % of the issue slots, 21 of 32
 // lanes).
 //
-// 20,000 atoms from 16 views at 512x512: 148 us after 47 us of sorting and filling, forward call 223 us; 284 us with a
+// 20,000 atoms from 16 views at 512x512: 143 us after 38 us of sorting and filling, forward call 229 us; 284 us with a
 // CTA per tile that sorted, walked and (empty ones) filled; 309 us with one entry per step on the scalar pipes.
 #ifndef VTX_SOFT_FWD_MINB
 #define VTX_SOFT_FWD_MINB 3
