@@ -1886,7 +1886,7 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
       float occ = 0.0f;
       const float R = sh.ssao_radius;
       const float2 Txy = make_float2(T.x, T.y), Bxy = make_float2(B.x, B.y), nxy = make_float2(n.x, n.y);
-      const float2 rab = make_float2(r.a, r.b);
+      const float2 mab = make_float2(-r.a, -r.b);
       // samples in groups of kSsaoGroup: the group's neighbour depths are loaded together
       for (int j0 = 0; j0 < sh.ssao_n; j0 += kSsaoGroup) {
         int at[kSsaoGroup];
@@ -1898,18 +1898,17 @@ __device__ __forceinline__ void resolve_pixel(const Geometry &g, const ShadePara
           dls[u] = 0.0f;
           if (j < sh.ssao_n) {
             const float kx = sh.kernel[j][0], ky = sh.kernel[j][1], kz = sh.kernel[j][2];
-            // x and y on the paired pipes: ball-and-stick frame 226 -> 223 us.  Each operation is the one that the
-            // scalar sums R (k . axis) + slope dz, 0.5 + f / den (...) contract to: another choice of the products
-            // that are fused moves a sample by an ulp, and one in 1e7 into the next pixel
-            const float2 sxy = __ffma2_rn(bc2(kz), nxy, __ffma2_rn(bc2(kx), Txy, __fmul2_rn(bc2(ky), Bxy)));
+            // x and y on the paired pipes (the products of a sum fused first to last, as the scalar form compiles):
+            // ball-and-stick frame 226 -> 223 us
+            const float2 dxy = __fmul2_rn(bc2(R), __ffma2_rn(bc2(kz), nxy, __ffma2_rn(bc2(kx), Txy, __fmul2_rn(bc2(ky), Bxy))));
             const float dzv = R * (kx * T.z + ky * B.z + kz * n.z);
             const float dl = -dzv;  // depth offset of the sample
             const float den = t + dl;
             dls[u] = dl;
             if (den > 0.0f) {
               const float fden = __fdiv_rn(v.f, den);  // one division for both offsets
-              const float2 shift = __ffma2_rn(bc2(R), sxy, __fmul2_rn(rab, bc2(dzv)));
-              const float2 cell = __ffma2_rn(make_float2(fden, -fden), shift, bc2(0.5f));
+              const float2 off = __fmul2_rn(make_float2(fden, -fden), __ffma2_rn(mab, bc2(dl), dxy));
+              const float2 cell = __fadd2_rn(bc2(0.5f), off);
               const int ix = px + __float2int_rd(cell.x);
               const int iy = py + __float2int_rd(cell.y);
               if ((unsigned)ix < (unsigned)g.W && (unsigned)iy < (unsigned)g.H) at[u] = iy * g.W + ix;
