@@ -832,13 +832,18 @@ struct SplatChoice {
 __device__ __forceinline__ SplatChoice splat_choice(const Geometry &g, const ViewParams &v, const ImageState &s) {
   if (!g.splat_auto) return {g.splat_max, 0};
   const float n = 4.0f * (float)s.n_rho;  // survivors (n_surv counts the slabs' unused slots too)
-  const float side = 2.0f * v.f * sqrtf(s.rho2 / fmaxf((float)s.n_rho, 1.0f)) + 1.2f, mean = side * side;
-  const float tests = mean * n, largest = __uint_as_float(s.rho_bits);
-  if (v.f * largest > 6.0f && largest * largest * (float)s.n_rho > 25.0f * s.rho2) return {32, 0};
-  if (!(mean <= 30.0f || (tests <= 1.6e7f && tests * mean * side <= 6.7e9f && v.f * largest <= 6.0f))) return {4, 0};
+  const float ms = 4.0f * s.rho2 * rcp_approx(fmaxf(n, 4.0f));  // mean square of R / z
+  const float side = fmaf(2.0f * v.f, sqrt_approx(ms), 1.2f), mean = side * side;
+  const float tests = mean * n, largest = __uint_as_float(s.rho_bits), lr = v.f * largest;
+  if (lr > 6.0f) {
+    if (largest * largest > 25.0f * ms) return {32, 0};
+    if (!(mean <= 30.0f)) return {4, 0};
+  } else if (!(mean <= 30.0f || (tests <= 1.6e7f && tests * mean * side <= 6.7e9f))) {
+    return {4, 0};
+  }
   const float held = fmaxf(n, 0.5f * (float)s.n_surv);  // a sparse view's slabs are mostly unused slots: each costs a step
   if (held > 155648.0f) return {256, 0};
-  return {256, held <= 450.0f * mean ? 3 : (held <= 1900.0f * mean ? 2 : (held <= 4000.0f * mean ? 1 : 0))};
+  return {256, (held <= 4000.0f * mean) + (held <= 1900.0f * mean) + (held <= 450.0f * mean)};
 }
 
 // Setup occupancy: 4 CTAs per SM (63 registers, a few bytes spilled) and 8
